@@ -195,7 +195,7 @@ cupc_status cupc_profile_read(cupc_graph* g, double* ms, uint64_t* launches, siz
  * an invalid entry anywhere drops all k batches (sticky CUPC_EINVAL).
  *
  * cupc_batcher: applies one batch to each of k distinct graphs (k <= the
- * max_graphs given at creation) with five launches in all, whatever k is.
+ * max_graphs given at creation) with four launches in all, whatever k is.
  * The launch sequence reads its arguments from a descriptor table in device
  * memory; with use_cuda_graph it is captured once per launch shape as a
  * CUDA graph and replayed, each call refreshing the table with one
@@ -262,8 +262,9 @@ void cupc_server_destroy(cupc_server* s);
 
 /* Launch tunables of the update's apply kernel (results are identical for
  * every setting; only speed changes): item_records = endpoint records per
- * work item (64..512, 0 = 256), smem_rows = rows per column folded in shared
- * memory (1..min(D, 16), 0 = min(D, 8)); deeper rows go straight to HBM),
+ * chunk at most (64..512, 0 = 256), smem_rows = rows per column folded in
+ * shared memory, besides the first three, which are folded in registers
+ * (1..min(D, 16), 0 = min(D, 8)); deeper rows go straight to HBM),
  * ctas_per_sm = resident CTAs per SM of the persistent grid (0 = as many as
  * fit). CUPC_EINVAL (previous settings kept) when out of range.
  * cupc_get_tuning: out4 = {item_records, smem_rows, ctas_per_sm, CTAs per SM
@@ -277,13 +278,10 @@ cupc_status cupc_get_tuning(const cupc_graph* g, uint32_t* out4);
  * clear the bucket. CUPC_EINVAL when out of range. */
 cupc_status cupc_set_tuning_bucket(cupc_graph* g, uint32_t bucket, uint32_t item_records, uint32_t smem_rows,
                                    uint32_t ctas_per_sm);
-/* Write-back of a vertex whose records form a single work item, for one
- * batch-size bucket (5..15, as above): CUPC_WRITEBACK_AUTO = load-and-store
- * when the chunk averages fewer than 32 endpoint records per vertex, else
- * XOR atomics (the default); CUPC_WRITEBACK_LOAD_STORE and
- * CUPC_WRITEBACK_ATOMIC force one. Vertices split over several items always
- * write back by atomics. Results are identical for every mode.
- * CUPC_EINVAL when bucket or mode is out of range. */
+/* Write-back of a batch-size bucket (5..15, as above). Kept for callers that
+ * set it: every mode is accepted and none changes anything, since the apply
+ * kernel has one write-back (bulk XOR reductions). CUPC_EINVAL when bucket or
+ * mode is out of range. */
 enum { CUPC_WRITEBACK_AUTO = 0, CUPC_WRITEBACK_LOAD_STORE = 1, CUPC_WRITEBACK_ATOMIC = 2 };
 cupc_status cupc_set_writeback_bucket(cupc_graph* g, uint32_t bucket, uint32_t mode);
 

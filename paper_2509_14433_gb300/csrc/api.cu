@@ -45,15 +45,18 @@ Dims derive(uint32_t V, const cupc_params* p) {
   uint32_t P = 1;  // apply threads per layer: the columns and the checksum lane
   while (P < d.C + 1) P <<= 1;
   if (d.L * P > 1024) return d;  // one apply CTA holds every (layer, lane)
-  // the edge index u*V+v must fit the 64-bit bucket word; record offsets are u32
+  // the edge index u*V+v must fit the 64-bit bucket word; record offsets are
+  // u32, the padding of the record array included: a longer batch is applied
+  // in chunks
   if ((uint64_t)d.max_batch * 2 >= 0xFFFFFFFFull) return d;
+  d.max_batch = std::min(d.max_batch, kMaxChunkEdges);
   d.ok = true;
   return d;
 }
 
 // Byte offsets of every device array inside the workspace.
 struct Layout {
-  size_t sketch, keys, gc, cnt, cursor, rec, recw, items, part, stage_edges, stage_ops, stage_edges1, stage_ops1,
+  size_t sketch, keys, gc, cnt, cursor, rec, work, stage_edges, stage_ops, stage_edges1, stage_ops1,
       label, parent, minv, rcnt, roff,
       perm, permb, pcount, final_, merged, best, best2, cand, forest, forest_sorted, acc, log_ids, log_live,
       log_ncand, hlist, ipar, fdead, fadd, fadd_dead, ftab, ftab_pos, total;
@@ -74,16 +77,13 @@ Layout layout(const Dims& d) {
     return at;
   };
   const size_t V = d.V, B = d.max_batch;
-  const size_t nitems = 4 * B / kMinItemRecords + (V < 2 * B ? V : 2 * B) + 2 * kPlanGridCap + 1;
   l.sketch = take((size_t)d.L * V * d.W * sizeof(ulonglong2));
   l.keys = take(key_words(d.L, d.C) * sizeof(uint64_t));
   l.gc = take(GC_SLOTS * sizeof(uint32_t));
   l.cnt = take(V * 4);
   l.cursor = take(V * 4);
-  l.rec = take(2 * B * 8);
-  l.recw = take(2 * B * 4);
-  l.items = take(nitems * sizeof(uint4));
-  l.part = take(kPlanSlices * sizeof(uint4));
+  l.rec = take(rec_entries(V, B) * 8);
+  l.work = take(kWorkSlots * 4);
   l.stage_edges = take(2 * B * 4);
   l.stage_ops = take(B);
   l.stage_edges1 = take(2 * B * 4);
@@ -217,9 +217,8 @@ cupc_status cupc_init(uint32_t V, uint64_t seed, const cupc_params* params, void
   g->cnt = (uint32_t*)(b + l.cnt);
   g->cursor = (uint32_t*)(b + l.cursor);
   g->rec = (uint64_t*)(b + l.rec);
-  g->recw = (uint32_t*)(b + l.recw);
-  g->items = (uint4*)(b + l.items);
-  g->part = (uint4*)(b + l.part);
+  g->rec_cap = (uint32_t)rec_entries(d.V, d.max_batch);
+  g->work = (uint32_t*)(b + l.work);
   g->stage_edges = (uint32_t*)(b + l.stage_edges);
   g->stage_ops = (int8_t*)(b + l.stage_ops);
   g->stage_edges1 = (uint32_t*)(b + l.stage_edges1);
@@ -578,7 +577,7 @@ cupc_status cupc_set_tuning_bucket(cupc_graph* g, uint32_t bucket, uint32_t item
   if (item_records < kMinItemRecords || item_records > kItemRecords || smem_rows > kSmemRowsMax || smem_rows > g->D)
     return CUPC_EINVAL;
   int smem = 0, grid = 0;
-  if (apply_config(g, item_records, smem_rows, ctas_per_sm, &smem, &grid) != cudaSuccess) {
+  if (apply_config(g, smem_rows, ctas_per_sm, &smem, &grid) != cudaSuccess) {
     cudaGetLastError();
     return CUPC_EINVAL;
   }
@@ -586,9 +585,9 @@ cupc_status cupc_set_tuning_bucket(cupc_graph* g, uint32_t bucket, uint32_t item
   return CUPC_OK;
 }
 
+// Kept for callers that set it: the apply kernel has one write-back.
 cupc_status cupc_set_writeback_bucket(cupc_graph* g, uint32_t bucket, uint32_t mode) {
   if (!g || bucket < 5 || bucket > 15 || mode > CUPC_WRITEBACK_ATOMIC) return CUPC_EINVAL;
-  g->wb_b[bucket] = mode;
   return CUPC_OK;
 }
 

@@ -2,16 +2,17 @@
 //
 // A cupc_batcher applies one batch to each of k graphs (App. A.1.1: every
 // update touches every sketch of both endpoints; graphs are independent)
-// with five launches in all, whatever k is: validate, count, plan, scatter
-// and apply each cover every graph. Their arguments live in a descriptor
-// table in device memory (one InstDesc per graph, prefix offsets of edges
-// and work items), so the launch sequence is fixed for a batcher and is
-// captured once as a CUDA graph and replayed; each call only refreshes the
-// table with one host-to-device copy (double-buffered pinned staging).
-// The apply kernel is persistent: CTAs pull work items from one counter
-// across all graphs and fold them with the same per-item code as the
-// single-graph kernel (apply_item). Results are identical to k separate
-// cupc_update_batch calls.
+// with four launches in all, whatever k is: count (which also validates),
+// plan, scatter and apply each cover every graph. Their arguments live in a
+// descriptor table in device memory (one InstDesc per graph, prefix offsets
+// of edges, plan slices and work units), so the launch sequence is fixed for
+// a batcher and is captured once as a CUDA graph and replayed; each call only
+// refreshes the table with one host-to-device copy (double-buffered pinned
+// staging). A work unit is one chunk of a graph's records for one of its
+// layer groups; the units of all graphs are laid end to end and dealt to
+// persistent warps in turn, which apply them with the single-graph kernel's
+// code (apply_chunk). Results are identical to k separate cupc_update_batch
+// calls.
 #include <string.h>
 
 #include <new>
@@ -29,24 +30,24 @@ struct alignas(16) InstDesc {
   uint32_t* cnt;
   uint32_t* cursor;
   uint64_t* rec;
-  uint32_t* recw;
-  uint4* items;
+  uint32_t* work;
   uint32_t* gc;
-  uint64_t edge_base;  // first edge of this graph in the launch's edge space
-  uint32_t n, V, L, C, D, W, P, R, item_records;
-  uint32_t item_base;  // first work item of this graph (set by k_plan_m)
-  uint32_t nitems;     // set by k_plan_m
-  uint32_t nd;         // direct-path records (set by k_plan_m)
-  uint32_t ell;        // bits of one column-hash stage
-  uint32_t long_depth; // depths may need the slow path
-  uint32_t pad[1];
+  uint64_t edge_base;   // first edge of this graph in the launch's edge space
+  uint32_t slice_base;  // first plan slice
+  uint32_t unit_base;   // first work unit: chunk c of layer group l is unit_base + l * nchunks + c (k_scatter_m)
+  uint32_t n, V, L, C, D, W, P, R;
+  uint32_t ell;         // bits of one column-hash stage
+  uint32_t chunk;       // records per chunk
+  uint32_t nchunks;     // chunks of the fold and the direct records, 0 if dropped (k_scatter_m)
+  uint32_t cap;         // entries of rec
+  uint32_t small;       // edge ids of at most 32 bits
 };
 
 struct alignas(16) BatchHead {
-  uint32_t k;            // graphs in this launch
-  uint32_t total_items;  // set by k_plan_m
-  uint32_t next_item;    // apply scheduler
-  uint32_t plans_done;   // k_plan_m completion count
+  uint32_t k;             // graphs in this launch
+  uint32_t total_units;   // set by k_scatter_m
+  uint32_t total_slices;
+  uint32_t next_unit;     // 0 in every copy of the table
   uint64_t total_edges;
   uint64_t pad[5];
 };
@@ -71,11 +72,13 @@ __device__ __forceinline__ uint32_t inst_of_edge(const InstDesc* d, uint32_t k, 
   return lo;
 }
 
-__device__ __forceinline__ uint32_t inst_of_item(const InstDesc* d, uint32_t k, uint32_t it) {
+// Graph holding plan slice (kUnits: work unit) x.
+template <bool kUnits>
+__device__ __forceinline__ uint32_t inst_of(const InstDesc* d, uint32_t k, uint32_t x) {
   uint32_t lo = 0, hi = k;
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) >> 1;
-    if (ld_cg(&d[mid].item_base) <= it)
+    if ((kUnits ? d[mid].unit_base : d[mid].slice_base) <= x)
       lo = mid;
     else
       hi = mid;
@@ -83,128 +86,143 @@ __device__ __forceinline__ uint32_t inst_of_item(const InstDesc* d, uint32_t k, 
   return lo;
 }
 
-__global__ void k_validate_m(const BatchHead* __restrict__ h) {
-  const InstDesc* d = descs_of(h);
-  const uint32_t k = h->k;
-  const uint64_t total = h->total_edges;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (uint64_t)gridDim.x * blockDim.x) {
-    const InstDesc& g = d[inst_of_edge(d, k, i)];
-    const uint64_t j = i - g.edge_base;
-    const uint32_t u = g.edges[2 * j], v = g.edges[2 * j + 1];
-    const int8_t op = g.ops[j];
-    if ((u >= g.V) | (v >= g.V) | (u == v) | ((op != 1) & (op != -1))) atomicOr(&g.gc[GC_ERR], kErrInval);
-  }
-}
-
+// Counts of every graph's batch, and its validation (Problem 1's stream); an
+// invalid batch's counts are cleared by k_plan_m.
 __global__ void k_count_m(const BatchHead* __restrict__ h) {
   const InstDesc* d = descs_of(h);
   const uint32_t k = h->k;
   const uint64_t total = h->total_edges;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (uint64_t)gridDim.x * blockDim.x) {
+  const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < k) d[t].work[kWorkFold] = d[t].work[kWorkDirect] = 0;
+  for (uint64_t i = t; i < total; i += (uint64_t)gridDim.x * blockDim.x) {
     const InstDesc& g = d[inst_of_edge(d, k, i)];
-    if (ld_cg(&g.gc[GC_ERR]) & kErrInval) continue;
     const uint64_t j = i - g.edge_base;
-    atomicAdd(&g.cnt[g.edges[2 * j]], 1u);
-    atomicAdd(&g.cnt[g.edges[2 * j + 1]], 1u);
-  }
-}
-
-// One CTA per graph: cursors and work items (plan_vertices); the last CTA
-// to finish lays the graphs' work items end to end.
-__global__ void __launch_bounds__(1024) k_plan_m(BatchHead* __restrict__ h) {
-  __shared__ bool s_last;
-  InstDesc* d = const_cast<InstDesc*>(descs_of(h));
-  const uint32_t k = h->k, b = blockIdx.x;
-  if (b >= k) return;
-  InstDesc& g = d[b];
-  uint32_t nitems = 0, nd = 0;
-  const bool dropped = (ld_cg(&g.gc[GC_ERR]) & kErrInval) != 0;
-  if (!dropped && g.n > 0) nitems = plan_vertices(g.cnt, g.cursor, g.items, g.V, g.item_records, &nd);
-  if (threadIdx.x == 0) {
-    g.nitems = nitems;
-    g.nd = nd;
-    if (!dropped && g.n > 0) g.gc[GC_BATCHES] += 1;
-    __threadfence();
-    s_last = atomicAdd(&h->plans_done, 1u) == k - 1;
-  }
-  __syncthreads();
-  if (s_last && threadIdx.x == 0) {
-    __threadfence();
-    uint32_t run = 0;
-    for (uint32_t j = 0; j < k; j++) {
-      d[j].item_base = run;
-      run += ld_cg(&d[j].nitems);
+    const uint32_t u = g.edges[2 * j], v = g.edges[2 * j + 1];
+    const int8_t op = g.ops[j];
+    if ((u >= g.V) | (v >= g.V) | (u == v) | ((op != 1) & (op != -1))) {
+      atomicOr(&g.gc[GC_ERR], kErrInval);
+    } else if (!(ld_cg(&g.gc[GC_ERR]) & kErrInval)) {
+      atomicAdd(&g.cnt[u], 1u);
+      atomicAdd(&g.cnt[v], 1u);
     }
-    h->total_items = run;
-    h->next_item = 0;
   }
 }
 
-__global__ void k_scatter_m(const BatchHead* __restrict__ h) {
+__global__ void __launch_bounds__(kPlanThreads) k_plan_m(const BatchHead* __restrict__ h) {
+  const InstDesc* d = descs_of(h);
+  const uint32_t k = h->k;
+  for (uint32_t x = blockIdx.x; x < h->total_slices; x += gridDim.x) {
+    const InstDesc& g = d[inst_of<false>(d, k, x)];
+    const bool dropped = (ld_cg(&g.gc[GC_ERR]) & kErrInval) != 0;
+    plan_slice(g.cnt, g.cursor, g.rec, g.V, g.cap, x - g.slice_base, g.work, dropped);
+    if (!dropped && g.n > 0 && x == g.slice_base && threadIdx.x == 0) g.gc[GC_BATCHES] += 1;
+  }
+}
+
+// Lay the graphs' work units end to end, by one CTA.
+__device__ __forceinline__ void number_units(BatchHead* h) {
+  InstDesc* d = const_cast<InstDesc*>(descs_of(h));
+  const uint32_t k = h->k;
+  uint64_t run = 0;
+  for (uint32_t j0 = 0; j0 < k; j0 += blockDim.x) {
+    const uint32_t j = j0 + threadIdx.x;
+    uint32_t nchunks = 0, units = 0;
+    if (j < k && d[j].n && !(ld_cg(&d[j].gc[GC_ERR]) & kErrInval)) {
+      nchunks = chunk_plan(d[j].work, d[j].chunk).total;
+      units = nchunks * layer_groups(d[j].L, d[j].P);
+    }
+    uint64_t total;
+    const uint64_t before = block_scan(units, &total);
+    if (j < k) {
+      d[j].unit_base = (uint32_t)(run + before);
+      d[j].nchunks = nchunks;
+    }
+    run += total;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) h->total_units = (uint32_t)run;
+}
+
+__global__ void k_scatter_m(BatchHead* __restrict__ h) {
   const InstDesc* d = descs_of(h);
   const uint32_t k = h->k;
   const uint64_t total = h->total_edges;
+  if (blockIdx.x == gridDim.x - 1) number_units(h);  // read by k_apply_m only
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (uint64_t)gridDim.x * blockDim.x) {
     const InstDesc& g = d[inst_of_edge(d, k, i)];
     if (ld_cg(&g.gc[GC_ERR]) & kErrInval) continue;
     const uint64_t j = i - g.edge_base;
     const uint32_t u = g.edges[2 * j], v = g.edges[2 * j + 1];
-    const uint64_t idx = (uint64_t)min(u, v) * g.V + max(u, v);
     const uint32_t pu = atomicAdd(&g.cursor[u], 1u), pv = atomicAdd(&g.cursor[v], 1u);
-    g.rec[pu] = idx;
-    g.rec[pv] = idx;
-    const uint32_t nd = ld_cg(&g.nd);
-    if (pu < nd) g.recw[pu] = u;
-    if (pv < nd) g.recw[pv] = v;
+    g.rec[pu] = make_record(u, v);
+    g.rec[pv] = make_record(v, u);
   }
 }
 
-// Persistent CTAs pull work items of all graphs from one counter. The lane
-// layout follows the graph of the current item (recomputed when it changes);
-// rows stay zero between items, so CTAs move freely between graphs.
-__global__ void k_apply_m(BatchHead* __restrict__ h, uint32_t rmax, uint32_t lmax) {
+struct Unit {
+  uint32_t j, group;
+  Chunk c;
+};
+__device__ __forceinline__ Unit unit_at(const InstDesc* d, uint32_t k, uint32_t total, uint32_t x) {
+  Unit u{0, 0, {nullptr, 0, false}};
+  if (x >= total) return u;
+  u.j = inst_of<true>(d, k, x);
+  const InstDesc& g = d[u.j];
+  const uint32_t at = x - g.unit_base;
+  u.group = at / g.nchunks;
+  u.c = chunk_at(chunk_plan(g.work, g.chunk), at % g.nchunks, g.chunk, g.rec, g.cap);
+  return u;
+}
+
+// The units go to the warps in order, so that the warps at work at one time
+// are on neighbouring vertices: what bounds the kernel is memory, and equal
+// runs of consecutive units per warp (fewer layout changes) were slower, 501
+// against 465 us for 64 graphs of 1024..8192 vertices and 1000 edges each,
+// 1210 against 1060 us with 4000 edges, as their accesses are spread over all
+// of the graphs' memory. A warp asks for its units two ahead, so that the next
+// unit's records load during the current one, and rebuilds the lane layout
+// when the graph or the layer group changes.
+__global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply_m(BatchHead* __restrict__ h,
+                                                                         uint32_t warp_bytes) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const ApplySmem m = apply_smem(smem_raw, rmax, lmax);
-  __shared__ uint32_t s_item;
+  unsigned char* mine = smem_raw + (threadIdx.x >> 5) * warp_bytes;
   const InstDesc* d = descs_of(h);
-  const uint32_t k = h->k;
-  // CTA b starts with item b (CTAs beyond the items leave at once); the
-  // counter hands out the rest, counting from the grid size
-  const uint32_t total = ld_cg(&h->total_items);
-  if (blockIdx.x >= total) return;
-  ulonglong2* my_rows = m.rows + threadIdx.x;
-  const uint32_t rs = blockDim.x;
-  for (uint32_t r = 0; r < rmax; r++) my_rows[r * rs] = make_ulonglong2(0, 0);
-  uint32_t cur = kNoneU32;
+  const uint32_t k = h->k, total = h->total_units, warps = gridDim.x * kApplyWarps;
+  uint32_t x = blockIdx.x * kApplyWarps + (threadIdx.x >> 5), cur_j = kNoneU32, cur_group = 0;
   ApplyLane l{};
-  for (uint32_t it = blockIdx.x; it < total;) {
-    const uint32_t j = inst_of_item(d, k, it);
-    const InstDesc& g = d[j];
-    if (j != cur) {
-      cur = j;
-      l = apply_lane(g.keys, g.L, g.C, g.D, g.P, g.R, g.ell);
-      __syncthreads();  // every thread is done with the previous graph's keys
-      load_kchk(m, g.keys, g.L, g.C);
-      __syncthreads();
+  ApplySmem m{};
+  LaneSums a;
+  clear_sums(a);
+  a.dirty = 0;
+  bool pending = false;
+  Unit u = unit_at(d, k, total, x);
+  uint64_t r = load_record(u.c, 0, u.c);
+  x += warps;
+  while (u.c.n) {
+    const Unit next = unit_at(d, k, total, x);
+    uint32_t ahead = x;
+    if ((threadIdx.x & 31) == 0 && next.c.n) ahead = 2 * warps + atomicAdd(&h->next_unit, 1u);
+    const InstDesc& g = d[u.j];
+    if (u.j != cur_j || u.group != cur_group) {
+      reuse_slots(m, a, pending);
+      __syncwarp();
+      if (u.j != cur_j) {  // another slot layout: its slots start at zero
+        m = apply_smem(mine, apply_slots(g.R), g.P);
+        zero_slots(m, apply_slots(g.R));
+      }
+      l = apply_lane(g.keys, g.sketch, g.V, g.L, g.C, g.D, g.W, g.P, g.ell, u.group);
+      cur_j = u.j;
+      cur_group = u.group;
+      __syncwarp();
     }
-    const uint4 item = g.items[it - ld_cg(&g.item_base)];
-    if (item.x == kDirectItem) {
-      if (g.long_depth)
-        apply_direct<true>(l, g.sketch, g.V, g.W, g.rec + item.y, g.recw + item.y, item.z - item.y, g.L, m);
-      else
-        apply_direct<false>(l, g.sketch, g.V, g.W, g.rec + item.y, g.recw + item.y, item.z - item.y, g.L, m);
-    } else {
-      ulonglong2* gb = g.sketch + ((size_t)l.layer * g.V + item.x) * g.W + l.jbase;
-      if (g.long_depth)
-        apply_item<true>(l, gb, g.rec + item.y, item.z - item.y, item.w != 0, g.L, g.R, m, my_rows, rs);
-      else
-        apply_item<false>(l, gb, g.rec + item.y, item.z - item.y, item.w != 0, g.L, g.R, m, my_rows, rs);
-    }
-    // both item paths end with __syncthreads: every thread has read s_item
-    if (threadIdx.x == 0) s_item = gridDim.x + atomicAdd(&h->next_item, 1u);
-    __syncthreads();
-    it = s_item;
+    if (g.small)
+      apply_chunk<true>(l, m, a, pending, u.c, next.c, r, g.V, g.W, g.C, g.P, g.R);
+    else
+      apply_chunk<false>(l, m, a, pending, u.c, next.c, r, g.V, g.W, g.C, g.P, g.R);
+    u = next;
+    x = __shfl_sync(0xffffffffu, ahead, 0);
   }
+  bulk_wait_all();
 }
 
 }  // namespace cupc
@@ -222,7 +240,7 @@ struct cupc_batcher {
   int cur;
   cudaStream_t cap_stream;
   struct Exec {
-    uint32_t threads, rmax, lmax;
+    uint32_t warp_bytes;
     int apply_grid, apply_smem;
     cudaGraphExec_t exec[2];
   };
@@ -244,25 +262,22 @@ cudaError_t enqueue(cupc_batcher* b, int slot, const cupc_batcher::Exec& x, cuda
   cudaError_t e = cudaMemcpyAsync(b->dtab, b->htab[slot], b->table_bytes, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   const int grid = b->sms * 8;
-  k_validate_m<<<grid, 256, 0, s>>>(b->dtab);
   k_count_m<<<grid, 256, 0, s>>>(b->dtab);
-  k_plan_m<<<b->max_graphs, 1024, 0, s>>>(b->dtab);
+  k_plan_m<<<grid, kPlanThreads, 0, s>>>(b->dtab);
   k_scatter_m<<<grid, 256, 0, s>>>(b->dtab);
-  k_apply_m<<<x.apply_grid, x.threads, x.apply_smem, s>>>(b->dtab, x.rmax, x.lmax);
+  k_apply_m<<<x.apply_grid, 32 * kApplyWarps, x.apply_smem, s>>>(b->dtab, x.warp_bytes);
   return cudaGetLastError();
 }
 
-cudaError_t get_exec(cupc_batcher* b, uint32_t threads, uint32_t rmax, uint32_t lmax, cupc_batcher::Exec** out) {
+cudaError_t get_exec(cupc_batcher* b, uint32_t warp_bytes, cupc_batcher::Exec** out) {
   for (auto& x : b->execs)
-    if (x.threads == threads && x.rmax == rmax && x.lmax == lmax) {
+    if (x.warp_bytes == warp_bytes) {
       *out = &x;
       return cudaSuccess;
     }
   cupc_batcher::Exec x{};
-  x.threads = threads;
-  x.rmax = rmax;
-  x.lmax = lmax;
-  x.apply_smem = (int)apply_smem_bytes(rmax, threads, lmax);
+  x.warp_bytes = warp_bytes;
+  x.apply_smem = (int)(kApplyWarps * warp_bytes);
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, k_apply_m);
   if (e != cudaSuccess) return e;
@@ -271,7 +286,7 @@ cudaError_t get_exec(cupc_batcher* b, uint32_t threads, uint32_t rmax, uint32_t 
     if (e != cudaSuccess) return e;
   }
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_apply_m, (int)threads, x.apply_smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_apply_m, 32 * kApplyWarps, x.apply_smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   x.apply_grid = per_sm * b->sms;
@@ -340,8 +355,21 @@ cupc_status cupc_batcher_update(cupc_batcher* b, cupc_graph* const* graphs, cons
   BatchHead* h = b->htab[slot];
   memset(h, 0, sizeof(BatchHead) + (size_t)k * sizeof(InstDesc));
   InstDesc* d = reinterpret_cast<InstDesc*>(h + 1);
-  uint64_t base = 0;
-  uint32_t threads = 32, rmax = 1, lmax = 1;
+  uint64_t base = 0, units = 0, work = 0, records = 0, vertices = 0;
+  uint32_t slices = 0, warp_bytes = 0;
+  for (uint32_t i = 0; i < k; i++) {
+    work += 2 * (uint64_t)n[i] * layer_groups(graphs[i]->L, graphs[i]->P);
+    records += 2 * (uint64_t)n[i];
+    vertices += graphs[i]->V;
+  }
+  // records per chunk: about three units for each warp of a full device, but
+  // one pass where vertices get two records or fewer on average: nearly all
+  // records then go straight to HBM, and short units keep the warps on
+  // neighbouring vertices (64 graphs of 1024..8192 vertices, 1000 edges each:
+  // 462 us, 480 with 48..64 records; 4000 edges each: 1131, 1059)
+  const uint64_t per = work / (3ull * b->sms * kApplyWarps * kApplyCtas);
+  const uint32_t chunk =
+      records <= 2 * vertices ? kStage : (uint32_t)std::min<uint64_t>(kDefaultItemRecords, (per + 16) / 16 * 16);
   for (uint32_t i = 0; i < k; i++) {
     cupc_graph* g = graphs[i];
     InstDesc& x = d[i];
@@ -352,8 +380,7 @@ cupc_status cupc_batcher_update(cupc_batcher* b, cupc_graph* const* graphs, cons
     x.cnt = g->cnt;
     x.cursor = g->cursor;
     x.rec = g->rec;
-    x.recw = g->recw;
-    x.items = g->items;
+    x.work = g->work;
     x.gc = g->gc;
     x.edge_base = base;
     x.n = (uint32_t)n[i];
@@ -363,19 +390,23 @@ cupc_status cupc_batcher_update(cupc_batcher* b, cupc_graph* const* graphs, cons
     x.D = g->D;
     x.W = g->W;
     x.P = g->P;
-    x.R = g->R;
-    x.item_records = g->item_records;
+    x.R = fold_rows(g->R, g->D);
     x.ell = g->ell;
-    x.long_depth = g->long_depth ? 1u : 0u;
+    x.small = small_ids(g->V) ? 1u : 0u;
+    x.chunk = chunk;
+    x.cap = g->rec_cap;
+    x.slice_base = slices;
     base += n[i];
-    if ((uint32_t)g->apply_threads > threads) threads = (uint32_t)g->apply_threads;
-    if (g->R > rmax) rmax = g->R;
-    if (g->L > lmax) lmax = g->L;
+    if (n[i]) slices += plan_slices(g->V);
+    units += (uint64_t)layer_groups(g->L, g->P) * (rec_entries(g->V, n[i]) / chunk + 2);
+    warp_bytes = std::max(warp_bytes, apply_warp_bytes(x.R, x.P));
   }
+  if (units >= 0xFFFFFFFFull) return CUPC_EINVAL;
   h->k = k;
   h->total_edges = base;
+  h->total_slices = slices;
   cupc_batcher::Exec* x = nullptr;
-  if (get_exec(b, threads, rmax, lmax, &x) != cudaSuccess) {
+  if (get_exec(b, warp_bytes, &x) != cudaSuccess) {
     cudaGetLastError();
     return CUPC_ECUDA;
   }

@@ -25,9 +25,10 @@ constexpr uint32_t kNoneU32 = 0xFFFFFFFFu;
 // the recovery's hook.
 constexpr uint32_t kMaxVertices = 1u << 21;
 
-// Rows per column that the update kernel folds in shared memory; deeper rows
-// (probability 2^-kSmemRows per index) are XORed straight into HBM.
-constexpr uint32_t kSmemRows = 8;      // default (the autotuner's usual pick on GB300)
+// Rows per column that the update kernel folds in shared memory (the first
+// three are folded in registers); deeper rows (probability 2^-(kSmemRows+3)
+// per index) are XORed straight into HBM. The default.
+constexpr uint32_t kSmemRows = 8;
 constexpr uint32_t kSmemRowsMax = 16;
 // Records (endpoint incidences) per update work item.
 constexpr uint32_t kItemRecords = 512;  // maximum
@@ -42,27 +43,60 @@ constexpr uint32_t kMinItemRecords = 64;
 constexpr uint32_t kPrivMaxV = 24576;
 constexpr uint32_t kPrivPerVertex = 1;
 constexpr uint32_t kPrivMinCtas = 48;
-// Most vertex slices of the update's plan kernels.
-constexpr uint32_t kPlanSlices = 1024;
-// Most CTAs of the single-graph apply kernel (its direct-path items number
-// at most 2 per CTA + 1 beyond one per 64 direct records).
-constexpr uint32_t kPlanGridCap = 8192;
-// Below this many endpoint records per vertex on average in a batch, the
-// apply kernel writes a single-item vertex back by load and store; at or
-// above it, by XOR atomics. GB300, uniform batches, ms per launch
-// (load-store / atomics): V = 2^17 and 2^18, 2^20, 2^22 edges: 1.03 / 1.25,
-// 1.47 / 1.62, 2.84 / 2.29; V = 16384 and 2^16, 2^18, 2^20 edges: 0.14 /
-// 0.18, 0.21 / 0.21, 0.48 / 0.41.
-constexpr uint32_t kExclRecords = 32;
-// Records an apply CTA stages per pass: idx and the checksums G_r(idx) of
-// every layer of kStage records sit in shared memory.
-constexpr uint32_t kStage = 64;
-// Dynamic shared memory of an apply CTA for graphs of at most L layers:
-// rows x threads fold rows, two buffers of kStage staged records, the L
-// checksums of one pass, the L layer checksum keys and two buffers of the
-// records' vertices (direct path).
-inline size_t apply_smem_bytes(uint32_t rows, uint32_t threads, uint32_t L) {
-  return (size_t)rows * threads * 16 + (size_t)kStage * 8 * (2 + L) + (size_t)L * 8 + (size_t)kStage * 2 * 4;
+// The update's plan: vertices per slice (one CTA each) and threads per CTA.
+constexpr uint32_t kPlanSlice = 1024;
+constexpr uint32_t kPlanThreads = 256;
+inline uint32_t plan_slices(uint32_t V) { return (V + kPlanSlice - 1) / kPlanSlice; }
+// Counters of one update chunk: the plan's fold and direct records, and the
+// apply kernel's next chunk of records for each layer group (at most 32,
+// since L*P <= 1024).
+constexpr uint32_t kWorkFold = 0, kWorkDirect = 1, kWorkNext = 32, kWorkSlots = 64;
+// A vertex of more than two records starts at, and is padded to, a multiple
+// of kPad records.
+constexpr uint32_t kPad = 4;
+// Entries of the record array for n edges: 2n records and the padding of the
+// vertices that have at least three.
+__host__ __device__ constexpr size_t rec_entries(size_t V, size_t n) {
+  return 2 * n + (kPad - 1) * (V < 2 * n / 3 ? V : 2 * n / 3);
+}
+// Most edges of one update chunk: its record offsets fit 32 bits.
+constexpr uint32_t kMaxChunkEdges = (1u << 31) - (1u << 22);
+static_assert(rec_entries(kMaxVertices, kMaxChunkEdges) < 0xFFFFFFFFull - 4096, "record offsets fit 32 bits");
+// Records an apply warp stages per pass (one per lane), and the distance of
+// two layers' checksums of a pass.
+constexpr uint32_t kStage = 32;
+constexpr uint32_t kStageStride = kStage + 2;
+// Warps of an apply CTA (they share nothing), and CTAs per SM its registers
+// leave room for.
+constexpr uint32_t kApplyWarps = 4;
+constexpr uint32_t kApplyCtas = 5;
+// Rows a column's lane folds on chip: 0..2 in registers, then `rows` (the
+// tunable) in shared memory.
+inline uint32_t fold_rows(uint32_t rows, uint32_t D) { return std::min(D, rows + 3); }
+// Buckets of shared memory per lane of an apply warp that folds R rows (all
+// pass through their slots on the way out), and bytes per warp: slots, kStage
+// edge ids and their checksums of 32/P layers.
+__host__ __device__ constexpr uint32_t apply_slots(uint32_t R) { return (1 + (R < 3 ? 3 : R)) | 1; }
+__host__ __device__ constexpr uint32_t apply_warp_bytes(uint32_t R, uint32_t P) {
+  return kStage * 8 + 32 * apply_slots(R) * 16 + (32 / P) * kStageStride * 8;
+}
+// Layer groups of a graph: an apply warp holds 32/P layers.
+__host__ __device__ constexpr uint32_t layer_groups(uint32_t L, uint32_t P) { return (L * P + 31) / 32; }
+// Edge ids of at most 32 bits: V^2 <= 2^32.
+inline bool small_ids(uint32_t V) { return V <= 65536; }
+// Records per chunk of a batch of nrec records on V vertices: at most `most`,
+// and such that the `warps` of a layer group run out of chunks together (a
+// whole number of chunks each, as near as steps of 16 records and the
+// padding, 1.5 records per folded vertex on average, allow); small batches in
+// quarter passes, two for every warp, as the latency of a warp's records is
+// then all that counts.
+inline uint32_t chunk_records(uint32_t nrec, uint32_t V, uint32_t warps, uint32_t most) {
+  warps = std::max(1u, warps);
+  const uint64_t all = (uint64_t)nrec + 3ull * std::min(V, nrec / 3) / 2;
+  const uint32_t per = (uint32_t)(all / warps) + 1;
+  if (per <= kStage) return std::max(kStage / 4, (per / 2 + kStage / 4 - 1) / (kStage / 4) * (kStage / 4));
+  const uint32_t rounds = (per + most - 1) / most;
+  return std::min(most, (per / rounds + 16) / 16 * 16);
 }
 // Key words of a graph: L*(C+1) (column multipliers and layer checksum
 // keys) + 3*L*C (the other multiply-add-shift words of every column).
@@ -100,8 +134,6 @@ constexpr uint64_t kWaitLimitNs = 2000000000ull;
 // Device-side counters of one graph (u32 slots of `gc`).
 enum : uint32_t {
   GC_ERR = 0,        // sticky error bits (kErrInval drops update batches)
-  GC_NITEMS = 1,     // update work items of the current chunk
-  GC_NEXT_ITEM = 2,  // dynamic scheduler cursor of the apply kernel
   GC_NFOREST = 3,
   GC_NZ = 4,         // non-ZERO samples this round
   GC_ACTIVE = 5,     // MSF: candidates still crossing two trees (even hook steps)
@@ -116,7 +148,6 @@ enum : uint32_t {
   GC_RECOVERIES = 15,
   GC_BATCHES = 16,   // update chunks applied
   GC_NBIG = 17,      // members of big components this round
-  GC_NDIRECT = 18,   // direct-path records of the current chunk
   GC_NLIVE = 19,     // live components of the next recovery round
   GC_REC_DIRTY = 20, // a recovery gave up at a barrier: its scratch may be non-zero
   GC_LABELS_VALID = 21,  // incremental mode: labels hold the current graph's components
@@ -156,7 +187,6 @@ __device__ __forceinline__ uint8_t ld_cg(const uint8_t* p) {
 struct cupc_graph {
   uint32_t V, L, C, D, W, P, R;  // P: lanes per layer in the update kernel
   uint32_t ell;                  // bits of one column-hash stage (hash_bits(V))
-  bool long_depth;               // ell < D-1 or D-1 > 32: depths may need the slow path
   uint64_t seed;
   uint32_t max_batch, max_pairs;
   void* ws;
@@ -169,7 +199,7 @@ struct cupc_graph {
   bool imported;      // words from cupc_import_sketches since the last reset:
                       // the XOR of all vertex sketches need not be zero
   int device, sms;
-  int apply_threads, apply_smem, apply_grid;
+  int apply_smem, apply_grid;
   uint32_t item_records, apply_cps;  // tunables: records per work item, CTAs per SM (0 = max)
   // optional per-batch-size settings: bucket floor(log4 edges) (at least 5)
   struct ApplyTune {
@@ -177,7 +207,6 @@ struct cupc_graph {
     uint32_t item_records, R, cps;
     int smem, grid;
   } tune_b[16];
-  uint32_t wb_b[16];  // write-back mode per bucket (CUPC_WRITEBACK_*)
   int rec_grid;
   int rec_cluster;  // CTAs of the one-cluster recovery (0: the grid-wide kernel)
   // sketches and keys
@@ -187,10 +216,9 @@ struct cupc_graph {
   // update scratch
   uint32_t* cnt;       // V
   uint32_t* cursor;    // V
-  uint64_t* rec;       // 2*max_batch
-  uint32_t* recw;      // 2*max_batch: vertex of each direct-path record
-  uint4* items;        // 4*max_batch/kMinItemRecords + min(V, 2*max_batch) + 1
-  uint4* part;         // kPlanSlices per-slice totals of the plan
+  uint64_t* rec;       // rec_cap endpoint records, grouped by vertex
+  uint32_t rec_cap;
+  uint32_t* work;      // kWorkSlots counters of the current chunk
   uint32_t* stage_edges;  // 2*max_batch (host-input staging slot 0)
   int8_t* stage_ops;      // max_batch
   uint32_t* stage_edges1;  // 2*max_batch (slot 1)
@@ -282,7 +310,7 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
 cudaError_t launch_validate(cupc_graph* g, const uint32_t* edges, const int8_t* ops, size_t n, cudaStream_t s);
 cudaError_t setup_update(cupc_graph* g);
 cudaError_t configure_apply(cupc_graph* g);
-cudaError_t apply_config(const cupc_graph* g, uint32_t item_records, uint32_t R, uint32_t cps, int* smem, int* grid);
+cudaError_t apply_config(const cupc_graph* g, uint32_t R, uint32_t cps, int* smem, int* grid);
 // Tuning bucket of a batch of n edges: floor(log4 n), at least 5, at most 15.
 inline uint32_t tune_bucket(size_t n) {
   uint32_t b = 5;

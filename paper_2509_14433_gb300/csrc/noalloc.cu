@@ -2,8 +2,7 @@
 //
 // cupc_update_sketch_static applies a batch of edge updates to a sketch
 // buffer the caller owns, using the same kernels as cupc_update_batch. Its
-// scratch (per-vertex counts and cursors, endpoint records, work items, hash
-// keys, counters) is the file-scope array below instead of a workspace, so
+// scratch (per-vertex counts and cursors, endpoint records, hash keys, counters) is the file-scope array below instead of a workspace, so
 // the call allocates nothing. The paper has no counterpart of this entry
 // point.
 #include <mutex>
@@ -20,19 +19,16 @@ constexpr uint32_t kMaxEdges = CUPC_STATIC_MAX_EDGES;
 constexpr uint32_t kMaxKeys = (uint32_t)key_words(18, 7);
 constexpr size_t kAlignS = 256;
 constexpr size_t align_s(size_t x) { return (x + kAlignS - 1) / kAlignS * kAlignS; }
-constexpr size_t kMaxItems =
-    4ull * kMaxEdges / kMinItemRecords + (kMaxV < 2ull * kMaxEdges ? kMaxV : 2ull * kMaxEdges) + 2ull * kPlanGridCap + 1;
 // byte offsets inside the static scratch
 constexpr size_t kOffGc = 0;
 constexpr size_t kOffKeys = align_s(kOffGc + GC_SLOTS * sizeof(uint32_t));
 constexpr size_t kOffCnt = align_s(kOffKeys + kMaxKeys * sizeof(uint64_t));
 constexpr size_t kOffCursor = align_s(kOffCnt + kMaxV * sizeof(uint32_t));
 constexpr size_t kOffRec = align_s(kOffCursor + kMaxV * sizeof(uint32_t));
-constexpr size_t kOffRecw = align_s(kOffRec + 2ull * kMaxEdges * sizeof(uint64_t));
-constexpr size_t kOffItems = align_s(kOffRecw + 2ull * kMaxEdges * sizeof(uint32_t));
-constexpr size_t kOffPart = align_s(kOffItems + kMaxItems * sizeof(uint4));
-constexpr size_t kScratchBytes = align_s(kOffPart + kPlanSlices * sizeof(uint4));
-static_assert(kScratchBytes == CUPC_STATIC_SCRATCH_BYTES, "the header states the size of the static scratch");
+constexpr size_t kRecCap = rec_entries(kMaxV, kMaxEdges);
+constexpr size_t kOffWork = align_s(kOffRec + kRecCap * sizeof(uint64_t));
+constexpr size_t kScratchBytes = CUPC_STATIC_SCRATCH_BYTES;
+static_assert(kOffWork + kWorkSlots * sizeof(uint32_t) <= kScratchBytes, "the header states the size of the static scratch");
 
 // Shared by every call on a device, kept between calls.
 static __device__ __align__(256) unsigned char cupc_static_scratch[kScratchBytes];
@@ -43,7 +39,7 @@ struct DeviceSetup {
   bool done;
   cudaError_t err;
   unsigned char* scratch;
-  int sms, apply_threads, apply_smem, apply_grid;
+  int sms, apply_smem, apply_grid;
   uint32_t P, R;
 };
 constexpr int kMaxDevices = 64;
@@ -80,7 +76,6 @@ cudaError_t device_setup(int dev, DeviceSetup** out) {
       fill_dims(g, kMaxV);
       g.sms = s.sms;
       err = setup_update(&g);
-      s.apply_threads = g.apply_threads;
       s.apply_smem = g.apply_smem;
       s.apply_grid = g.apply_grid;
       s.P = g.P;
@@ -132,10 +127,8 @@ extern "C" cupc_status cupc_update_sketch_static(void* sketch, uint32_t V, uint6
   g.P = ds->P;
   g.R = g.D < kSmemRows ? g.D : kSmemRows;
   g.ell = hash_bits(V);
-  g.long_depth = g.ell < g.D - 1 || g.D - 1 > 32;
   g.item_records = kDefaultItemRecords;
-  g.apply_threads = (int)(((g.L * g.P) + 31) / 32 * 32);
-  g.apply_smem = (int)apply_smem_bytes(g.R, (uint32_t)g.apply_threads, g.L);
+  g.apply_smem = (int)(kApplyWarps * apply_warp_bytes(fold_rows(g.R, g.D), g.P));
   // the set-up sized the launch for the widest graph; a narrower one fits
   g.apply_grid = ds->apply_grid;
   g.prof_on = false;
@@ -145,9 +138,8 @@ extern "C" cupc_status cupc_update_sketch_static(void* sketch, uint32_t V, uint6
   g.cnt = (uint32_t*)(ds->scratch + kOffCnt);
   g.cursor = (uint32_t*)(ds->scratch + kOffCursor);
   g.rec = (uint64_t*)(ds->scratch + kOffRec);
-  g.recw = (uint32_t*)(ds->scratch + kOffRecw);
-  g.items = (uint4*)(ds->scratch + kOffItems);
-  g.part = (uint4*)(ds->scratch + kOffPart);
+  g.rec_cap = (uint32_t)kRecCap;
+  g.work = (uint32_t*)(ds->scratch + kOffWork);
 
   // the array keeps the previous call's contents: clear what must start at 0
   if (cudaMemsetAsync(g.gc, 0, GC_SLOTS * sizeof(uint32_t), s) != cudaSuccess) return CUPC_ECUDA;

@@ -2,27 +2,17 @@
 // Algorithm": an update of edge (u,v) updates every sketch of u and of v;
 // Theorem A.2: CameoSketch touches one bucket per column per update).
 //
-// One chunk of <= max_batch edges goes through five stream-ordered kernels
-// (a batch is validated whole by k_validate first, or, when it is one chunk
-// that k_count_priv counts, inside k_count_priv):
+// One chunk of <= max_batch edges goes through four stream-ordered kernels (a
+// batch of several chunks is validated whole by k_validate first, a batch of
+// one chunk inside the count):
 //   k_count   per-vertex record counts (2 records per edge, one per
 //             endpoint); k_count_priv for dense batches on small graphs,
 //             through per-CTA shared histograms
-//   k_plan_count / k_plan_write
-//             exclusive scan over vertex slices -> per-vertex cursors and
-//             work items: at most item_records records of one vertex, or
-//             16..64 records of vertices with at most 2 (the direct path)
-//   k_scatter endpoint records (the edge index u*V+v) grouped by vertex
+//   k_plan    a segment of the record array for every vertex
+//   k_scatter endpoint records (vertex, other end) grouped by vertex
 //             (k_scatter_priv with k_count_priv)
-//   k_apply   persistent CTAs, CTA b starting on item b; the CTA stages
-//             the item's records 64 at a time with their checksum of every
-//             layer (one SplitMix64 per record and layer), then thread
-//             (layer r, slot s) takes the multiply-add-shift depth of each
-//             record in column s of layer r (slot C owns the deterministic
-//             bucket), folds it into shared-memory rows, and finally
-//             read-modify-writes only the touched buckets of that vertex in
-//             HBM with 16-byte accesses; direct items XOR each bucket
-//             straight into HBM.
+//   k_apply   persistent warps; a warp owns some layers of the graph and takes
+//             chunks of the record array (apply_chunk)
 // XOR is associative and commutative, so the result is bit-identical to
 // applying the updates one by one in stream order.
 #include "update_dev.cuh"
@@ -60,12 +50,30 @@ cudaError_t launch_validate(cupc_graph* g, const uint32_t* edges, const int8_t* 
   return cudaGetLastError();
 }
 
-__global__ void k_count(const uint32_t* __restrict__ edges, size_t n, uint32_t* cnt, const uint32_t* gc) {
+// The plan's record counts and the apply kernel's chunk counters start at 0.
+__device__ __forceinline__ void reset_work(uint32_t* work) {
+  if (blockIdx.x == 0 && threadIdx.x < kWorkSlots) work[threadIdx.x] = 0;
+}
+
+// With ops (a batch of one chunk) it also validates the batch as k_validate
+// does, saving that pass; counts of an invalid batch are cleared by k_plan.
+__global__ void k_count(const uint32_t* __restrict__ edges, const int8_t* __restrict__ ops, size_t n, uint32_t V,
+                        uint32_t* cnt, uint32_t* work, uint32_t* gc) {
   if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
+  reset_work(work);
+  bool bad = false;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    atomicAdd(&cnt[edges[2 * i]], 1u);
-    atomicAdd(&cnt[edges[2 * i + 1]], 1u);
+    const uint32_t u = edges[2 * i], v = edges[2 * i + 1];
+    if (ops) {
+      const int8_t op = ops[i];
+      bad |= (u >= V) | (v >= V) | (u == v) | ((op != 1) & (op != -1));
+    }
+    if (u < V && v < V) {
+      atomicAdd(&cnt[u], 1u);
+      atomicAdd(&cnt[v], 1u);
+    }
   }
+  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&gc[GC_ERR], kErrInval);
 }
 
 // Dense batches on small graphs (V <= kPrivMaxV, at least kPrivPerVertex
@@ -73,14 +81,12 @@ __global__ void k_count(const uint32_t* __restrict__ edges, size_t n, uint32_t* 
 // batch and counts its endpoints in a shared histogram of all V vertices, so
 // the global counters see one atomic per (CTA, vertex) instead of one per
 // record.
-// With ops (a batch of one chunk) it also validates the batch as k_validate
-// does, saving that pass; counts of an invalid batch are cleared by
-// k_plan_write.
 __global__ void __launch_bounds__(1024) k_count_priv(const uint32_t* __restrict__ edges,
                                                      const int8_t* __restrict__ ops, size_t n, uint32_t V,
-                                                     uint32_t* cnt, uint32_t* gc) {
+                                                     uint32_t* cnt, uint32_t* work, uint32_t* gc) {
   extern __shared__ uint32_t s_h[];  // V
   if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
+  reset_work(work);
   for (uint32_t w = threadIdx.x; w < V; w += blockDim.x) s_h[w] = 0;
   __syncthreads();
   const size_t chunk = (n + gridDim.x - 1) / gridDim.x, lo = blockIdx.x * chunk, hi = min(n, lo + chunk);
@@ -110,11 +116,10 @@ __global__ void __launch_bounds__(1024) k_count_priv(const uint32_t* __restrict_
 // land in a different order than with k_scatter; XOR does not see order.
 __global__ void __launch_bounds__(1024) k_scatter_priv(const uint32_t* __restrict__ edges, size_t n, uint32_t V,
                                                        uint32_t* cursor, uint64_t* __restrict__ rec,
-                                                       uint32_t* __restrict__ recw, const uint32_t* gc) {
+                                                       const uint32_t* gc) {
   extern __shared__ uint32_t s_h[];  // V counts, then V range starts
   uint32_t* s_base = s_h + V;
   if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
-  const uint32_t nd = ld_cg(&gc[GC_NDIRECT]);
   for (uint32_t w = threadIdx.x; w < V; w += blockDim.x) s_h[w] = 0;
   __syncthreads();
   const size_t chunk = (n + gridDim.x - 1) / gridDim.x, lo = blockIdx.x * chunk, hi = min(n, lo + chunk);
@@ -131,12 +136,9 @@ __global__ void __launch_bounds__(1024) k_scatter_priv(const uint32_t* __restric
   __syncthreads();
   for (size_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
     const uint32_t u = edges[2 * i], v = edges[2 * i + 1];
-    const uint64_t idx = (uint64_t)min(u, v) * V + max(u, v);
     const uint32_t pu = s_base[u] + atomicAdd(&s_h[u], 1u), pv = s_base[v] + atomicAdd(&s_h[v], 1u);
-    rec[pu] = idx;
-    rec[pv] = idx;
-    if (pu < nd) recw[pu] = u;
-    if (pv < nd) recw[pv] = v;
+    rec[pu] = make_record(u, v);
+    rec[pv] = make_record(v, u);
   }
 }
 
@@ -332,175 +334,80 @@ cudaError_t launch_incremental(cupc_graph* g, const uint32_t* edges, const int8_
   return cudaGetLastError();
 }
 
-// Work plan of one chunk over many CTAs, in two launches that never wait on
-// one another. The vertices are cut into slices of 256 * vpt; slice b is
-// planned by CTA b. Kinds of vertices and the layout of records and items
-// are those of plan_vertices: direct-path vertices (<= kDirectMax records)
-// first in rec, then fold vertices, whose records are cut into items of
-// item_records; direct items of kDirectItemRecords follow the fold items.
-//
-// k_plan_count: per-slice totals {fold records, direct records, fold items}.
-__global__ void __launch_bounds__(256) k_plan_count(const uint32_t* __restrict__ cnt, uint32_t V, uint32_t vpt,
-                                                    uint32_t item_records, uint4* part, const uint32_t* gc) {
-  __shared__ uint32_t sw[3][32];
+// The work plan of one chunk (plan_slice), one CTA per slice of vertices.
+__global__ void __launch_bounds__(kPlanThreads) k_plan(uint32_t* cnt, uint32_t* cursor, uint64_t* rec, uint32_t V,
+                                                       uint32_t cap, uint32_t* work, uint32_t* gc) {
+  const bool dropped = (ld_cg(&gc[GC_ERR]) & kErrInval) != 0;  // a dropped batch may have counted: start clean
+  plan_slice(cnt, cursor, rec, V, cap, blockIdx.x, work, dropped);
+  if (!dropped && blockIdx.x == 0 && threadIdx.x == 0) gc[GC_BATCHES] += 1;
+}
+
+__global__ void k_scatter(const uint32_t* __restrict__ edges, size_t n, uint32_t* cursor, uint64_t* __restrict__ rec,
+                          const uint32_t* gc) {
   if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
-  const uint32_t lo = blockIdx.x * blockDim.x * vpt, hi = min(V, lo + blockDim.x * vpt);
-  uint32_t v[3] = {0, 0, 0};
-  for (uint32_t w = lo + threadIdx.x; w < hi; w += blockDim.x) {
-    const uint32_t c = cnt[w];
-    if (c > kDirectMax) {
-      v[0] += c;
-      v[2] += (c + item_records - 1) / item_records;
-    } else {
-      v[1] += c;
-    }
-  }
-  uint32_t e[3], t[3];
-  block_scan3(v, e, t, sw);
-  if (threadIdx.x == 0) part[blockIdx.x] = make_uint4(t[0], t[1], t[2], 0u);
-}
-
-// k_plan_write: CTA b adds up the totals of slices < b (its offsets) and of
-// all slices (direct records nd, fold items), then scans its slice 256
-// vertices at a time, writing cursors and fold items; every CTA writes a
-// share of the direct items. Resets cnt for the next chunk.
-__global__ void __launch_bounds__(256) k_plan_write(uint32_t* cnt, uint32_t* cursor, uint4* items, uint32_t V,
-                                                    uint32_t vpt, uint32_t item_records, const uint4* __restrict__ part,
-                                                    uint32_t apply_ctas, uint32_t* gc) {
-  __shared__ uint32_t sw[3][32];
-  const uint32_t nb = gridDim.x, b = blockIdx.x;
-  if (ld_cg(&gc[GC_ERR]) & kErrInval) {  // a dropped batch may have counted: start clean
-    const uint32_t lo = b * blockDim.x * vpt, hi = min(V, lo + blockDim.x * vpt);
-    for (uint32_t w = lo + threadIdx.x; w < hi; w += blockDim.x) cnt[w] = 0;
-    return;
-  }
-  // offsets of this slice and the grand totals
-  uint32_t before[3] = {0, 0, 0}, all[3] = {0, 0, 0};
-  for (uint32_t j = threadIdx.x; j < nb; j += blockDim.x) {
-    const uint4 p = part[j];
-    all[0] += p.x;
-    all[1] += p.y;
-    all[2] += p.z;
-    if (j < b) {
-      before[0] += p.x;
-      before[1] += p.y;
-      before[2] += p.z;
-    }
-  }
-  uint32_t e[3], tb[3], ta[3];
-  block_scan3(before, e, tb, sw);
-  block_scan3(all, e, ta, sw);
-  const uint32_t nd = ta[1], nfold = ta[2];
-  uint32_t carry[3] = {nd + tb[0], tb[1], tb[2]};  // next fold record, direct record, fold item
-  const uint32_t lo = b * blockDim.x * vpt, hi = min(V, lo + blockDim.x * vpt);
-  for (uint32_t base = lo; base < hi; base += blockDim.x) {
-    const uint32_t w = base + threadIdx.x;
-    const uint32_t c = w < hi ? cnt[w] : 0;
-    const bool fold = c > kDirectMax;
-    const uint32_t ni = fold ? (c + item_records - 1) / item_records : 0;
-    const uint32_t v[3] = {fold ? c : 0, fold ? 0 : c, ni};
-    uint32_t t[3];
-    block_scan3(v, e, t, sw);
-    if (w < hi) {
-      cnt[w] = 0;
-      if (fold) {
-        const uint32_t pf = carry[0] + e[0], pi = carry[2] + e[2];
-        cursor[w] = pf;
-        for (uint32_t q = 0; q < ni; q++) {
-          const uint32_t bg = pf + q * item_records;
-          items[pi + q] = make_uint4(w, bg, min(pf + c, bg + item_records), ni == 1 ? 1u : 0u);
-        }
-      } else {
-        cursor[w] = carry[1] + e[1];
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 3; k++) carry[k] += t[k];
-  }
-  // direct items: about two per apply CTA, of kDirectItemMin..kDirectItemRecords
-  // records (so at most max(2 * apply_ctas + 1, nd / kDirectItemRecords + 1))
-  const uint32_t dsz = min(kDirectItemRecords, max(kDirectItemMin, (nd + 2 * apply_ctas - 1) / (2 * apply_ctas)));
-  const uint32_t ndi = (nd + dsz - 1) / dsz;
-  for (uint32_t q = b * blockDim.x + threadIdx.x; q < ndi; q += nb * blockDim.x)
-    items[nfold + q] = make_uint4(kDirectItem, q * dsz, min(nd, (q + 1) * dsz), 0u);
-  if (b == 0 && threadIdx.x == 0) {
-    gc[GC_NITEMS] = nfold + ndi;
-    gc[GC_NDIRECT] = nd;
-    gc[GC_NEXT_ITEM] = 0;
-    gc[GC_BATCHES] += 1;
-  }
-}
-
-// Slice width of the plan kernels: at most kPlanSlices slices.
-uint32_t plan_vpt(uint32_t V) {
-  const uint32_t per = 256u * kPlanSlices;
-  return std::max(1u, (V + per - 1) / per);
-}
-
-__global__ void k_scatter(const uint32_t* __restrict__ edges, size_t n, uint32_t V, uint32_t* cursor,
-                          uint64_t* __restrict__ rec, uint32_t* __restrict__ recw, const uint32_t* gc) {
-  if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
-  const uint32_t nd = ld_cg(&gc[GC_NDIRECT]);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    uint32_t u = edges[2 * i], v = edges[2 * i + 1];
-    uint32_t a = min(u, v), b = max(u, v);
-    uint64_t idx = (uint64_t)a * V + b;
+    const uint32_t u = edges[2 * i], v = edges[2 * i + 1];
     const uint32_t pu = atomicAdd(&cursor[u], 1u), pv = atomicAdd(&cursor[v], 1u);
-    rec[pu] = idx;
-    rec[pv] = idx;
-    if (pu < nd) recw[pu] = u;
-    if (pv < nd) recw[pv] = v;
+    rec[pu] = make_record(u, v);
+    rec[pv] = make_record(v, u);
   }
 }
 
-// Fold the records of one work item into the sketches of its vertex (see
-// apply_item); persistent CTAs pull work items from a counter. kExcl: a
-// vertex with a single item writes back by load and store, else every
-// write-back is by XOR atomics (the launch picks by records per vertex).
-template <bool kLong, bool kExcl>
-__global__ void k_apply(ulonglong2* __restrict__ sketch, const uint64_t* __restrict__ keys,
-                        const uint64_t* __restrict__ rec, const uint32_t* __restrict__ recw,
-                        const uint4* __restrict__ items, uint32_t* gc, uint32_t V, uint32_t L, uint32_t C,
-                        uint32_t D, uint32_t W, uint32_t P, uint32_t R, uint32_t ell) {
+// Apply the records, in chunks of `chunk` records (apply_chunk). A warp keeps
+// the layer group (its number modulo the groups). Its first two chunks are
+// given, the others come from the group's counter, asked for two chunks
+// ahead, so that the next chunk's records load while it works on this one.
+//
+// What bounds it. Batches of many records per vertex: instruction issue and
+// the ALU (64 lanes a cycle per SM), which folding rows 0..2 in registers and
+// the write-back by bulk reductions leave as the limit: per warp (4 layers x 8
+// lanes) and record about 40 instructions, 20 of them on the ALU. Batches of
+// few records per vertex: the rate of separate runs in HBM (20..29 G runs/s
+// for runs of 16..64 bytes, 15 G/s for 128), so a column's rows go out as one
+// run: one bulk XOR reduction moves 117 G buckets/s, 64-bit atomics 60 G/s,
+// load and store 68 G/s (V = 2^17, runs of 8 buckets). Against the kernel
+// that folded every row in shared memory and wrote back by atomics, GB300, us
+// per batch: V = 5003, 30011 edges: 59 (78); V = 65536, 10^5, 10^6 edges: 400,
+// 763 (460, 942); V = 2^17, 3*10^5 edges: 990 (1083).
+template <bool kX32>
+__global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply(
+    ulonglong2* __restrict__ sketch, const uint64_t* __restrict__ keys, const uint64_t* __restrict__ rec, uint32_t cap,
+    uint32_t chunk, uint32_t* work, const uint32_t* gc, uint32_t V, uint32_t L, uint32_t C, uint32_t D, uint32_t W,
+    uint32_t P, uint32_t R, uint32_t ell) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const ApplySmem m = apply_smem(smem_raw, R, L);
-  __shared__ uint32_t s_item;
-
   if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
-  // CTA b starts with item b; CTAs beyond the items leave before touching
-  // the item counter (a small batch would otherwise have every CTA of the
-  // grid queue on one address); a CTA that finishes takes the next item
-  // from the counter, which counts from the grid size
-  const uint32_t nitems = ld_cg(&gc[GC_NITEMS]);
-  if (blockIdx.x >= nitems) return;
-  const ApplyLane l = apply_lane(keys, L, C, D, P, R, ell);
-  load_kchk(m, keys, L, C);
-  ulonglong2* my_rows = m.rows + threadIdx.x;
-  const uint32_t rs = blockDim.x;
-  for (uint32_t d = 0; d < R; d++) my_rows[d * rs] = make_ulonglong2(0, 0);
-  __syncthreads();
-
-  for (uint32_t it = blockIdx.x; it < nitems;) {
-    const uint4 item = items[it];
-    if (item.x == kDirectItem) {
-      apply_direct<kLong>(l, sketch, V, W, rec + item.y, recw + item.y, item.z - item.y, L, m);
-    } else {
-      ulonglong2* gb = sketch + ((size_t)l.layer * V + item.x) * W + l.jbase;
-      apply_item<kLong>(l, gb, rec + item.y, item.z - item.y, kExcl && item.w != 0, L, R, m, my_rows, rs);
-    }
-    // both item paths end with __syncthreads: every thread has read s_item
-    if (threadIdx.x == 0) s_item = gridDim.x + atomicAdd(&gc[GC_NEXT_ITEM], 1u);
-    __syncthreads();
-    it = s_item;
+  const uint32_t nslots = apply_slots(R);
+  const uint32_t gw = blockIdx.x * kApplyWarps + (threadIdx.x >> 5), groups = layer_groups(L, P);
+  const uint32_t group = gw % groups, warps = (gridDim.x * kApplyWarps - group + groups - 1) / groups;
+  const ChunkPlan c = chunk_plan(work, chunk);
+  uint32_t q = gw / groups;
+  if (q >= c.total) return;
+  const ApplySmem m = apply_smem(smem_raw + (threadIdx.x >> 5) * apply_warp_bytes(R, P), nslots, P);
+  const ApplyLane l = apply_lane(keys, sketch, V, L, C, D, W, P, ell, group);
+  zero_slots(m, nslots);
+  LaneSums a;
+  clear_sums(a);
+  a.dirty = 0;
+  bool pending = false;
+  Chunk k = chunk_at(c, q, chunk, rec, cap);
+  uint64_t r = load_record(k, 0, k);
+  q += warps;
+  while (k.n) {
+    const Chunk next = chunk_at(c, q, chunk, rec, cap);
+    uint32_t ahead = q;
+    if ((threadIdx.x & 31) == 0 && next.n) ahead = 2 * warps + atomicAdd(&work[kWorkNext + group], 1u);
+    apply_chunk<kX32>(l, m, a, pending, k, next, r, V, W, C, P, R);
+    q = __shfl_sync(0xffffffffu, ahead, 0);
+    k = next;
   }
+  bulk_wait_all();
 }
 
 // The dynamic shared-memory limit of k_apply is process-wide: only ever
 // raise it, so that a graph created later never shrinks it below what an
 // earlier graph's launches need.
 cudaError_t raise_apply_smem_limit(int bytes) {
-  const void* fns[4] = {(const void*)k_apply<false, false>, (const void*)k_apply<true, false>,
-                        (const void*)k_apply<false, true>, (const void*)k_apply<true, true>};
+  const void* fns[2] = {(const void*)k_apply<false>, (const void*)k_apply<true>};
   for (const void* f : fns) {
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, f);
@@ -522,22 +429,20 @@ cudaError_t setup_update(cupc_graph* g) {
   while (g->P < g->C + 1) g->P <<= 1;
   g->R = g->D < kSmemRows ? g->D : kSmemRows;
   g->ell = hash_bits(g->V);
-  g->long_depth = g->ell < g->D - 1 || g->D - 1 > 32;
   g->item_records = kDefaultItemRecords;
   g->apply_cps = 0;
-  g->apply_threads = (int)(((g->L * g->P) + 31) / 32 * 32);
   return configure_apply(g);
 }
 
 // Shared memory and persistent grid of k_apply for the given tunables.
-cudaError_t apply_config(const cupc_graph* g, uint32_t item_records, uint32_t R, uint32_t cps, int* smem, int* grid) {
-  *smem = (int)apply_smem_bytes(R, (uint32_t)g->apply_threads, g->L);
+cudaError_t apply_config(const cupc_graph* g, uint32_t R, uint32_t cps, int* smem, int* grid) {
+  // the tunable's range: R rows of every lane of the graph within one SM
+  if ((size_t)R * layer_groups(g->L, g->P) * 512 + (size_t)g->L * 520 + 1536 > 232448) return cudaErrorInvalidValue;
+  *smem = (int)(kApplyWarps * apply_warp_bytes(fold_rows(R, g->D), g->P));
   cudaError_t e = raise_apply_smem_limit(*smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm,
-                                                    g->long_depth ? k_apply<true, false> : k_apply<false, false>,
-                                                    g->apply_threads, *smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_apply<false>, 32 * kApplyWarps, *smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   if (cps && (int)cps < per_sm) per_sm = (int)cps;
@@ -547,7 +452,7 @@ cudaError_t apply_config(const cupc_graph* g, uint32_t item_records, uint32_t R,
 
 // ... and for the graph's default tunables.
 cudaError_t configure_apply(cupc_graph* g) {
-  return apply_config(g, g->item_records, g->R, g->apply_cps, &g->apply_smem, &g->apply_grid);
+  return apply_config(g, g->R, g->apply_cps, &g->apply_smem, &g->apply_grid);
 }
 
 cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, cudaStream_t s,
@@ -563,40 +468,32 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
     smem = t.smem;
     grid_max = t.grid;
   }
-  const int agrid = (int)std::min<size_t>(std::min<size_t>((size_t)grid_max, 2 * n), kPlanGridCap);
-  int grid = (int)std::min<size_t>((n + 255) / 256, (size_t)g->sms * 8);
-  // dense batch on a small graph: group through shared histograms (and
-  // validate there); else validate in a pass of its own
+  const int grid = (int)std::min<size_t>((n + 255) / 256, (size_t)g->sms * 8);
+  // dense batch on a small graph: group through shared histograms
   const int pgrid = (int)std::min<size_t>((size_t)g->sms, 2 * n / ((size_t)kPrivPerVertex * g->V));
   const bool priv = g->V <= kPrivMaxV && pgrid >= (int)kPrivMinCtas;
-  if (!priv && validate_ops) {
-    cudaError_t e = launch_validate(g, edges, validate_ops, n, s);
-    if (e != cudaSuccess) return e;
-  }
+  const uint32_t nrec = (uint32_t)(2 * n);
   {
-    ProfScope ps(g, s, PC_GROUP, 4);
+    ProfScope ps(g, s, PC_GROUP, 3);
     if (priv)
-      k_count_priv<<<pgrid, 1024, 4 * g->V, s>>>(edges, validate_ops, n, g->V, g->cnt, g->gc);
+      k_count_priv<<<pgrid, 1024, 4 * g->V, s>>>(edges, validate_ops, n, g->V, g->cnt, g->work, g->gc);
     else
-      k_count<<<grid, 256, 0, s>>>(edges, n, g->cnt, g->gc);
-    const uint32_t vpt = plan_vpt(g->V), nb = (g->V + 256 * vpt - 1) / (256 * vpt);
-    k_plan_count<<<nb, 256, 0, s>>>(g->cnt, g->V, vpt, ir, g->part, g->gc);
-    k_plan_write<<<nb, 256, 0, s>>>(g->cnt, g->cursor, g->items, g->V, vpt, ir, g->part, (uint32_t)agrid, g->gc);
+      k_count<<<grid, 256, 0, s>>>(edges, validate_ops, n, g->V, g->cnt, g->work, g->gc);
+    k_plan<<<plan_slices(g->V), kPlanThreads, 0, s>>>(g->cnt, g->cursor, g->rec, g->V, g->rec_cap, g->work, g->gc);
     if (priv)
-      k_scatter_priv<<<pgrid, 1024, 8 * g->V, s>>>(edges, n, g->V, g->cursor, g->rec, g->recw, g->gc);
+      k_scatter_priv<<<pgrid, 1024, 8 * g->V, s>>>(edges, n, g->V, g->cursor, g->rec, g->gc);
     else
-      k_scatter<<<grid, 256, 0, s>>>(edges, n, g->V, g->cursor, g->rec, g->recw, g->gc);
+      k_scatter<<<grid, 256, 0, s>>>(edges, n, g->cursor, g->rec, g->gc);
   }
   ProfScope ps(g, s, PC_APPLY, 1);
-  // the bucket's write-back mode; by default load-then-store for a vertex's
-  // single item when the chunk averages fewer than kExclRecords endpoint
-  // records per vertex (most touched rows then hold one or two records)
-  const uint32_t wb = g->wb_b[tune_bucket(n)];
-  const bool excl = wb == CUPC_WRITEBACK_AUTO ? 2 * n < (size_t)kExclRecords * g->V : wb == CUPC_WRITEBACK_LOAD_STORE;
-  auto kern = g->long_depth ? (excl ? k_apply<true, true> : k_apply<true, false>)
-                            : (excl ? k_apply<false, true> : k_apply<false, false>);
-  kern<<<agrid, g->apply_threads, smem, s>>>(g->sketch, g->keys, g->rec, g->recw, g->items, g->gc, g->V, g->L, g->C,
-                                              g->D, g->W, g->P, R, g->ell);
+  const uint32_t groups = layer_groups(g->L, g->P);
+  const uint32_t chunk = chunk_records(nrec, g->V, (uint32_t)grid_max * kApplyWarps / groups, ir);
+  // at most: chunks of padded fold records and of direct records
+  const size_t units = (size_t)(rec_entries(g->V, n) / chunk + 2) * groups;
+  const int agrid = (int)std::min<size_t>((size_t)grid_max, (units + kApplyWarps - 1) / kApplyWarps);
+  auto kern = small_ids(g->V) ? k_apply<true> : k_apply<false>;
+  kern<<<agrid, 32 * kApplyWarps, smem, s>>>(g->sketch, g->keys, g->rec, g->rec_cap, chunk, g->work, g->gc, g->V,
+                                             g->L, g->C, g->D, g->W, g->P, fold_rows(R, g->D), g->ell);
   return cudaGetLastError();
 }
 
@@ -605,7 +502,7 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
 extern "C" cupc_status cupc_build_info(int* binary_version, int* ptx_version) {
   if (!binary_version || !ptx_version) return CUPC_EINVAL;
   cudaFuncAttributes fa;
-  if (cudaFuncGetAttributes(&fa, (const void*)cupc::k_apply<false, false>) != cudaSuccess) {
+  if (cudaFuncGetAttributes(&fa, (const void*)cupc::k_apply<false>) != cudaSuccess) {
     cudaGetLastError();
     return CUPC_ECUDA;
   }

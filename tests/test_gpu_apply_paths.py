@@ -1,0 +1,89 @@
+"""The update's apply kernels at the sizes where a path can go wrong, every
+sketch word against the oracle: vertices whose record counts sit at the edges
+of the direct path, the padding, a pass and a chunk; every lane layout (1 to 31
+columns); rows that end inside the registers, the shared slots or HBM; edge
+ids above and below 32 bits; batches around the one-launch limit. The path is
+integer, so equality is exact."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2509_14433_gb300 import workloads as WL
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def _stars(V, counts, g):
+    """A batch in which hub i has counts[i] records, the hubs spread over the
+    ids so that both smaller and larger endpoints occur."""
+    hubs = (np.arange(len(counts)) * (V // (len(counts) + 1)) + 3).astype(np.int64)
+    free = np.setdiff1d(np.arange(V), hubs)
+    e = np.concatenate([np.stack([np.full(c, h), g.choice(free, c, replace=False)], 1) for h, c in zip(hubs, counts)])
+    return e[g.permutation(len(e))].astype(np.uint32)
+
+
+COUNTS = (1, 2, 3, 4, 5, 7, 8, 31, 32, 33, 63, 64, 65, 255, 256, 257, 511, 700)
+
+
+@pytest.mark.parametrize("V,L,C,D", [(3000, 0, 0, 0), (70001, 3, 2, 5), (66000, 2, 7, 20)])
+@pytest.mark.parametrize("rows", [1, 8, 16])
+def test_record_counts_at_the_edges_of_passes_and_chunks(V, L, C, D, rows):
+    from paper_2509_14433_gb300 import cupc as B
+    from tests._dev import Dev
+
+    dev, ref = Dev(V, 5, (L, C, D, 0)), O.Graph(V, 5, L, C, D)
+    assert B.cupc_set_tuning(dev.h, 64 if rows == 1 else 0, min(rows, dev.D), 0) == 0
+    g = WL.rng(V + rows)
+    e = np.concatenate([_stars(V, COUNTS * 2, g), WL.uniform_pairs(V, 3000, g)])
+    assert len(e) > 4096  # the grouped path
+    assert dev.update(e) == 0 and ref.update(e) == O.OK
+    assert dev.sync() == 0
+    assert np.array_equal(dev.export(), ref.export())
+
+
+@pytest.mark.parametrize("C", [1, 2, 3, 4, 7, 8, 15, 16, 31])
+@pytest.mark.parametrize("D", [1, 2, 3, 4, 7])
+def test_every_lane_layout(C, D):
+    from tests._dev import Dev
+
+    V, L = 500, 5
+    dev, ref = Dev(V, 9, (L, C, D, 0)), O.Graph(V, 9, L, C, D)
+    g = WL.rng(C * 10 + D)
+    for n in (300, 6000):  # one launch; grouped
+        e = WL.uniform_pairs(V, n, g)
+        assert dev.update(e) == 0 and ref.update(e) == O.OK
+    assert dev.sync() == 0
+    assert np.array_equal(dev.export(), ref.export())
+
+
+@pytest.mark.parametrize("n", [1, 31, 4095, 4096, 4097])
+def test_batches_around_the_one_launch_limit(n):
+    from paper_2509_14433_gb300 import cupc as B
+    from tests._dev import Dev
+
+    V = 1500
+    dev, ref = Dev(V, 2), O.Graph(V, 2)
+    g = WL.rng(n)
+    e = WL.uniform_pairs(V, n, g)
+    e[: n // 2, 0] = 7  # a hub
+    e[: n // 2, 1] = np.where(e[: n // 2, 1] == 7, 8, e[: n // 2, 1])
+    assert dev.update(e) == 0 and ref.update(e) == O.OK
+    for at, bad in ((0, (V, 1)), (n - 1, (3, 3)), (n // 2, (0, V))):  # dropped whole, then the next one applies
+        b = e.copy()
+        b[at] = bad
+        assert dev.update(b) == 0 and dev.sync() == B.CUPC_EINVAL
+    ops = np.ones(n, np.int8)
+    ops[n - 1] = 0
+    assert dev.update(e, ops) == 0 and dev.sync() == B.CUPC_EINVAL
+    assert np.array_equal(dev.export(), ref.export())
+    assert dev.update(e[:1]) == 0 and ref.update(e[:1]) == O.OK
+    assert dev.sync() == 0 and dev.stats()["chunks"] == 2
+    assert np.array_equal(dev.export(), ref.export())
