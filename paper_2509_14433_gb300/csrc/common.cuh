@@ -84,6 +84,9 @@ __host__ __device__ constexpr uint32_t apply_warp_bytes(uint32_t R, uint32_t P) 
 __host__ __device__ constexpr uint32_t layer_groups(uint32_t L, uint32_t P) { return (L * P + 31) / 32; }
 // Edge ids of at most 32 bits: V^2 <= 2^32.
 inline bool small_ids(uint32_t V) { return V <= 65536; }
+// Batches of at most kSmallEdges edges are applied by one launch (k_small).
+constexpr uint32_t kSmallEdges = 4096;
+constexpr uint32_t kSmallThreads = 256;
 // Records per chunk of a batch of nrec records on V vertices: at most `most`,
 // and such that the `warps` of a layer group run out of chunks together (a
 // whole number of chunks each, as near as steps of 16 records and the
@@ -112,9 +115,14 @@ inline uint32_t hash_bits(uint32_t V) {
 // Threads of the recovery kernel and members per reduction work item.
 constexpr uint32_t kRecThreads = 256;
 constexpr uint32_t kRecSpan = 8;  // also the largest "small" component
+// Buckets of a sum the recovery reads at a time (two per lane), and the
+// counters of components that need more than one such pass.
+constexpr uint32_t kPrefix = 64;
+constexpr uint32_t kRetries = 3;
 // Members per CTA tile when reducing big components.
 constexpr uint32_t kRecTile = 64;
 constexpr uint32_t kWarpBuckets = 8;  // buckets per lane in the recovery: W <= 256
+static_assert(32 * kWarpBuckets <= kPrefix * (kRetries + 1), "a counter for every pass but the last");
 // Crossing candidates at or below which a recovery hook finishes in one CTA
 // (shared memory) instead of across the grid.
 constexpr uint32_t kSmallHook = 1024;
@@ -157,6 +165,7 @@ enum : uint32_t {
   GC_NSORTED = 26,       // length of forest_sorted
   GC_NFADD = 27,         // incremental mode: merge edges recorded in fadd since the last recovery
   GC_BATCH_MERGE = 28,   // the current batch merged two components (incremental mode)
+  GC_RETRY = 29,         // [kRetries] components that need another kPrefix buckets, per pass
   GC_SLOTS = 32
 };
 

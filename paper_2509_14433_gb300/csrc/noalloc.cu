@@ -145,10 +145,7 @@ extern "C" cupc_status cupc_update_sketch_static(void* sketch, uint32_t V, uint6
   if (cudaMemsetAsync(g.gc, 0, GC_SLOTS * sizeof(uint32_t), s) != cudaSuccess) return CUPC_ECUDA;
   if (cudaMemsetAsync(g.cnt, 0, (size_t)V * sizeof(uint32_t), s) != cudaSuccess) return CUPC_ECUDA;
   if (launch_keys(&g, s) != cudaSuccess) return CUPC_ECUDA;
-  if (n > 0) {
-    if (launch_validate(&g, edges, ops, n, s) != cudaSuccess) return CUPC_ECUDA;
-    if (launch_update_chunk(&g, edges, n, s) != cudaSuccess) return CUPC_ECUDA;
-  }
+  if (n > 0 && launch_update_chunk(&g, edges, n, s, ops) != cudaSuccess) return CUPC_ECUDA;
   if (status_out && cudaMemcpyAsync(status_out, g.gc + GC_ERR, sizeof(uint32_t), cudaMemcpyDefault, s) != cudaSuccess)
     return CUPC_ECUDA;
   return CUPC_OK;

@@ -403,6 +403,48 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply(
   bulk_wait_all();
 }
 
+// A small batch (n <= kSmallEdges edges, one chunk) in one launch: every CTA
+// validates the whole batch, so that none needs to wait for another, then
+// its warps XOR their records' buckets straight into HBM, P records (a lane
+// each) and one layer group at a time. What bounds it is latency: the launch,
+// the batch's loads and one pass per warp.
+template <bool kX32>
+__global__ void __launch_bounds__(kSmallThreads) k_small(ulonglong2* __restrict__ sketch,
+                                                         const uint64_t* __restrict__ keys,
+                                                         const uint32_t* __restrict__ edges,
+                                                         const int8_t* __restrict__ ops, uint32_t n, uint32_t* gc,
+                                                         uint32_t V, uint32_t L, uint32_t C, uint32_t D, uint32_t W,
+                                                         uint32_t P, uint32_t ell) {
+  const uint32_t lane = threadIdx.x & 31, gw = blockIdx.x * (kSmallThreads / 32) + (threadIdx.x >> 5);
+  const uint32_t groups = layer_groups(L, P), s = lane % P;
+  // this warp's records and lanes, in flight during the validation
+  const uint32_t i = gw / groups * P + s;  // record i: endpoint i & 1 of edge i / 2
+  const bool have = i < 2 * n;
+  const uint32_t w = have ? edges[i] : 0, other = have ? edges[i ^ 1] : 0;
+  const ApplyLane l = apply_lane(keys, sketch, V, L, C, D, W, P, ell, gw % groups);
+  bool drop = (ld_cg(&gc[GC_ERR]) & kErrInval) != 0, bad = false;
+#pragma unroll 4
+  for (uint32_t j = threadIdx.x; j < n; j += kSmallThreads) {
+    const uint32_t u = edges[2 * j], v = edges[2 * j + 1];
+    const int8_t op = ops[j];
+    bad |= (u >= V) | (v >= V) | (u == v) | ((op != 1) & (op != -1));
+  }
+  if (__syncthreads_or(bad)) {
+    if (threadIdx.x == 0) atomicOr(&gc[GC_ERR], kErrInval);
+    drop = true;
+  }
+  if (__syncthreads_or(drop)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) gc[GC_BATCHES] += 1;
+  const uint64_t x = record_id(make_record(w, other), V), c = mix64(x ^ l.kchk);  // of this lane's layer
+  for (uint32_t k = 0; k < P; k++) {
+    const uint32_t from = (lane & ~(P - 1)) + k;
+    const bool in = __shfl_sync(0xffffffffu, have, from);
+    const uint32_t wk = __shfl_sync(0xffffffffu, w, from);
+    const uint64_t xk = __shfl_sync(0xffffffffu, x, from), ck = __shfl_sync(0xffffffffu, c, from);
+    if (l.active && in) xor_bucket_atomic(l.base + (size_t)wk * W + lane_depth<kX32>(l, xk), make_ulonglong2(xk, ck));
+  }
+}
+
 // The dynamic shared-memory limit of k_apply is process-wide: only ever
 // raise it, so that a graph created later never shrinks it below what an
 // earlier graph's launches need.
@@ -458,6 +500,15 @@ cudaError_t configure_apply(cupc_graph* g) {
 cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, cudaStream_t s,
                                 const int8_t* validate_ops) {
   if (n == 0) return cudaSuccess;
+  if (validate_ops && n <= kSmallEdges) {
+    ProfScope ps(g, s, PC_APPLY, 1);
+    const uint32_t warps = (uint32_t)((2 * n + g->P - 1) / g->P) * layer_groups(g->L, g->P);
+    const uint32_t grid = (warps + kSmallThreads / 32 - 1) / (kSmallThreads / 32);
+    auto kern = small_ids(g->V) ? k_small<true> : k_small<false>;
+    kern<<<grid, kSmallThreads, 0, s>>>(g->sketch, g->keys, edges, validate_ops, (uint32_t)n, g->gc, g->V, g->L, g->C,
+                                        g->D, g->W, g->P, g->ell);
+    return cudaGetLastError();
+  }
   // the setting of this batch size's bucket, else the graph's default
   uint32_t ir = g->item_records, R = g->R;
   int smem = g->apply_smem, grid_max = g->apply_grid;
