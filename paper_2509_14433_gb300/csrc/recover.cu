@@ -9,12 +9,12 @@
 //   group       live vertices grouped by component label (count, segment
 //               offsets, scatter); round 0 skips it: every vertex is its own
 //               component
-//   reduce      components of at most kRecSpan members: a warp per span,
-//               lane l XORs buckets l + 32q of layer r of each member; bigger
-//               ones in CTA tiles sized to the grid, thread t XORs bucket t.
-//               A component inside one span or tile is sampled in place; one
-//               over several is XORed into its accumulator and sampled by the
-//               last span or tile to finish
+//   reduce      components of at most kRecSpan members: a warp per span;
+//               bigger ones in CTA tiles sized to the grid. A component inside
+//               one span or tile is sampled in place; one over several is
+//               XORed into its accumulator and sampled by the last span or
+//               tile to finish. Buckets are read kPrefix at a time, the later
+//               ones only where the earlier ones do not decide the sample
 //   sample      ZERO / GOOD(edge) / FAIL, first good bucket in index order;
 //               32 samples of a warp are booked at once
 //   hook        minimum spanning forest (weights = edge ids) of the candidate
@@ -146,6 +146,7 @@ __device__ __forceinline__ uint32_t warp_grab(uint32_t* ctr, uint32_t key, bool 
 }
 
 constexpr uint32_t kBigFlag = 0x80000000u;  // roff[K] flag: K's members are in permb
+constexpr uint32_t kParts = kRecThreads / kPrefix;  // members a CTA reads side by side
 constexpr uint32_t kTileSegs = 2 + kRecTile / (kRecSpan + 1);  // components meeting one tile
 
 
@@ -281,6 +282,39 @@ __device__ void small_hook(const RecArgs& a, uint32_t n, unsigned char* smem) {
   if (tid == 0) a.gc[GC_NFOREST] = s_f0 + s_nf;
 }
 
+// Add a warp's part of component K's sum (buckets base + lane + 32q) to
+// acc[K]; the last of the component's `nparts` parts gets the whole sum in
+// `acc` (true) and leaves acc[K] and the part count zero.
+__device__ __forceinline__ bool join_parts(const RecArgs& a, ulonglong2 (&acc)[2], uint32_t K, uint32_t base,
+                                           uint32_t W, uint32_t nparts) {
+  const uint32_t lane = threadIdx.x & 31;
+  ulonglong2* dst = a.acc + (size_t)K * W;
+#pragma unroll
+  for (uint32_t q = 0; q < 2; q++) {
+    const uint32_t b = base + lane + 32 * q;
+    if (b < W && (acc[q].x | acc[q].y)) {
+      atomicXor(&dst[b].x, acc[q].x);
+      atomicXor(&dst[b].y, acc[q].y);
+    }
+  }
+  __threadfence();
+  uint32_t prev = 0;
+  if (lane == 0) prev = atomicAdd(&a.pcount[K], 1u);
+  if (__shfl_sync(0xffffffffu, prev, 0) + 1 != nparts) return false;
+  __threadfence();
+#pragma unroll
+  for (uint32_t q = 0; q < 2; q++) {
+    const uint32_t b = base + lane + 32 * q;
+    acc[q] = make_ulonglong2(0, 0);
+    if (b < W) {
+      acc[q] = __ldcg(dst + b);
+      dst[b] = make_ulonglong2(0, 0);
+    }
+  }
+  if (lane == 0) a.pcount[K] = 0;
+  return true;
+}
+
 __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
   __shared__ int s_ok;
   __shared__ uint32_t t_w[kRecTile], t_k[kRecTile + 1];
@@ -341,6 +375,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
     gc[GC_ACTIVE_ODD] = 0;
     gc[GC_NMEMBERS] = 0;
     gc[GC_NBIG] = 0;
+    for (uint32_t p = 0; p < kRetries; p++) gc[GC_RETRY + p] = 0;
     gc[GC_RECOVERIES] += 1;
   }
   for (uint32_t r = gtid; r < a.L; r += gstride) {
@@ -498,49 +533,179 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
       nmem = ld_cg(&gc[GC_NMEMBERS]);
     }
 
-    // ---- reduce + sample, one warp per span of members (round 0: one
-    // vertex per span, every vertex is its own component). A component over
-    // several spans is XORed into acc[K]; the last span to finish samples it.
-    if (multi) {
-      // big components (more than kRecSpan members): each CTA takes one
-      // contiguous chunk of their members and walks it in tiles of up to
-      // kRecTile, thread t XORing bucket t of every member (8 rows in
-      // flight). A component's partial sum carries from one tile to the
-      // next, so that a CTA ends each component once: a component inside
-      // one chunk is sampled by one warp, one over several chunks is XORed
-      // into acc[K] once per chunk (the last chunk to finish samples it).
-      const uint32_t nbig = ld_cg(&gc[GC_NBIG]);
-      const uint32_t chunk = max(8u, (((nbig + nb - 1) / nb) + 7) & ~7u);
-      const uint32_t c0 = min(nbig, blockIdx.x * chunk), c1 = min(nbig, c0 + chunk);
+    // ---- reduce + sample. The sample is the first good bucket in index
+    // order, so the first kPrefix buckets of a sum nearly always decide it
+    // (they hold the deterministic bucket and 1.8 columns or more, each of
+    // which has a good bucket with probability 0.8): only they are read,
+    // XORed and tested, and the next kPrefix ones only for the components
+    // that need them. At V = 2^17 that is 64 of 239 buckets.
+    //
+    // Small components (and every vertex in round 0): one warp per span of
+    // members. A component over several spans is XORed into acc[K]; the last
+    // span to finish samples it.
+    uint32_t st_k = kNoneU32, st_res = 0, nst = 0;  // this lane's stashed sample
+    uint64_t st_e = 0;
+    auto stash = [&](uint32_t K, uint32_t res, uint64_t e) {
+      if (lane == nst) {
+        st_k = K;
+        st_res = res;
+        st_e = e;
+      }
+      if (++nst == 32) {  // book 32 samples at once, one per lane
+        book_samples(a, r, multi, st_k, st_res, st_e);
+        st_k = kNoneU32;
+        nst = 0;
+      }
+    };
+    const ulonglong2* layer = a.sketch + (size_t)r * V * W;
+    if (!multi) {
+      // two vertices at a time, the next two's rows in flight
+      const uint32_t step = 2 * nwarps;
+      ulonglong2 nx[2][2];
+      auto load = [&](uint32_t w0) {
+#pragma unroll
+        for (uint32_t k = 0; k < 2; k++)
+#pragma unroll
+          for (uint32_t q = 0; q < 2; q++) {
+            const uint32_t b = lane + 32 * q;
+            nx[k][q] = w0 + k < V && b < W ? __ldg(layer + (size_t)(w0 + k) * W + b) : make_ulonglong2(0, 0);
+          }
+      };
+      load(2 * gwarp);
+      for (uint32_t w0 = 2 * gwarp; w0 < V; w0 += step) {
+        ulonglong2 acc[2][2];
+#pragma unroll
+        for (uint32_t k = 0; k < 2; k++)
+#pragma unroll
+          for (uint32_t q = 0; q < 2; q++) acc[k][q] = nx[k][q];
+        load(w0 + step);
+#pragma unroll
+        for (uint32_t k = 0; k < 2; k++) {
+          if (w0 + k >= V) break;
+          uint64_t e = 0;
+          uint32_t res = warp_sample_prefix(acc[k], W, V, kchk, e);
+          for (uint32_t base = kPrefix; res == 2 && base < W; base += kPrefix) {
+            ulonglong2 more[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+            warp_xor_part(more, layer + (size_t)(w0 + k) * W, base, W, lane);
+            if (warp_find(more, base, W, V, kchk, e)) res = 1;
+          }
+          stash(w0 + k, res, e);
+        }
+      }
+    } else {
+      const uint32_t nspans = (nmem + kRecSpan - 1) / kRecSpan;
+      for (uint32_t sp = gwarp; sp < nspans; sp += nwarps) {
+        const uint32_t i0 = sp * kRecSpan, cnt = min(kRecSpan, nmem - i0);
+        uint32_t mw = 0, mk = kNoneU32;
+        if (lane < cnt) {
+          mw = ld_cg(&a.perm[i0 + lane]);
+          mk = ld_cg(&a.label[mw]);
+        }
+        if (lane < cnt) {  // every member's first buckets head for L2 while the first ones fold
+          const ulonglong2* row = layer + (size_t)mw * W;
+#pragma unroll
+          for (uint32_t b = 0; b < kPrefix; b += 8)
+            if (b < W) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + b));
+        }
+        uint32_t i = 0;
+        while (i < cnt) {
+          const uint32_t K = __shfl_sync(0xffffffffu, mk, i);
+          const uint32_t rest = ~(__ballot_sync(0xffffffffu, mk == K) >> i);
+          const uint32_t j = i + (rest ? (uint32_t)__ffs(rest) - 1 : 32 - i);
+          ulonglong2 acc[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+          for (uint32_t m0 = i; m0 < j; m0 += 4) {
+            ulonglong2 x[4][2];
+#pragma unroll
+            for (uint32_t k = 0; k < 4; k++) {
+              const uint32_t w = __shfl_sync(0xffffffffu, mw, m0 + k);
+#pragma unroll
+              for (uint32_t q = 0; q < 2; q++) {
+                const uint32_t b = lane + 32 * q;
+                x[k][q] = m0 + k < j && b < W ? __ldg(layer + (size_t)w * W + b) : make_ulonglong2(0, 0);
+              }
+            }
+#pragma unroll
+            for (uint32_t k = 0; k < 4; k++)
+#pragma unroll
+              for (uint32_t q = 0; q < 2; q++) {
+                acc[q].x ^= x[k][q].x;
+                acc[q].y ^= x[k][q].y;
+              }
+          }
+          const uint32_t s0 = ld_cg(&a.roff[K]), s1 = ld_cg(&a.rcnt[K]);
+          const uint32_t nsp = (s1 - 1) / kRecSpan - s0 / kRecSpan + 1;
+          if (nsp == 1 || join_parts(a, acc, K, 0, W, nsp)) {
+            uint64_t e = 0;
+            uint32_t res = warp_sample_prefix(acc, W, V, kchk, e);
+            for (uint32_t base = kPrefix; res == 2 && base < W; base += kPrefix) {
+              ulonglong2 more[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+              for (uint32_t m = s0; m < s1; m++)  // at most kRecSpan members
+                warp_xor_part(more, layer + (size_t)ld_cg(&a.perm[m]) * W, base, W, lane);
+              if (warp_find(more, base, W, V, kchk, e)) res = 1;
+            }
+            stash(K, res, e);
+          }
+          i = j;
+        }
+      }
+    }
+    if (nst) book_samples(a, r, multi, st_k, st_res, st_e);
+
+    // Big components (more than kRecSpan members): each CTA takes one
+    // contiguous chunk of their members and walks it in tiles of kRecTile;
+    // thread t XORs bucket base + t % kPrefix of every fourth member (8 rows in
+    // flight). A component's partial sums carry from one tile to the next, so
+    // that a CTA ends each component once: a component inside one chunk is
+    // sampled by one warp, one over several chunks is XORed into acc[K] once
+    // per chunk (the last chunk to finish samples it). Components whose first
+    // buckets hold no good one are marked (merged[K], unused until the
+    // relabel) and take another pass over the next kPrefix buckets.
+    const uint32_t nbig = multi ? ld_cg(&gc[GC_NBIG]) : 0;
+    const uint32_t chunk = max(8u, (((nbig + nb - 1) / nb) + 7) & ~7u);
+    const uint32_t c0 = min(nbig, blockIdx.x * chunk), c1 = min(nbig, c0 + chunk);
+    for (uint32_t base = 0;; base += kPrefix) {
+      const uint32_t part = tid / kPrefix, bk = base + tid % kPrefix;
       ulonglong2 acc1 = make_ulonglong2(0, 0);
       for (uint32_t m0 = c0; m0 < c1; m0 += kRecTile) {
         const uint32_t cnt = min(kRecTile, c1 - m0);
         if (tid < cnt) {
-          const uint32_t w = ld_cg(&a.permb[m0 + tid]);
-          t_w[tid] = w;
-          t_k[tid] = ld_cg(&a.label[w]);
+          const uint32_t w = ld_cg(&a.permb[m0 + tid]), K = ld_cg(&a.label[w]);
+          t_w[tid] = base == 0 || ld_cg(&a.merged[K]) ? w : kNoneU32;
+          t_k[tid] = K;
         } else if (tid == cnt) {  // the next tile's first label, or none at the chunk's end
           t_k[cnt] = m0 + cnt < c1 ? ld_cg(&a.label[ld_cg(&a.permb[m0 + cnt])]) : kNoneU32;
         }
         __syncthreads();
+        // members after which a component's part of this chunk ends
+        const uint32_t e0 = __ballot_sync(0xffffffffu, lane < cnt && t_k[lane + 1] != t_k[lane]);
+        const uint32_t e1 = __ballot_sync(0xffffffffu, lane + 32 < cnt && t_k[lane + 33] != t_k[lane + 32]);
         uint32_t nseg = 0;
-        for (uint32_t m = 0; m < cnt; m += 8) {
+        for (uint32_t m = 0; m < cnt; m += 32) {
+          const uint32_t ends = m ? e1 : e0;
           ulonglong2 x[8];
 #pragma unroll
           for (uint32_t k = 0; k < 8; k++) {
+            const uint32_t mm = m + kParts * k + part;
             x[k] = make_ulonglong2(0, 0);
-            if (tid < W && m + k < cnt) x[k] = __ldg(a.sketch + ((size_t)r * V + t_w[m + k]) * W + tid);
+            if (mm < cnt && bk < W && t_w[mm] != kNoneU32) x[k] = __ldg(layer + (size_t)t_w[mm] * W + bk);
           }
 #pragma unroll
           for (uint32_t k = 0; k < 8; k++) {
-            const uint32_t mm = m + k;
-            if (mm < cnt) {
+            const uint32_t four = ends >> (kParts * k) & ((1u << kParts) - 1);
+            if (four == 0) {
               acc1.x ^= x[k].x;
               acc1.y ^= x[k].y;
-              if (t_k[mm + 1] != t_k[mm]) {  // a component's part of this chunk ends here
+              continue;
+            }
+            for (uint32_t j = 0; j < kParts; j++) {
+              if (j == part) {
+                acc1.x ^= x[k].x;
+                acc1.y ^= x[k].y;
+              }
+              if (four >> j & 1) {
                 t_stage[nseg][tid] = acc1;
                 acc1 = make_ulonglong2(0, 0);
-                if (tid == 0) t_seg_k[nseg] = t_k[mm];
+                if (tid == 0) t_seg_k[nseg] = t_k[m + kParts * k + j];
                 nseg++;
               }
             }
@@ -549,134 +714,39 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
         __syncthreads();
         for (uint32_t sg = tid >> 5; sg < nseg; sg += wpb) {
           const uint32_t K = t_seg_k[sg];
+          if (base && !ld_cg(&a.merged[K])) continue;
           const uint32_t s0 = ld_cg(&a.roff[K]) & ~kBigFlag, s1 = ld_cg(&a.rcnt[K]);
           const uint32_t ntk = (s1 - 1) / chunk - s0 / chunk + 1;  // chunks it meets
-          ulonglong2 acc[kWarpBuckets];
+          ulonglong2 acc[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
 #pragma unroll
-          for (uint32_t q = 0; q < kWarpBuckets; q++) acc[q] = t_stage[sg][lane + 32 * q];
-          bool mine = true;
-          if (ntk > 1) {
-            ulonglong2* dst = a.acc + (size_t)K * W;
+          for (uint32_t p = 0; p < kParts; p++)
 #pragma unroll
-            for (uint32_t q = 0; q < kWarpBuckets; q++) {
-              const uint32_t b = lane + 32 * q;
-              if (b < W && (acc[q].x | acc[q].y)) {
-                atomicXor(&dst[b].x, acc[q].x);
-                atomicXor(&dst[b].y, acc[q].y);
-              }
+            for (uint32_t q = 0; q < 2; q++) {
+              const ulonglong2 v = t_stage[sg][kPrefix * p + lane + 32 * q];
+              acc[q].x ^= v.x;
+              acc[q].y ^= v.y;
             }
-            __threadfence();
-            uint32_t prev = 0;
-            if (lane == 0) prev = atomicAdd(&a.pcount[K], 1u);
-            mine = __shfl_sync(0xffffffffu, prev, 0) + 1 == ntk;
-            if (mine) {
-              __threadfence();
-#pragma unroll
-              for (uint32_t q = 0; q < kWarpBuckets; q++) {
-                const uint32_t b = lane + 32 * q;
-                acc[q] = make_ulonglong2(0, 0);
-                if (b < W) {
-                  acc[q] = __ldcg(dst + b);
-                  dst[b] = make_ulonglong2(0, 0);
-                }
-              }
-              if (lane == 0) a.pcount[K] = 0;
-            }
-          }
-          if (mine) {
+          if (ntk == 1 || join_parts(a, acc, K, base, W, ntk)) {
             uint64_t e = 0;
-            const uint32_t res = warp_sample(acc, W, V, kchk, e);
-            book_samples(a, r, multi, lane == 0 ? K : kNoneU32, res, e);
+            uint32_t res = 2;
+            if (base == 0)
+              res = warp_sample_prefix(acc, W, V, kchk, e);
+            else if (warp_find(acc, base, W, V, kchk, e))
+              res = 1;
+            const bool again = res == 2 && base + kPrefix < W;
+            if (lane == 0 && (again || base)) a.merged[K] = again ? 1 : 0;
+            if (again) {
+              if (lane == 0) atomicAdd(&gc[GC_RETRY + base / kPrefix], 1u);
+            } else {
+              book_samples(a, r, multi, lane == 0 ? K : kNoneU32, res, e);
+            }
           }
         }
         __syncthreads();
       }
+      CUPC_GRID_SYNC();
+      if (base + kPrefix >= W || ld_cg(&gc[GC_RETRY + base / kPrefix]) == 0) break;
     }
-
-    // small components (and every vertex in round 0): one warp per span
-    const uint32_t span = multi ? kRecSpan : 1u;
-    const uint32_t nspans = (nmem + span - 1) / span;
-    uint32_t st_k = kNoneU32, st_res = 0, nst = 0;  // this lane's stashed sample
-    uint64_t st_e = 0;
-    for (uint32_t sp = gwarp; sp < nspans; sp += nwarps) {
-      const uint32_t i0 = sp * span, cnt = min(span, nmem - i0);
-      if (!multi && sp + nwarps < nspans && lane * 8 < W)  // round 0: bring this warp's next row to L2
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.sketch + (size_t)(sp + nwarps) * W + lane * 8));
-      uint32_t mw = 0, mk = kNoneU32;
-      if (lane < cnt) {
-        mw = multi ? ld_cg(&a.perm[i0 + lane]) : i0 + lane;
-        mk = multi ? ld_cg(&a.label[mw]) : mw;
-      }
-      if (multi && lane < cnt) {  // every member's row heads for L2 while the first ones fold
-        const ulonglong2* row = a.sketch + ((size_t)r * V + mw) * W;
-        for (uint32_t b = 0; b < W; b += 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + b));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(row + W - 1));
-      }
-      uint32_t i = 0;
-      while (i < cnt) {
-        const uint32_t K = __shfl_sync(0xffffffffu, mk, i);
-        const uint32_t rest = ~(__ballot_sync(0xffffffffu, mk == K) >> i);
-        const uint32_t j = i + (rest ? (uint32_t)__ffs(rest) - 1 : 32 - i);
-        ulonglong2 acc[kWarpBuckets];
-#pragma unroll
-        for (uint32_t q = 0; q < kWarpBuckets; q++) acc[q] = make_ulonglong2(0, 0);
-        for (uint32_t m = i; m < j; m++) {
-          const uint32_t w = __shfl_sync(0xffffffffu, mw, m);
-          warp_xor_row(acc, a.sketch + ((size_t)r * V + w) * W, W, lane);
-        }
-        uint32_t nsp = 1;
-        if (multi) {
-          const uint32_t s0 = ld_cg(&a.roff[K]), s1 = ld_cg(&a.rcnt[K]);
-          nsp = (s1 - 1) / span - s0 / span + 1;
-        }
-        bool mine = true;
-        if (nsp > 1) {
-          ulonglong2* dst = a.acc + (size_t)K * W;
-#pragma unroll
-          for (uint32_t q = 0; q < kWarpBuckets; q++) {
-            const uint32_t b = lane + 32 * q;
-            if (b < W && (acc[q].x | acc[q].y)) {
-              atomicXor(&dst[b].x, acc[q].x);
-              atomicXor(&dst[b].y, acc[q].y);
-            }
-          }
-          __threadfence();
-          uint32_t prev = 0;
-          if (lane == 0) prev = atomicAdd(&a.pcount[K], 1u);
-          mine = __shfl_sync(0xffffffffu, prev, 0) + 1 == nsp;
-          if (mine) {  // the last span: every other span's XOR is in acc[K]
-            __threadfence();
-#pragma unroll
-            for (uint32_t q = 0; q < kWarpBuckets; q++) {
-              const uint32_t b = lane + 32 * q;
-              acc[q] = make_ulonglong2(0, 0);
-              if (b < W) {
-                acc[q] = __ldcg(dst + b);
-                dst[b] = make_ulonglong2(0, 0);
-              }
-            }
-            if (lane == 0) a.pcount[K] = 0;
-          }
-        }
-        if (mine) {
-          uint64_t e = 0;
-          const uint32_t res = warp_sample(acc, W, V, kchk, e);
-          if (lane == nst) {
-            st_k = K;
-            st_res = res;
-            st_e = e;
-          }
-          if (++nst == 32) {  // book 32 samples at once, one per lane
-            book_samples(a, r, multi, st_k, st_res, st_e);
-            st_k = kNoneU32;
-            nst = 0;
-          }
-        }
-        i = j;
-      }
-    }
-    if (nst) book_samples(a, r, multi, st_k, st_res, st_e);
-    CUPC_GRID_SYNC();
     if (gtid == 0) gc[GC_ROUNDS] = r + 1;
     if (ld_cg(&gc[GC_NZ]) == 0) {
       if (gtid == 0) gc[GC_COMPLETE] = 1;
@@ -794,6 +864,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
       gc[GC_ACTIVE] = 0;
       gc[GC_ACTIVE_ODD] = 0;
       gc[GC_NLIVE] = 0;
+      for (uint32_t p = 0; p < kRetries; p++) gc[GC_RETRY + p] = 0;
     }
     CUPC_GRID_SYNC();
     // new labels; the members of next round's live components are counted

@@ -73,6 +73,46 @@ __device__ __forceinline__ uint32_t warp_sample(const ulonglong2 (&acc)[NQ], uin
   return found ? 1u : 2u;
 }
 
+// Whether buckets base + lane + 32q, q < 2, of a warp's sum hold a good one;
+// `edge` is the first one's id, in index order.
+__device__ __forceinline__ bool warp_find(const ulonglong2 (&acc)[2], uint32_t base, uint32_t W, uint32_t V,
+                                          uint64_t kchk, uint64_t& edge) {
+  const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+  for (uint32_t q = 0; q < 2; q++) {
+    const bool good = base + lane + 32 * q < W && acc[q].x != 0 && mix64(acc[q].x ^ kchk) == acc[q].y &&
+                      edge_id_ordered(acc[q].x, V);
+    const uint32_t m = __ballot_sync(0xffffffffu, good);
+    if (m) {
+      edge = __shfl_sync(0xffffffffu, acc[q].x, __ffs(m) - 1);
+      return true;
+    }
+  }
+  return false;
+}
+
+// The sample as far as the first kPrefix buckets decide it: 0 ZERO, 1 GOOD,
+// 2 none of them is good.
+__device__ __forceinline__ uint32_t warp_sample_prefix(const ulonglong2 (&acc)[2], uint32_t W, uint32_t V,
+                                                       uint64_t kchk, uint64_t& edge) {
+  if (__shfl_sync(0xffffffffu, (acc[0].x | acc[0].y) == 0 ? 1u : 0u, 0)) return 0;
+  return warp_find(acc, 0, W, V, kchk, edge) ? 1u : 2u;
+}
+
+// Buckets base + lane + 32q, q < 2, of one member's row into acc.
+__device__ __forceinline__ void warp_xor_part(ulonglong2 (&acc)[2], const ulonglong2* __restrict__ row, uint32_t base,
+                                              uint32_t W, uint32_t lane) {
+#pragma unroll
+  for (uint32_t q = 0; q < 2; q++) {
+    const uint32_t b = base + lane + 32 * q;
+    if (b < W) {
+      const ulonglong2 x = __ldg(row + b);
+      acc[q].x ^= x.x;
+      acc[q].y ^= x.y;
+    }
+  }
+}
+
 // lane l XORs buckets l + 32q of one member's row into acc
 template <uint32_t NQ>
 __device__ __forceinline__ void warp_xor_row(ulonglong2 (&acc)[NQ], const ulonglong2* __restrict__ row, uint32_t W,
