@@ -85,7 +85,11 @@ __host__ __device__ constexpr uint32_t layer_groups(uint32_t L, uint32_t P) { re
 // Edge ids of at most 32 bits: V^2 <= 2^32.
 inline bool small_ids(uint32_t V) { return V <= 65536; }
 // Batches of at most kSmallEdges edges are applied by one launch (k_small).
-constexpr uint32_t kSmallEdges = 4096;
+// Against the grouped path, us, uniform batches: V = 1024, 4096 edges 13 (27),
+// 8192 edges 21 (29), 12000 edges 31 (31); V = 2^14, 8192 edges 56 (72), 12000
+// edges 84 (94); V = 2^17, 4096 edges 40 (46), 8192 edges 83 (86), 12000 edges
+// 120 (118); R-MAT on V = 2^17, 8192 edges 58 (72).
+constexpr uint32_t kSmallEdges = 8192;
 constexpr uint32_t kSmallThreads = 256;
 // Records per chunk of a batch of nrec records on V vertices: at most `most`,
 // and such that the `warps` of a layer group run out of chunks together (a
@@ -112,20 +116,22 @@ inline uint32_t hash_bits(uint32_t V) {
   if (lg < 1) lg = 1;
   return 65 - 2 * lg;
 }
-// Threads of the recovery kernel and members per reduction work item.
-constexpr uint32_t kRecThreads = 256;
-constexpr uint32_t kRecSpan = 8;  // also the largest "small" component
+// Threads of a CTA of the grid-wide recovery, one CTA per SM (two of half the
+// registers, with twice the warps for the reduce, spill: 221 against 186 us at
+// V = 2^14), and the members of a component over several runs that one warp
+// may read again alone.
+constexpr uint32_t kRecThreads = 512;
+constexpr uint32_t kRecSpan = 32;
 // Buckets of a sum the recovery reads at a time (two per lane), and the
 // counters of components that need more than one such pass.
 constexpr uint32_t kPrefix = 64;
 constexpr uint32_t kRetries = 3;
-// Members per CTA tile when reducing big components.
-constexpr uint32_t kRecTile = 64;
 constexpr uint32_t kWarpBuckets = 8;  // buckets per lane in the recovery: W <= 256
 static_assert(32 * kWarpBuckets <= kPrefix * (kRetries + 1), "a counter for every pass but the last");
 // Crossing candidates at or below which a recovery hook finishes in one CTA
 // (shared memory) instead of across the grid.
 constexpr uint32_t kSmallHook = 1024;
+constexpr uint32_t kHookBytes = 2 * kSmallHook * (8 + 4 + 4);  // its shared memory
 // One-cluster recovery (recover_small.cu): graphs of at most kClMaxV
 // vertices keep their per-vertex recovery state in one CTA's shared memory
 // (26 bytes a vertex); kClThreads threads per CTA. Measured on GB300 (one
@@ -155,7 +161,6 @@ enum : uint32_t {
   GC_BAR_COUNT = 13,
   GC_RECOVERIES = 15,
   GC_BATCHES = 16,   // update chunks applied
-  GC_NBIG = 17,      // members of big components this round
   GC_NLIVE = 19,     // live components of the next recovery round
   GC_REC_DIRTY = 20, // a recovery gave up at a barrier: its scratch may be non-zero
   GC_LABELS_VALID = 21,  // incremental mode: labels hold the current graph's components
@@ -246,9 +251,8 @@ struct cupc_graph {
   uint32_t* minv;    // V
   uint32_t* rcnt;    // V
   uint32_t* roff;    // V
-  uint32_t* perm;    // V: members of small components, grouped
-  uint32_t* permb;   // V: members of big components, grouped
-  uint32_t* pcount;  // V: spans of a component reduced so far
+  uint32_t* perm;    // V: members of live components, grouped
+  uint32_t* pcount;  // V: runs of a component reduced so far
   uint8_t* final_;   // V
   uint8_t* merged;   // V
   uint64_t* best;    // V

@@ -9,12 +9,12 @@
 //   group       live vertices grouped by component label (count, segment
 //               offsets, scatter); round 0 skips it: every vertex is its own
 //               component
-//   reduce      components of at most kRecSpan members: a warp per span;
-//               bigger ones in CTA tiles sized to the grid. A component inside
-//               one span or tile is sampled in place; one over several is
-//               XORed into its accumulator and sampled by the last span or
-//               tile to finish. Buckets are read kPrefix at a time, the later
-//               ones only where the earlier ones do not decide the sample
+//   reduce      an equal run of the live members per warp, lane l XORing
+//               buckets l and l + 32 of layer r of each. A component inside
+//               one run is sampled in place; one over several is XORed into
+//               its accumulator and sampled by the last run to finish.
+//               Buckets are read kPrefix at a time, the later ones only where
+//               the earlier ones do not decide the sample
 //   sample      ZERO / GOOD(edge) / FAIL, first good bucket in index order;
 //               32 samples of a warp are booked at once
 //   hook        minimum spanning forest (weights = edge ids) of the candidate
@@ -23,7 +23,8 @@
 //               still cross two trees, then one CTA finishes in shared
 //               memory; it adds exactly the edges Kruskal in ascending id
 //               order would
-//   relabel     every vertex takes the minimum vertex id of its component
+//   relabel     every vertex takes the root of its component (after the last
+//               round, its minimum vertex id)
 // A component whose merged sketch is ZERO has an empty cut; it is not sampled
 // again until it changes. With one live component left its merged sketch is
 // zero by linearity, so the round is logged without reading its layer.
@@ -31,6 +32,24 @@
 
 namespace cupc {
 
+
+// Release and acquire at device scope: what a CTA wrote before its arrival is
+// seen by every CTA after the barrier (__syncthreads orders the CTA's other
+// threads with the arriving one). Cheaper than the sequentially consistent
+// fences of __threadfence.
+__device__ __forceinline__ void red_release(uint32_t* p, uint32_t v) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
+}
 
 // Grid barrier for a cooperative launch: CTA thread 0 adds one to an arrival
 // counter that only grows during the launch (the host zeroes it before) and
@@ -44,11 +63,9 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* gc, uint32_t nblocks, uin
     epoch += 1;
     const uint32_t target = epoch * nblocks;
     int ok = 1;
-    __threadfence();
-    atomicAdd(&gc[GC_BAR_COUNT], 1u);
-    volatile uint32_t* cnt = gc + GC_BAR_COUNT;
+    red_release(&gc[GC_BAR_COUNT], 1u);
     uint64_t t0 = 0;
-    for (uint32_t spin = 0; *cnt < target; spin++) {
+    for (uint32_t spin = 0; ld_acquire(gc + GC_BAR_COUNT) < target; spin++) {
       if ((spin & 63) == 63) {
         const uint64_t t = global_timer_ns();
         if (t0 == 0) t0 = t;
@@ -64,22 +81,29 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* gc, uint32_t nblocks, uin
         }
       }
     }
-    __threadfence();
     *s_ok = ok;
   }
   __syncthreads();
   return *s_ok != 0;
 }
 
-// Root of x in the hook forest; points x straight at it. Other threads may
-// rewrite parent[] concurrently, but only ever to an ancestor, so every value
-// read is an ancestor and the walk ends at the same root.
+// Root of x in the hook forest; points x straight at it and, on the way, every
+// second node at its grandparent: the walks of one phase start together, so
+// they shorten each other's paths. Other threads may rewrite parent[]
+// concurrently, but only ever to an ancestor, so every value read is an
+// ancestor and the walk ends at the same root.
 __device__ __forceinline__ uint32_t find_root(uint32_t* parent, uint32_t x, uint32_t V) {
   uint32_t r = x;
   for (uint32_t k = 0; k < V; k++) {
     const uint32_t p = ld_cg(&parent[r]);
     if (p == r) break;
-    r = p;
+    const uint32_t g = ld_cg(&parent[p]);
+    if (g == p) {
+      r = p;
+      break;
+    }
+    parent[r] = g;
+    r = g;
   }
   if (r != x && ld_cg(&parent[x]) != r) parent[x] = r;
   return r;
@@ -145,11 +169,6 @@ __device__ __forceinline__ uint32_t warp_grab(uint32_t* ctr, uint32_t key, bool 
   return pos;
 }
 
-constexpr uint32_t kBigFlag = 0x80000000u;  // roff[K] flag: K's members are in permb
-constexpr uint32_t kParts = kRecThreads / kPrefix;  // members a CTA reads side by side
-constexpr uint32_t kTileSegs = 2 + kRecTile / (kRecSpan + 1);  // components meeting one tile
-
-
 // Root in a shared-memory forest with path halving; concurrent halving only
 // ever points a node at an ancestor.
 __device__ __forceinline__ uint32_t s_find(volatile uint32_t* par, uint32_t x) {
@@ -170,8 +189,8 @@ __device__ __forceinline__ uint32_t s_find(volatile uint32_t* par, uint32_t x) {
 // edge hook once, the larger under the smaller), over local node ids, with
 // __syncthreads between steps and pointer jumping after each hook step.
 // Publishes parent[] of the roots that hooked and appends the forest edges.
-// smem: 32 KB.
-__device__ void small_hook(const RecArgs& a, uint32_t n, unsigned char* smem) {
+// smem: kHookBytes.
+static __device__ __noinline__ void small_hook(const RecArgs& a, uint32_t n, unsigned char* smem) {
   constexpr uint32_t kPer = kSmallHook / kRecThreads;  // candidates per thread
   constexpr uint32_t kNodeBits = 11;                    // nodes < 2 * kSmallHook
   static_assert(2 * kSmallHook <= (1u << kNodeBits), "node ids fit the key");
@@ -276,7 +295,10 @@ __device__ void small_hook(const RecArgs& a, uint32_t n, unsigned char* smem) {
     const uint32_t lab = s_lab[x];
     if (lab == kNoneU32) continue;  // an id whose claim lost
     const uint32_t rt = s_find(s_par, x);
-    if (rt != x) a.parent[lab] = s_lab[rt];
+    if (rt != x) {
+      a.parent[lab] = s_lab[rt];
+      a.final_[s_lab[rt]] = 0;  // it absorbed another component: live
+    }
     a.pcount[lab] = 0;
   }
   if (tid == 0) a.gc[GC_NFOREST] = s_f0 + s_nf;
@@ -297,11 +319,11 @@ __device__ __forceinline__ bool join_parts(const RecArgs& a, ulonglong2 (&acc)[2
       atomicXor(&dst[b].y, acc[q].y);
     }
   }
-  __threadfence();
+  __syncwarp();
   uint32_t prev = 0;
-  if (lane == 0) prev = atomicAdd(&a.pcount[K], 1u);
+  if (lane == 0) prev = atom_add_acq_rel(&a.pcount[K], 1u);
+  __syncwarp();
   if (__shfl_sync(0xffffffffu, prev, 0) + 1 != nparts) return false;
-  __threadfence();
 #pragma unroll
   for (uint32_t q = 0; q < 2; q++) {
     const uint32_t b = base + lane + 32 * q;
@@ -315,15 +337,54 @@ __device__ __forceinline__ bool join_parts(const RecArgs& a, ulonglong2 (&acc)[2
   return true;
 }
 
-__global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
+// Buckets base + lane + 32q of the four members that lanes m0 .. m0+3 hold in
+// mw (kNoneU32: none), all in flight at once.
+__device__ __forceinline__ void load_rows(ulonglong2 (&x)[4][2], const ulonglong2* __restrict__ layer, uint32_t mw,
+                                          uint32_t m0, uint32_t base, uint32_t W) {
+#pragma unroll
+  for (uint32_t k = 0; k < 4; k++) {
+    const uint32_t w = __shfl_sync(0xffffffffu, mw, m0 + k);
+#pragma unroll
+    for (uint32_t q = 0; q < 2; q++) {
+      const uint32_t b = base + (threadIdx.x & 31) + 32 * q;
+      x[k][q] = w != kNoneU32 && b < W ? __ldg(layer + (size_t)w * W + b) : make_ulonglong2(0, 0);
+    }
+  }
+}
+
+// The first good one of buckets [base, base + kPrefix) of the sum of the
+// members perm[s0..s1), by one warp: its edge id, or kNone. Seldom called, so
+// not inlined: its registers would add to the caller's.
+static __device__ __noinline__ uint64_t read_on(const ulonglong2* __restrict__ layer, const uint32_t* perm, uint32_t s0,
+                                                uint32_t s1, uint32_t base, uint32_t W, uint32_t V, uint64_t kchk) {
+  const uint32_t lane = threadIdx.x & 31;
+  ulonglong2 sum[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+  for (uint32_t t0 = s0; t0 < s1; t0 += 32) {
+    const uint32_t mw = t0 + lane < s1 ? ld_cg(&perm[t0 + lane]) : kNoneU32;
+    for (uint32_t m0 = 0; m0 < min(32u, s1 - t0); m0 += 4) {
+      ulonglong2 x[4][2];
+      load_rows(x, layer, mw, m0, base, W);
+#pragma unroll
+      for (uint32_t k = 0; k < 4; k++)
+#pragma unroll
+        for (uint32_t q = 0; q < 2; q++) {
+          sum[q].x ^= x[k][q].x;
+          sum[q].y ^= x[k][q].y;
+        }
+    }
+  }
+  uint64_t e = 0;
+  return warp_find(sum, base, W, V, kchk, e) ? e : kNone;
+}
+
+__global__ void __launch_bounds__(kRecThreads, 1) k_recover(RecArgs a) {
   __shared__ int s_ok;
-  __shared__ uint32_t t_w[kRecTile], t_k[kRecTile + 1];
-  static_assert(kRecTile <= kRecThreads, "one member id per thread");
-  static_assert(sizeof(ulonglong2) * kTileSegs * kRecThreads >= 2 * kSmallHook * (8 + 4 + 4),
-                "small_hook lives in t_stage");
+  extern __shared__ __align__(16) unsigned char s_dyn[];  // small_hook; a reduce's partial sums
+  constexpr uint32_t kSlots = 2 * (kRecThreads / 32);  // a warp's first and last component
+  __shared__ uint32_t s_pk[kSlots];
   static_assert(kSmallHook % kRecThreads == 0, "small_hook: whole candidates per thread");
-  __shared__ ulonglong2 t_stage[kTileSegs][kRecThreads];
-  __shared__ uint32_t t_seg_k[kTileSegs];
+  static_assert(kSlots == 32 && kSlots * kPrefix * sizeof(ulonglong2) <= kHookBytes, "partial sums: one per lane id");
+  ulonglong2* s_part = reinterpret_cast<ulonglong2*>(s_dyn);  // [kSlots][kPrefix]
   const uint32_t V = a.V, W = a.W, nb = gridDim.x, tid = threadIdx.x, lane = tid & 31;
   const uint32_t gtid = blockIdx.x * blockDim.x + tid, gstride = gridDim.x * blockDim.x;
   const uint32_t wpb = blockDim.x >> 5, gwarp = blockIdx.x * wpb + (tid >> 5), nwarps = gridDim.x * wpb;
@@ -374,7 +435,6 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
     gc[GC_ACTIVE] = 0;
     gc[GC_ACTIVE_ODD] = 0;
     gc[GC_NMEMBERS] = 0;
-    gc[GC_NBIG] = 0;
     for (uint32_t p = 0; p < kRetries; p++) gc[GC_RETRY + p] = 0;
     gc[GC_RECOVERIES] += 1;
   }
@@ -494,31 +554,21 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
       for (uint32_t base = blockIdx.x * blockDim.x; base < V; base += gstride) {
         const uint32_t K = base + tid;
         const uint32_t c = K < V ? ld_cg(&a.rcnt[K]) : 0;
-        const bool big = c > kRecSpan;
-        uint32_t is = big ? 0 : c, ib = big ? c : 0;
+        uint32_t inc = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t ys = __shfl_up_sync(0xffffffffu, is, o), yb = __shfl_up_sync(0xffffffffu, ib, o);
-          if (lane >= (uint32_t)o) {
-            is += ys;
-            ib += yb;
-          }
+          const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= (uint32_t)o) inc += y;
         }
-        const uint32_t ts = __shfl_sync(0xffffffffu, is, 31), tb = __shfl_sync(0xffffffffu, ib, 31);
-        uint32_t bs = 0, bb = 0;
-        if (lane == 31 && ts) bs = atomicAdd(&gc[GC_NMEMBERS], ts);
-        if (lane == 31 && tb) bb = atomicAdd(&gc[GC_NBIG], tb);
-        bs = __shfl_sync(0xffffffffu, bs, 31);
-        bb = __shfl_sync(0xffffffffu, bb, 31);
+        uint32_t at = 0;
+        if (lane == 31 && inc) at = atomicAdd(&gc[GC_NMEMBERS], inc);
+        at = __shfl_sync(0xffffffffu, at, 31) + inc - c;
         if (c) {
-          const uint32_t at = big ? bb + ib - c : bs + is - c;
-          a.roff[K] = big ? (at | kBigFlag) : at;
+          a.roff[K] = at;
           a.rcnt[K] = at;  // scatter cursor, then the segment end
         }
         if (K < V) {
           a.parent[K] = K;
-          a.minv[K] = kNoneU32;
-          a.merged[K] = 0;
         }
       }
       CUPC_GRID_SYNC();
@@ -527,7 +577,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
         const uint32_t K = w < V ? ld_cg(&a.label[w]) : 0;
         const bool live = w < V && !ld_cg(&a.final_[K]);
         const uint32_t pos = warp_grab(a.rcnt, K, live);
-        if (live) ((ld_cg(&a.roff[K]) & kBigFlag) ? a.permb : a.perm)[pos] = w;
+        if (live) a.perm[pos] = w;
       }
       CUPC_GRID_SYNC();
       nmem = ld_cg(&gc[GC_NMEMBERS]);
@@ -540,47 +590,154 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
     // XORed and tested, and the next kPrefix ones only for the components
     // that need them. At V = 2^17 that is 64 of 239 buckets.
     //
-    // Small components (and every vertex in round 0): one warp per span of
-    // members. A component over several spans is XORed into acc[K]; the last
-    // span to finish samples it.
+    // Round 0: a warp per vertex. Later rounds: every warp takes an equal run
+    // of the member list; a component inside one run is sampled by its warp,
+    // the parts of one over several runs are summed by the CTA, and one over
+    // several CTAs is XORed into acc[K] and sampled by the last CTA to finish
+    // (XORs of every warp of the device into one giant component's acc[K]
+    // would queue: 42 us against 8 at V = 2^14).
     uint32_t st_k = kNoneU32, st_res = 0, nst = 0;  // this lane's stashed sample
     uint64_t st_e = 0;
+    auto book_stash = [&]() {  // up to 32 samples at once, one per lane
+      if (nst) book_samples(a, r, multi, st_k, st_res, st_e);
+      st_k = kNoneU32;
+      nst = 0;
+    };
     auto stash = [&](uint32_t K, uint32_t res, uint64_t e) {
       if (lane == nst) {
         st_k = K;
         st_res = res;
         st_e = e;
       }
-      if (++nst == 32) {  // book 32 samples at once, one per lane
-        book_samples(a, r, multi, st_k, st_res, st_e);
-        st_k = kNoneU32;
-        nst = 0;
-      }
+      if (++nst == 32) book_stash();
     };
     const ulonglong2* layer = a.sketch + (size_t)r * V * W;
-    if (!multi) {
-      // two vertices at a time, the next two's rows in flight
-      const uint32_t step = 2 * nwarps;
-      ulonglong2 nx[2][2];
-      auto load = [&](uint32_t w0) {
+    const uint32_t run = (nmem + nwarps - 1) / nwarps, p0 = gwarp * run, p1 = min(nmem, p0 + run);
+    // The sum of component K over [s0, s1) of the list, or this CTA's part of
+    // it (nparts > 1), is complete: sample it.
+    auto complete = [&](uint32_t base, uint32_t K, ulonglong2(&acc)[2], uint32_t s0, uint32_t s1, uint32_t nparts,
+                        bool here) {
+      if (nparts > 1 && !join_parts(a, acc, K, base, W, nparts)) return;
+      uint64_t e = 0;
+      uint32_t res = 2;
+      if (base == 0)
+        res = warp_sample_prefix(acc, W, V, kchk, e);
+      else if (warp_find(acc, base, W, V, kchk, e))
+        res = 1;
+      // this warp's own, or a short one: reads on at once
+      here = here || s1 - s0 <= kRecSpan;
+      for (uint32_t b = base + kPrefix; here && res == 2 && b < W; b += kPrefix) {
+        const uint64_t more = read_on(layer, a.perm, s0, s1, b, W, V, kchk);
+        if (more != kNone) {
+          e = more;
+          res = 1;
+        }
+      }
+      const bool again = !here && res == 2 && base + kPrefix < W;
+      if (lane == 0 && (again || base)) a.merged[K] = again ? 1 : 0;
+      if (!again)
+        stash(K, res, e);
+      else if (lane == 0)
+        atomicAdd(&gc[GC_RETRY + base / kPrefix], 1u);
+    };
+    auto reduce_run = [&](uint32_t base) {
+      const uint32_t wid = tid >> 5;
+      if (lane < 2) s_pk[2 * wid + lane] = kNoneU32;
+      __syncwarp();
+      ulonglong2 acc[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+      uint32_t K = kNoneU32;  // the component being summed
+      auto finish = [&]() {
+        if (K == kNoneU32 || (base && !ld_cg(&a.merged[K]))) return;
+        const uint32_t s0 = ld_cg(&a.roff[K]), s1 = ld_cg(&a.rcnt[K]);
+        if (s0 >= p0 && s1 <= p1) {
+          complete(base, K, acc, s0, s1, 1, true);
+        } else {  // it goes on in a neighbouring run
+          const uint32_t slot = 2 * wid + (s0 < p0 ? 0 : 1);
+          if (lane == 0) s_pk[slot] = K;
 #pragma unroll
-        for (uint32_t k = 0; k < 2; k++)
+          for (uint32_t q = 0; q < 2; q++) s_part[slot * kPrefix + lane + 32 * q] = acc[q];
+        }
+      };
+      for (uint32_t t0 = p0; t0 < p1; t0 += 32) {
+        const uint32_t cnt = min(32u, p1 - t0);
+        uint32_t mw = kNoneU32, mk = kNoneU32;
+        if (lane < cnt) {
+          mw = ld_cg(&a.perm[t0 + lane]);
+          mk = ld_cg(&a.label[mw]);
+          if (base && !ld_cg(&a.merged[mk])) mw = kNoneU32;  // not read again
+        }
+        uint32_t before = __shfl_up_sync(0xffffffffu, mk, 1);
+        if (lane == 0) before = K;
+        const uint32_t heads = __ballot_sync(0xffffffffu, lane < cnt && mk != before);
+        if (mw != kNoneU32) {  // the members' rows head for L2
+#pragma unroll
+          for (uint32_t b = 0; b < kPrefix; b += 8)
+            if (base + b < W) asm volatile("prefetch.global.L2 [%0];" ::"l"(layer + (size_t)mw * W + base + b));
+        }
+        for (uint32_t m0 = 0; m0 < cnt; m0 += 4) {
+          ulonglong2 x[4][2];
+          load_rows(x, layer, mw, m0, base, W);
+          const uint32_t h = heads >> m0 & 0xFu;
+          for (uint32_t m = 0; m < 4;) {  // the parts of components among the four
+            if (h >> m & 1) {
+              finish();
+              K = __shfl_sync(0xffffffffu, mk, m0 + m);
+              acc[0] = acc[1] = make_ulonglong2(0, 0);
+            }
+            const uint32_t more = h & (~1u << m), end = more ? (uint32_t)__ffs((int)more) - 1 : 4u;
+#pragma unroll
+            for (uint32_t k = 0; k < 4; k++)
+              if (k >= m && k < end) {
+#pragma unroll
+                for (uint32_t q = 0; q < 2; q++) {
+                  acc[q].x ^= x[k][q].x;
+                  acc[q].y ^= x[k][q].y;
+                }
+              }
+            m = end;
+          }
+        }
+      }
+      finish();
+      __syncthreads();
+      // the CTA's parts of one component, together
+      const uint32_t pk = s_pk[lane], crun = run * wpb;
+      for (uint32_t slot = wid; slot < kSlots; slot += wpb) {
+        const uint32_t C = __shfl_sync(0xffffffffu, pk, slot);
+        uint32_t parts = __ballot_sync(0xffffffffu, pk == C);
+        if (C == kNoneU32 || (uint32_t)__ffs((int)parts) - 1 != slot) continue;
+        ulonglong2 sum[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+        for (; parts; parts &= parts - 1) {
+          const ulonglong2* v = s_part + (__ffs((int)parts) - 1) * kPrefix + lane;
+#pragma unroll
+          for (uint32_t q = 0; q < 2; q++) {
+            sum[q].x ^= v[32 * q].x;
+            sum[q].y ^= v[32 * q].y;
+          }
+        }
+        const uint32_t s0 = ld_cg(&a.roff[C]), s1 = ld_cg(&a.rcnt[C]);
+        complete(base, C, sum, s0, s1, (s1 - 1) / crun - s0 / crun + 1, false);
+      }
+      __syncthreads();
+    };
+    if (!multi) {
+      // four vertices' rows in flight; the next four's head for L2
+      constexpr uint32_t kAtOnce = 4;
+      const uint32_t step = kAtOnce * nwarps;
+      for (uint32_t w0 = kAtOnce * gwarp; w0 < V; w0 += step) {
+        const uint32_t ahead = w0 + step + lane / 8;  // lane: 128 bytes of a row
+        if (ahead < V && lane % 8 * 8 < W)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(layer + (size_t)ahead * W + lane % 8 * 8));
+        ulonglong2 acc[kAtOnce][2];
+#pragma unroll
+        for (uint32_t k = 0; k < kAtOnce; k++)
 #pragma unroll
           for (uint32_t q = 0; q < 2; q++) {
             const uint32_t b = lane + 32 * q;
-            nx[k][q] = w0 + k < V && b < W ? __ldg(layer + (size_t)(w0 + k) * W + b) : make_ulonglong2(0, 0);
+            acc[k][q] = w0 + k < V && b < W ? __ldg(layer + (size_t)(w0 + k) * W + b) : make_ulonglong2(0, 0);
           }
-      };
-      load(2 * gwarp);
-      for (uint32_t w0 = 2 * gwarp; w0 < V; w0 += step) {
-        ulonglong2 acc[2][2];
 #pragma unroll
-        for (uint32_t k = 0; k < 2; k++)
-#pragma unroll
-          for (uint32_t q = 0; q < 2; q++) acc[k][q] = nx[k][q];
-        load(w0 + step);
-#pragma unroll
-        for (uint32_t k = 0; k < 2; k++) {
+        for (uint32_t k = 0; k < kAtOnce; k++) {
           if (w0 + k >= V) break;
           uint64_t e = 0;
           uint32_t res = warp_sample_prefix(acc[k], W, V, kchk, e);
@@ -593,161 +750,22 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
         }
       }
     } else {
-      const uint32_t nspans = (nmem + kRecSpan - 1) / kRecSpan;
-      for (uint32_t sp = gwarp; sp < nspans; sp += nwarps) {
-        const uint32_t i0 = sp * kRecSpan, cnt = min(kRecSpan, nmem - i0);
-        uint32_t mw = 0, mk = kNoneU32;
-        if (lane < cnt) {
-          mw = ld_cg(&a.perm[i0 + lane]);
-          mk = ld_cg(&a.label[mw]);
-        }
-        if (lane < cnt) {  // every member's first buckets head for L2 while the first ones fold
-          const ulonglong2* row = layer + (size_t)mw * W;
-#pragma unroll
-          for (uint32_t b = 0; b < kPrefix; b += 8)
-            if (b < W) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + b));
-        }
-        uint32_t i = 0;
-        while (i < cnt) {
-          const uint32_t K = __shfl_sync(0xffffffffu, mk, i);
-          const uint32_t rest = ~(__ballot_sync(0xffffffffu, mk == K) >> i);
-          const uint32_t j = i + (rest ? (uint32_t)__ffs(rest) - 1 : 32 - i);
-          ulonglong2 acc[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
-          for (uint32_t m0 = i; m0 < j; m0 += 4) {
-            ulonglong2 x[4][2];
-#pragma unroll
-            for (uint32_t k = 0; k < 4; k++) {
-              const uint32_t w = __shfl_sync(0xffffffffu, mw, m0 + k);
-#pragma unroll
-              for (uint32_t q = 0; q < 2; q++) {
-                const uint32_t b = lane + 32 * q;
-                x[k][q] = m0 + k < j && b < W ? __ldg(layer + (size_t)w * W + b) : make_ulonglong2(0, 0);
-              }
-            }
-#pragma unroll
-            for (uint32_t k = 0; k < 4; k++)
-#pragma unroll
-              for (uint32_t q = 0; q < 2; q++) {
-                acc[q].x ^= x[k][q].x;
-                acc[q].y ^= x[k][q].y;
-              }
-          }
-          const uint32_t s0 = ld_cg(&a.roff[K]), s1 = ld_cg(&a.rcnt[K]);
-          const uint32_t nsp = (s1 - 1) / kRecSpan - s0 / kRecSpan + 1;
-          if (nsp == 1 || join_parts(a, acc, K, 0, W, nsp)) {
-            uint64_t e = 0;
-            uint32_t res = warp_sample_prefix(acc, W, V, kchk, e);
-            for (uint32_t base = kPrefix; res == 2 && base < W; base += kPrefix) {
-              ulonglong2 more[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
-              for (uint32_t m = s0; m < s1; m++)  // at most kRecSpan members
-                warp_xor_part(more, layer + (size_t)ld_cg(&a.perm[m]) * W, base, W, lane);
-              if (warp_find(more, base, W, V, kchk, e)) res = 1;
-            }
-            stash(K, res, e);
-          }
-          i = j;
-        }
-      }
+      reduce_run(0);
     }
-    if (nst) book_samples(a, r, multi, st_k, st_res, st_e);
-
-    // Big components (more than kRecSpan members): each CTA takes one
-    // contiguous chunk of their members and walks it in tiles of kRecTile;
-    // thread t XORs bucket base + t % kPrefix of every fourth member (8 rows in
-    // flight). A component's partial sums carry from one tile to the next, so
-    // that a CTA ends each component once: a component inside one chunk is
-    // sampled by one warp, one over several chunks is XORed into acc[K] once
-    // per chunk (the last chunk to finish samples it). Components whose first
-    // buckets hold no good one are marked (merged[K], unused until the
-    // relabel) and take another pass over the next kPrefix buckets.
-    const uint32_t nbig = multi ? ld_cg(&gc[GC_NBIG]) : 0;
-    const uint32_t chunk = max(8u, (((nbig + nb - 1) / nb) + 7) & ~7u);
-    const uint32_t c0 = min(nbig, blockIdx.x * chunk), c1 = min(nbig, c0 + chunk);
-    for (uint32_t base = 0;; base += kPrefix) {
-      const uint32_t part = tid / kPrefix, bk = base + tid % kPrefix;
-      ulonglong2 acc1 = make_ulonglong2(0, 0);
-      for (uint32_t m0 = c0; m0 < c1; m0 += kRecTile) {
-        const uint32_t cnt = min(kRecTile, c1 - m0);
-        if (tid < cnt) {
-          const uint32_t w = ld_cg(&a.permb[m0 + tid]), K = ld_cg(&a.label[w]);
-          t_w[tid] = base == 0 || ld_cg(&a.merged[K]) ? w : kNoneU32;
-          t_k[tid] = K;
-        } else if (tid == cnt) {  // the next tile's first label, or none at the chunk's end
-          t_k[cnt] = m0 + cnt < c1 ? ld_cg(&a.label[ld_cg(&a.permb[m0 + cnt])]) : kNoneU32;
-        }
-        __syncthreads();
-        // members after which a component's part of this chunk ends
-        const uint32_t e0 = __ballot_sync(0xffffffffu, lane < cnt && t_k[lane + 1] != t_k[lane]);
-        const uint32_t e1 = __ballot_sync(0xffffffffu, lane + 32 < cnt && t_k[lane + 33] != t_k[lane + 32]);
-        uint32_t nseg = 0;
-        for (uint32_t m = 0; m < cnt; m += 32) {
-          const uint32_t ends = m ? e1 : e0;
-          ulonglong2 x[8];
-#pragma unroll
-          for (uint32_t k = 0; k < 8; k++) {
-            const uint32_t mm = m + kParts * k + part;
-            x[k] = make_ulonglong2(0, 0);
-            if (mm < cnt && bk < W && t_w[mm] != kNoneU32) x[k] = __ldg(layer + (size_t)t_w[mm] * W + bk);
-          }
-#pragma unroll
-          for (uint32_t k = 0; k < 8; k++) {
-            const uint32_t four = ends >> (kParts * k) & ((1u << kParts) - 1);
-            if (four == 0) {
-              acc1.x ^= x[k].x;
-              acc1.y ^= x[k].y;
-              continue;
-            }
-            for (uint32_t j = 0; j < kParts; j++) {
-              if (j == part) {
-                acc1.x ^= x[k].x;
-                acc1.y ^= x[k].y;
-              }
-              if (four >> j & 1) {
-                t_stage[nseg][tid] = acc1;
-                acc1 = make_ulonglong2(0, 0);
-                if (tid == 0) t_seg_k[nseg] = t_k[m + kParts * k + j];
-                nseg++;
-              }
-            }
-          }
-        }
-        __syncthreads();
-        for (uint32_t sg = tid >> 5; sg < nseg; sg += wpb) {
-          const uint32_t K = t_seg_k[sg];
-          if (base && !ld_cg(&a.merged[K])) continue;
-          const uint32_t s0 = ld_cg(&a.roff[K]) & ~kBigFlag, s1 = ld_cg(&a.rcnt[K]);
-          const uint32_t ntk = (s1 - 1) / chunk - s0 / chunk + 1;  // chunks it meets
-          ulonglong2 acc[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
-#pragma unroll
-          for (uint32_t p = 0; p < kParts; p++)
-#pragma unroll
-            for (uint32_t q = 0; q < 2; q++) {
-              const ulonglong2 v = t_stage[sg][kPrefix * p + lane + 32 * q];
-              acc[q].x ^= v.x;
-              acc[q].y ^= v.y;
-            }
-          if (ntk == 1 || join_parts(a, acc, K, base, W, ntk)) {
-            uint64_t e = 0;
-            uint32_t res = 2;
-            if (base == 0)
-              res = warp_sample_prefix(acc, W, V, kchk, e);
-            else if (warp_find(acc, base, W, V, kchk, e))
-              res = 1;
-            const bool again = res == 2 && base + kPrefix < W;
-            if (lane == 0 && (again || base)) a.merged[K] = again ? 1 : 0;
-            if (again) {
-              if (lane == 0) atomicAdd(&gc[GC_RETRY + base / kPrefix], 1u);
-            } else {
-              book_samples(a, r, multi, lane == 0 ? K : kNoneU32, res, e);
-            }
-          }
-        }
-        __syncthreads();
-      }
+    book_stash();
+    CUPC_GRID_SYNC();
+    // Components of more than kRecSpan members that no warp holds alone and whose buckets
+    // so far hold no good one are marked (merged[K], unused until the
+    // relabel): another pass over the next kPrefix buckets.
+    for (uint32_t base = kPrefix; multi && base < W && ld_cg(&gc[GC_RETRY + base / kPrefix - 1]); base += kPrefix) {
+      reduce_run(base);
+      book_stash();
       CUPC_GRID_SYNC();
-      if (base + kPrefix >= W || ld_cg(&gc[GC_RETRY + base / kPrefix]) == 0) break;
     }
-    if (gtid == 0) gc[GC_ROUNDS] = r + 1;
+    if (gtid == 0) {
+      gc[GC_ROUNDS] = r + 1;
+      gc[GC_NLIVE] = 0;  // every CTA has read it
+    }
     if (ld_cg(&gc[GC_NZ]) == 0) {
       if (gtid == 0) gc[GC_COMPLETE] = 1;
       break;
@@ -771,6 +789,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
         uint64_t e = 0;
         uint32_t ra = 0, rb = 0;
         if (K < V) {
+          if (iter == 0) a.rcnt[K] = 0;  // the relabel counts again
           const ulonglong2 c = __ldcg(&a.cand[K]);
           if (c.x != kNone) {
             e = c.x;
@@ -796,7 +815,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
       const uint32_t nact = ld_cg(&gc[act]);
       if (nact == 0) break;
       if (nact <= kSmallHook) {  // finish in one CTA behind a single barrier
-        if (blockIdx.x == 0) small_hook(a, nact, reinterpret_cast<unsigned char*>(&t_stage[0][0]));
+        if (blockIdx.x == 0) small_hook(a, nact, s_dyn);
         CUPC_GRID_SYNC();
         break;
       }
@@ -822,6 +841,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
           at = __shfl_sync(0xffffffffu, at, 0);
           if (hook) {
             a.parent[x] = o;
+            a.final_[o] = 0;  // it absorbs another component: live
             a.forest[at + __popc(m & ((1u << lane) - 1))] = e;
           }
         }
@@ -830,57 +850,26 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
       CUPC_GRID_SYNC();
     }
 
-    // ---- relabel to the minimum vertex id of each component; clear the
-    // round's scratch
-    for (uint32_t base = gwarp * 32; base < V; base += nwarps * 32) {
-      const uint32_t w = base + lane;
-      bool lab = false;
-      uint32_t root = 0;
-      if (w < V) {
-        a.rcnt[w] = 0;
-        a.cand[w] = make_ulonglong2(kNone, 0);
-        a.best0[w] = kNone;
-        a.best1[w] = kNone;
-        if (ld_cg(&a.label[w]) == w) {
-          lab = true;
-          root = find_root(a.parent, w, V);
-        }
-      }
-      const uint32_t act = __ballot_sync(0xffffffffu, lab);
-      if (lab) {  // the lanes of one root: min id and "merged" with one write each
-        const uint32_t peers = __match_any_sync(act, root);
-        const uint32_t mn = __reduce_min_sync(peers, w);
-        const bool mg = __any_sync(peers, root != w);
-        if (lane == (uint32_t)__ffs(peers) - 1) {
-          atomicMin(&a.minv[root], mn);
-          if (mg) a.merged[root] = 1;
-        }
-      }
-    }
+    // ---- relabel to the root of each component; the members of next round's
+    // live components are counted here; clear the round's scratch
     if (gtid == 0) {
       gc[GC_NZ] = 0;
       gc[GC_NMEMBERS] = 0;
-      gc[GC_NBIG] = 0;
       gc[GC_ACTIVE] = 0;
       gc[GC_ACTIVE_ODD] = 0;
-      gc[GC_NLIVE] = 0;
       for (uint32_t p = 0; p < kRetries; p++) gc[GC_RETRY + p] = 0;
     }
-    CUPC_GRID_SYNC();
-    // new labels; the members of next round's live components are counted
-    // here (a merged component is live; an unmerged one keeps its flag)
     for (uint32_t base = gwarp * 32; base < V; base += nwarps * 32) {
       const uint32_t w = base + lane;
       uint32_t nl = 0;
       bool live = false;
       if (w < V) {
-        const uint32_t K = ld_cg(&a.label[w]);
-        const uint32_t root = find_root(a.parent, K, V);
-        nl = ld_cg(&a.minv[root]);
-        const bool mg = ld_cg(&a.merged[root]) != 0;
+        a.cand[w] = make_ulonglong2(kNone, 0);
+        a.best0[w] = kNone;
+        a.best1[w] = kNone;
+        nl = find_root(a.parent, ld_cg(&a.label[w]), V);
         a.label[w] = nl;
-        if (w == root && mg) a.final_[nl] = 0;
-        live = mg || !ld_cg(&a.final_[root]);
+        live = !ld_cg(&a.final_[nl]);
       }
       // the member that took position 0 of its component counts the component
       const uint32_t m_first = __ballot_sync(0xffffffffu, warp_grab(a.rcnt, nl, live) == 0 && live);
@@ -888,6 +877,18 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_recover(RecArgs a) {
     }
     CUPC_GRID_SYNC();
   }
+  // ---- labels: the rounds need one id per component (its root), the result
+  // is the minimum vertex id
+  for (uint32_t base = gwarp * 32; base < V; base += nwarps * 32) {
+    const uint32_t w = base + lane;
+    const uint32_t act = __ballot_sync(0xffffffffu, w < V);
+    if (w < V) {  // the first of the lanes of one component has their minimum
+      const uint32_t K = ld_cg(&a.label[w]), peers = __match_any_sync(act, K);
+      if (lane == (uint32_t)__ffs(peers) - 1 && w < ld_cg(&a.minv[K])) atomicMin(&a.minv[K], w);
+    }
+  }
+  CUPC_GRID_SYNC();
+  for (uint32_t w = gtid; w < V; w += gstride) a.label[w] = ld_cg(&a.minv[ld_cg(&a.label[w])]);
   // a complete recovery starts an incremental epoch
   if (a.inc && gtid == 0) gc[GC_LABELS_VALID] = ld_cg(&gc[GC_COMPLETE]);
 #undef CUPC_GRID_SYNC
@@ -906,12 +907,14 @@ __global__ void k_wait_selftest(uint32_t* gc, uint32_t absent, uint64_t limit_ns
 
 cudaError_t setup_recover(cupc_graph* g) {
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_recover, kRecThreads, 0);
+  cudaError_t e = cudaFuncSetAttribute(k_recover, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHookBytes);
+  if (e != cudaSuccess) return e;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_recover, kRecThreads, kHookBytes);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   // about four vertices per warp in round 0 (every vertex samples its own
   // sketch); fewer CTAs for small V keep the grid barriers cheap
-  uint32_t want = (g->V + 31) / 32;
+  uint32_t want = (g->V + kRecThreads / 8 - 1) / (kRecThreads / 8);
   if (want < 16) want = 16;
   uint32_t cap = (uint32_t)(per_sm * g->sms);
   g->rec_grid = (int)(want < cap ? want : cap);
@@ -933,7 +936,6 @@ cudaError_t launch_recover(cupc_graph* g, cudaStream_t s, bool force) {
   a.rcnt = g->rcnt;
   a.roff = g->roff;
   a.perm = g->perm;
-  a.permb = g->permb;
   a.pcount = g->pcount;
   a.final_ = g->final_;
   a.merged = g->merged;
@@ -965,7 +967,8 @@ cudaError_t launch_recover(cupc_graph* g, cudaStream_t s, bool force) {
   if (e != cudaSuccess) return e;
   ProfScope ps(g, s, PC_RECOVER, 1);
   void* args[] = {&a};
-  return cudaLaunchCooperativeKernel((const void*)k_recover, dim3(g->rec_grid), dim3(kRecThreads), args, 0, s);
+  return cudaLaunchCooperativeKernel((const void*)k_recover, dim3(g->rec_grid), dim3(kRecThreads), args, kHookBytes,
+                                     s);
 }
 
 }  // namespace cupc

@@ -11,7 +11,7 @@ struct RecArgs {
   const ulonglong2* sketch;
   const uint64_t* keys;
   uint32_t V, L, C, D, W;
-  uint32_t *label, *parent, *minv, *rcnt, *roff, *perm, *permb, *pcount;
+  uint32_t *label, *parent, *minv, *rcnt, *roff, *perm, *pcount;
   uint8_t *final_, *merged;
   uint64_t *best0, *best1, *forest, *log_ids;
   ulonglong2* cand;  // {edge, label[u] << 32 | label[v]} of a component's candidate
