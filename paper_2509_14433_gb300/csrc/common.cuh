@@ -158,18 +158,20 @@ enum : uint32_t {
   GC_COMPLETE = 10,
   GC_LOGLEN = 11,
   GC_ACTIVE_ODD = 12,  // MSF: same count for odd hook steps
-  GC_BAR_COUNT = 13,
+  GC_BAR_COUNT = 13,   // arrivals at the grid barriers of a recovery
+  GC_BAR_DONE = 14,    // CTAs that left the recovery
   GC_RECOVERIES = 15,
   GC_BATCHES = 16,   // update chunks applied
+  GC_SORT_DONE = 17, // CTAs of the forest sort that are done
   GC_NLIVE = 19,     // live components of the next recovery round
   GC_REC_DIRTY = 20, // a recovery gave up at a barrier: its scratch may be non-zero
   GC_LABELS_VALID = 21,  // incremental mode: labels hold the current graph's components
   GC_FOREST_SORTED = 22, // forest_sorted holds the last recovery's forest
-  GC_BATCH_DEL = 24,     // the current batch deletes an edge (incremental mode)
+  GC_BATCH_DEL = 24,     // number of the last batch that deletes an edge (incremental mode)
   GC_WARM = 25,          // incremental mode: forest edges were deleted: warm-start recovery
   GC_NSORTED = 26,       // length of forest_sorted
   GC_NFADD = 27,         // incremental mode: merge edges recorded in fadd since the last recovery
-  GC_BATCH_MERGE = 28,   // the current batch merged two components (incremental mode)
+  GC_BATCH_MERGE = 28,   // number of the last batch that merged two components (incremental mode)
   GC_RETRY = 29,         // [kRetries] components that need another kPrefix buckets, per pass
   GC_SLOTS = 32
 };
@@ -179,6 +181,11 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
   z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
   return z ^ (z >> 31);
+}
+
+// Key j of a graph: K(j) = mix(seed + phi * (j + 1)).
+__host__ __device__ __forceinline__ uint64_t graph_key(uint64_t seed, uint32_t j) {
+  return mix64(seed + 0x9E3779B97F4A7C15ull * (uint64_t)(j + 1));
 }
 
 __device__ __forceinline__ uint64_t global_timer_ns() {
@@ -209,6 +216,7 @@ struct cupc_graph {
   bool dirty;
   bool inc;           // incremental labels (cupc_set_incremental)
   bool forest_stale;  // an update since the last full recovery
+  uint32_t inc_batch; // incremental mode: batches so far
   bool sort_pending;  // incremental mode: a recovery ran; the next update sorts its forest first
   bool imported;      // words from cupc_import_sketches since the last reset:
                       // the XOR of all vertex sketches need not be zero
@@ -335,5 +343,6 @@ cudaError_t setup_recover(cupc_graph* g);
 cudaError_t launch_recover(cupc_graph* g, cudaStream_t s, bool force = false);
 cudaError_t launch_query(cupc_graph* g, const uint32_t* pairs, size_t m, uint8_t* out, cudaStream_t s);
 cudaError_t launch_forest_sort(cupc_graph* g, cudaStream_t s);
+cudaError_t launch_copy_forest(cupc_graph* g, uint64_t* out, size_t cap, cudaStream_t s);
 cudaError_t launch_incremental(cupc_graph* g, const uint32_t* edges, const int8_t* ops, size_t n, cudaStream_t s);
 }  // namespace cupc
