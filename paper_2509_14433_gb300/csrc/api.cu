@@ -416,13 +416,17 @@ cupc_status cupc_spanning_forest(cupc_graph* g, uint64_t* edge_ids_out, size_t c
   }
   g->forest_stale = false;
   CUPC_TRY(launch_forest_sort(g, s));
+  // into device memory the ids go at once, behind one synchronisation; into
+  // host memory once their number is known
+  const bool direct = edge_ids_out && (uintptr_t)edge_ids_out % 8 == 0 && is_device_ptr(edge_ids_out);
+  if (direct) CUPC_TRY(launch_copy_forest(g, edge_ids_out, cap, s));
   uint32_t h[GC_SLOTS];
   CUPC_TRY(cudaMemcpyAsync(h, g->gc, sizeof(h), cudaMemcpyDeviceToHost, s));
   CUPC_TRY(cudaStreamSynchronize(s));
   *n_out = h[GC_NFOREST];
   if (h[GC_ERR] & (kErrTimeout | kErrInval)) return cupc_sync(g, stream);
   if (cap < h[GC_NFOREST] || (!edge_ids_out && h[GC_NFOREST])) return CUPC_EINVAL;
-  if (h[GC_NFOREST]) {
+  if (h[GC_NFOREST] && !direct) {
     CUPC_TRY(cudaMemcpyAsync(edge_ids_out, g->forest_sorted, h[GC_NFOREST] * sizeof(uint64_t), cudaMemcpyDefault,
                              s));
     CUPC_TRY(cudaStreamSynchronize(s));

@@ -52,8 +52,7 @@ __device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
 }
 
 // Grid barrier for a cooperative launch: CTA thread 0 adds one to an arrival
-// counter that only grows during the launch (the host zeroes it before) and
-// waits until all CTAs of this barrier have arrived. The wait is bounded:
+// counter that only grows during the launch (zero before it) and waits until all CTAs of this barrier have arrived. The wait is bounded:
 // after kWaitLimitNs it records kErrTimeout and returns false in every
 // thread of the CTA, which must then return.
 __device__ __forceinline__ bool grid_barrier(uint32_t* gc, uint32_t nblocks, uint32_t& epoch, int* s_ok,
@@ -65,7 +64,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* gc, uint32_t nblocks, uin
     int ok = 1;
     red_release(&gc[GC_BAR_COUNT], 1u);
     uint64_t t0 = 0;
-    for (uint32_t spin = 0; ld_acquire(gc + GC_BAR_COUNT) < target; spin++) {
+    for (uint32_t spin = 0; ld_acquire(&gc[GC_BAR_COUNT]) < target; spin++) {
       if ((spin & 63) == 63) {
         const uint64_t t = global_timer_ns();
         if (t0 == 0) t0 = t;
@@ -377,7 +376,8 @@ static __device__ __noinline__ uint64_t read_on(const ulonglong2* __restrict__ l
   return warp_find(sum, base, W, V, kchk, e) ? e : kNone;
 }
 
-__global__ void __launch_bounds__(kRecThreads, 1) k_recover(RecArgs a) {
+// The recovery; false if there was nothing to do (no barrier was met).
+__device__ __forceinline__ bool recover_body(const RecArgs& a) {
   __shared__ int s_ok;
   extern __shared__ __align__(16) unsigned char s_dyn[];  // small_hook; a reduce's partial sums
   constexpr uint32_t kSlots = 2 * (kRecThreads / 32);  // a warp's first and last component
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kRecThreads, 1) k_recover(RecArgs a) {
   uint32_t* gc = a.gc;
   uint32_t epoch = 0;
 #define CUPC_GRID_SYNC() \
-  if (!grid_barrier(gc, nb, epoch, &s_ok)) return
+  if (!grid_barrier(gc, nb, epoch, &s_ok)) return true
 
   // incremental mode: the updates since the last recovery kept the labels
   // exact (see k_incr), so there is nothing to recover; or they deleted
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kRecThreads, 1) k_recover(RecArgs a) {
   // the components are unions of the fragments of the remaining forest, and
   // Boruvka starts from those (warm start) instead of from single vertices
   const bool valid = ld_cg(&gc[GC_LABELS_VALID]) != 0, warm = !a.force && valid && ld_cg(&gc[GC_WARM]) != 0;
-  if (!a.force && valid && !warm) return;
+  if (!a.force && valid && !warm) return false;
   const uint32_t nsorted = warm ? min(ld_cg(&gc[GC_NSORTED]), V) : 0;
   const uint32_t nadd = warm ? min(ld_cg(&gc[GC_NFADD]), V) : 0;
   // after a recovery that gave up at a barrier, the reduce accumulators and
@@ -892,6 +892,18 @@ __global__ void __launch_bounds__(kRecThreads, 1) k_recover(RecArgs a) {
   // a complete recovery starts an incremental epoch
   if (a.inc && gtid == 0) gc[GC_LABELS_VALID] = ld_cg(&gc[GC_COMPLETE]);
 #undef CUPC_GRID_SYNC
+  return true;
+}
+
+// The last CTA to leave zeroes the barrier's counters for the next launch,
+// also when the CTAs gave up at a barrier.
+__global__ void __launch_bounds__(kRecThreads, 1) k_recover(RecArgs a) {
+  if (!recover_body(a)) return;
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(&a.gc[GC_BAR_DONE], 1u) == gridDim.x - 1) {
+    a.gc[GC_BAR_COUNT] = 0;
+    a.gc[GC_BAR_DONE] = 0;
+  }
 }
 
 // Self-test of the bounded waits: every CTA but `absent` meets at two grid
@@ -963,8 +975,6 @@ cudaError_t launch_recover(cupc_graph* g, cudaStream_t s, bool force) {
     ProfScope ps(g, s, PC_RECOVER, 1);
     return launch_recover_cluster(g, a, s);
   }
-  cudaError_t e = cudaMemsetAsync(g->gc + GC_BAR_COUNT, 0, sizeof(uint32_t), s);
-  if (e != cudaSuccess) return e;
   ProfScope ps(g, s, PC_RECOVER, 1);
   void* args[] = {&a};
   return cudaLaunchCooperativeKernel((const void*)k_recover, dim3(g->rec_grid), dim3(kRecThreads), args, kHookBytes,
@@ -1024,73 +1034,131 @@ cudaError_t launch_query(cupc_graph* g, const uint32_t* pairs, size_t m, uint8_t
   return cudaGetLastError();
 }
 
-// ---- forest ids in ascending order: bitonic sort of 1024-id chunks in
-// shared memory, then each id's final rank = its rank in its chunk + its
-// lower bound in every other chunk (ids are distinct).
+// ---- forest ids in ascending order: bitonic sort of 1024-id chunks, one id
+// a thread (partners within a warp exchange by shuffles, farther ones through
+// shared memory), then each id's final rank = its rank in its chunk + its
+// lower bound in every other chunk (ids are distinct), a CTA taking the other
+// chunks through shared memory one after the other, the next one in flight.
+// V = 2^14 on GB300: 6 + 9 us; 14 + 29 us with the exchanges all in shared
+// memory and the searches in global memory.
 constexpr uint32_t kSortChunk = 1024;
 
-__global__ void __launch_bounds__(512) k_sort_chunks(uint64_t* ids, const uint32_t* gc) {
-  __shared__ uint64_t s[kSortChunk];
-  if (ld_cg(&gc[GC_FOREST_SORTED])) return;  // done since the last recovery
-  const uint32_t n = ld_cg(&gc[GC_NFOREST]);
-  const uint32_t base = blockIdx.x * kSortChunk;
-  if (base >= n) return;
-  for (uint32_t i = threadIdx.x; i < kSortChunk; i += blockDim.x) s[i] = base + i < n ? ids[base + i] : kNone;
-  __syncthreads();
+__device__ __forceinline__ void sort_chunk(uint64_t* ids, uint32_t n, uint64_t (&s)[2][kSortChunk]) {
+  const uint32_t tid = threadIdx.x, at = blockIdx.x * kSortChunk + tid;
+  if (blockIdx.x * kSortChunk >= n) return;
+  uint64_t v = at < n ? ids[at] : kNone;
+  uint32_t buf = 0;
+#pragma unroll
   for (uint32_t k = 2; k <= kSortChunk; k <<= 1) {
+#pragma unroll
     for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-      for (uint32_t i = threadIdx.x; i < kSortChunk; i += blockDim.x) {
-        uint32_t p = i ^ j;
-        if (p > i) {
-          bool up = (i & k) == 0;
-          uint64_t x = s[i], y = s[p];
-          if ((x > y) == up) {
-            s[i] = y;
-            s[p] = x;
-          }
-        }
+      uint64_t y;
+      if (j >= 32) {
+        s[buf][tid] = v;
+        __syncthreads();
+        y = s[buf][tid ^ j];
+        buf ^= 1;  // the next exchange's writes do not meet this one's reads
+      } else {
+        y = __shfl_xor_sync(0xffffffffu, v, j);
       }
-      __syncthreads();
+      v = ((tid & j) == 0) == ((tid & k) == 0) ? min(v, y) : max(v, y);
     }
   }
-  for (uint32_t i = threadIdx.x; i < kSortChunk && base + i < n; i += blockDim.x) ids[base + i] = s[i];
+  if (at < n) ids[at] = v;
 }
 
-__global__ void k_merge_rank(const uint64_t* __restrict__ ids, uint64_t* __restrict__ out, const uint32_t* gc) {
+__device__ __forceinline__ void merge_rank(const uint64_t* ids, uint64_t* out, uint32_t n,
+                                           uint64_t (&s)[2][kSortChunk], uint32_t* gc) {
+  const uint32_t nch = (n + kSortChunk - 1) / kSortChunk, tid = threadIdx.x, at = blockIdx.x * kSortChunk + tid;
+  if (blockIdx.x < nch) {
+    const uint64_t x = at < n ? ld_cg(&ids[at]) : kNone;
+    uint32_t rank = tid;
+    auto load = [&](uint32_t k) {  // chunk blockIdx.x + k, cyclically
+      const uint32_t c = blockIdx.x + k < nch ? blockIdx.x + k : blockIdx.x + k - nch;
+      const uint32_t i = c * kSortChunk + tid;
+      return k < nch && i < n ? ld_cg(&ids[i]) : kNone;
+    };
+    uint64_t next = load(1);
+    for (uint32_t k = 1; k < nch; k++) {
+      uint64_t* c = s[k & 1];
+      c[tid] = next;
+      next = load(k + 1);
+      __syncthreads();
+      uint32_t lo = 0;  // ids of the chunk below x; the ids past its end are kNone
+#pragma unroll
+      for (uint32_t step = kSortChunk / 2; step > 0; step >>= 1)
+        if (c[lo + step - 1] < x) lo += step;
+      if (c[lo] < x) lo++;
+      rank += lo;
+    }
+    if (at < n) out[rank] = x;
+  }
+  __syncthreads();
+  if (tid == 0 && atomicAdd(&gc[GC_SORT_DONE], 1u) == gridDim.x - 1) {  // every CTA has read the flag above
+    gc[GC_SORT_DONE] = 0;
+    gc[GC_NSORTED] = n;
+    gc[GC_FOREST_SORTED] = 1;
+  }
+}
+
+__global__ void __launch_bounds__(kSortChunk) k_sort_chunks(uint64_t* ids, const uint32_t* gc) {
+  __shared__ uint64_t s[2][kSortChunk];
+  if (ld_cg(&gc[GC_FOREST_SORTED])) return;  // done since the last recovery
+  sort_chunk(ids, ld_cg(&gc[GC_NFOREST]), s);
+}
+
+__global__ void __launch_bounds__(kSortChunk) k_merge_rank(const uint64_t* ids, uint64_t* out, uint32_t* gc) {
+  __shared__ uint64_t s[2][kSortChunk];
+  if (ld_cg(&gc[GC_FOREST_SORTED])) return;
+  merge_rank(ids, out, ld_cg(&gc[GC_NFOREST]), s, gc);
+}
+
+// Both steps in one launch, where the chunks are the CTAs of one cluster
+// (whose barrier orders the chunks' stores before the other CTAs' loads): in
+// incremental mode most launches find the forest sorted, and cost only that.
+__global__ void __launch_bounds__(kSortChunk) k_sort_cluster(uint64_t* ids, uint64_t* out, uint32_t* gc) {
+  __shared__ uint64_t s[2][kSortChunk];
   if (ld_cg(&gc[GC_FOREST_SORTED])) return;
   const uint32_t n = ld_cg(&gc[GC_NFOREST]);
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint64_t x = ids[i];
-  const uint32_t mine = i / kSortChunk, nch = (n + kSortChunk - 1) / kSortChunk;
-  uint32_t rank = i - mine * kSortChunk;
-  for (uint32_t c = 0; c < nch; c++) {
-    if (c == mine) continue;
-    uint32_t lo = c * kSortChunk, hi = min(n, lo + kSortChunk);
-    while (lo < hi) {  // first position with ids[pos] >= x
-      uint32_t mid = (lo + hi) >> 1;
-      if (ids[mid] < x)
-        lo = mid + 1;
-      else
-        hi = mid;
-    }
-    rank += lo - c * kSortChunk;
-  }
-  out[rank] = x;
-}
-
-__global__ void k_mark_sorted(uint32_t* gc) {
-  if (gc[GC_FOREST_SORTED]) return;
-  gc[GC_NSORTED] = gc[GC_NFOREST];
-  gc[GC_FOREST_SORTED] = 1;
+  sort_chunk(ids, n, s);
+  cluster_sync_all();
+  merge_rank(ids, out, n, s, gc);
 }
 
 cudaError_t launch_forest_sort(cupc_graph* g, cudaStream_t s) {
-  uint32_t nch = (g->V + kSortChunk - 1) / kSortChunk;
-  ProfScope ps(g, s, PC_SORT, 3);
-  k_sort_chunks<<<nch, 512, 0, s>>>(g->forest, g->gc);
-  k_merge_rank<<<(g->V + 255) / 256, 256, 0, s>>>(g->forest, g->forest_sorted, g->gc);
-  k_mark_sorted<<<1, 1, 0, s>>>(g->gc);
+  const uint32_t nch = (g->V + kSortChunk - 1) / kSortChunk;
+  if (nch <= 8) {  // the largest portable cluster
+    ProfScope ps(g, s, PC_SORT, 1);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = nch;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nch);
+    cfg.blockDim = dim3(kSortChunk);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_sort_cluster, g->forest, g->forest_sorted, g->gc);
+  }
+  ProfScope ps(g, s, PC_SORT, 2);
+  k_sort_chunks<<<nch, kSortChunk, 0, s>>>(g->forest, g->gc);
+  k_merge_rank<<<nch, kSortChunk, 0, s>>>(g->forest, g->forest_sorted, g->gc);
+  return cudaGetLastError();
+}
+
+// The sorted forest into the caller's device memory, unless it does not fit
+// or an error is pending (the caller then reports that and copies nothing).
+__global__ void k_copy_forest(const uint64_t* __restrict__ ids, uint64_t* __restrict__ out, size_t cap,
+                              const uint32_t* gc) {
+  const uint32_t n = ld_cg(&gc[GC_NFOREST]);
+  if (n > cap || (ld_cg(&gc[GC_ERR]) & (kErrTimeout | kErrInval))) return;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = ids[i];
+}
+
+cudaError_t launch_copy_forest(cupc_graph* g, uint64_t* out, size_t cap, cudaStream_t s) {
+  k_copy_forest<<<(int)std::min<size_t>((g->V + 255) / 256, (size_t)g->sms * 4), 256, 0, s>>>(g->forest_sorted, out, cap,
+                                                                                               g->gc);
   return cudaGetLastError();
 }
 

@@ -30,6 +30,12 @@ struct RecArgs {
   uint32_t* gc;
 };
 
+// Barrier of a thread-block cluster; arrive has release and wait acquire
+// semantics at cluster scope.
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // u < v for an edge id x = u*V + v (32-bit division when x fits 32 bits).
 __device__ __forceinline__ bool edge_id_ordered(uint64_t x, uint32_t V) {
   if ((x >> 32) == 0) {

@@ -40,10 +40,6 @@ namespace {
 // Members of a warp's range whose rows are prefetched ahead of the fold.
 constexpr uint32_t kClAhead = 4;
 
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // Rows of two members at once, all loads issued before the first XOR.
 template <uint32_t NQ>
 __device__ __forceinline__ void warp_xor_rows2(ulonglong2 (&acc)[NQ], const ulonglong2* __restrict__ r0,
