@@ -20,9 +20,8 @@
 namespace cupc {
 
 __global__ void k_keys(uint64_t seed, uint64_t* keys, uint32_t n) {
-  const uint64_t phi = 0x9E3779B97F4A7C15ull;
   for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-    keys[j] = mix64(seed + phi * (uint64_t)(j + 1));
+    keys[j] = graph_key(seed, j);
 }
 
 cudaError_t launch_keys(cupc_graph* g, cudaStream_t s) {
@@ -156,7 +155,7 @@ __global__ void __launch_bounds__(1024) k_scatter_priv(const uint32_t* __restric
 // and sets GC_WARM: the next recovery starts from the fragments of the
 // remaining forest. In a batch that both merges and deletes, an edge the
 // batch inserts (a merge) and then deletes is found by a second lookup pass
-// (k_incr_dead) once all of the batch's merges are recorded.
+// (k_incr_rest) once all of the batch's merges are recorded.
 __device__ __forceinline__ uint32_t inc_find(uint32_t* par, uint32_t x, uint32_t V) {
   for (uint32_t k = 0; k < V; k++) {  // a path is shorter than V
     const uint32_t y = ld_cg(&par[x]);
@@ -183,6 +182,7 @@ struct IncArgs {
   unsigned long long* ftab;
   uint32_t* ftab_pos;
   uint32_t ftab_bits, V;
+  uint32_t batch;  // number of this batch: what gc[GC_BATCH_DEL] and gc[GC_BATCH_MERGE] hold if it deletes, merges
   uint32_t* gc;
 };
 
@@ -258,24 +258,32 @@ __global__ void k_incr(const uint32_t* __restrict__ edges, const int8_t* __restr
     }
   }
   if (__any_sync(0xffffffffu, cut) && (threadIdx.x & 31) == 0) gc[GC_LABELS_VALID] = 0;
-  if (__any_sync(0xffffffffu, del) && (threadIdx.x & 31) == 0) gc[GC_BATCH_DEL] = 1;
-  if (__any_sync(0xffffffffu, merged) && (threadIdx.x & 31) == 0) gc[GC_BATCH_MERGE] = 1;
+  if (__any_sync(0xffffffffu, del) && (threadIdx.x & 31) == 0) gc[GC_BATCH_DEL] = a.batch;
+  if (__any_sync(0xffffffffu, merged) && (threadIdx.x & 31) == 0) gc[GC_BATCH_MERGE] = a.batch;
   if (__any_sync(0xffffffffu, warm) && (threadIdx.x & 31) == 0) gc[GC_WARM] = 1;
 }
 
+// The rest of a batch, once k_incr has recorded all of its merges.
+//
+// Labels after the merges: every vertex takes its label's root. Merges are
+// exact whatever else the batch did: a delete can only split components, and
+// one that removed a forest edge has set GC_WARM, so the next query recovers
+// from the fragments of the remaining forest.
+//
 // A batch that both merges and deletes: k_incr looked each delete up in the
 // merge edges recorded before the batch, so an edge this batch inserted (and
 // recorded as a merge) and then deleted again, in stream order, is looked up
-// again here, once every merge of the batch is in the table.
-__global__ void k_incr_dead(const uint32_t* __restrict__ edges, const int8_t* __restrict__ ops, size_t n,
-                            IncArgs a) {
+// again here.
+__global__ void k_incr_rest(const uint32_t* __restrict__ edges, const int8_t* __restrict__ ops, size_t n,
+                            uint32_t* label, IncArgs a) {
   uint32_t* gc = a.gc;
-  if ((ld_cg(&gc[GC_ERR]) & kErrInval) || !ld_cg(&gc[GC_LABELS_VALID]) || !ld_cg(&gc[GC_BATCH_MERGE]) ||
-      !ld_cg(&gc[GC_BATCH_DEL]))
-    return;
-  const uint32_t V = a.V, mask = (1u << a.ftab_bits) - 1u;
+  if ((ld_cg(&gc[GC_ERR]) & kErrInval) || !ld_cg(&gc[GC_LABELS_VALID]) || ld_cg(&gc[GC_BATCH_MERGE]) != a.batch) return;
+  const uint32_t V = a.V, t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  for (uint32_t w = t; w < V; w += stride) label[w] = inc_find(a.ipar, label[w], V);
+  if (ld_cg(&gc[GC_BATCH_DEL]) != a.batch) return;
+  const uint32_t mask = (1u << a.ftab_bits) - 1u;
   bool warm = false;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+  for (size_t i = t; i < n; i += stride) {
     if (ops[i] >= 0) continue;
     const uint32_t u = edges[2 * i], v = edges[2 * i + 1];
     const uint64_t id = (uint64_t)min(u, v) * V + max(u, v);
@@ -291,17 +299,7 @@ __global__ void k_incr_dead(const uint32_t* __restrict__ edges, const int8_t* __
       }
     }
   }
-  if (__any_sync(0xffffffffu, warm) && (threadIdx.x & 31) == 0) gc[GC_WARM] = 1;
-}
-
-// Labels after the merges: every vertex takes its label's root. Merges are
-// exact whatever else the batch did: a delete can only split components,
-// and one that removed a forest edge has set GC_WARM, so the next query
-// recovers from the fragments of the remaining forest.
-__global__ void k_incr_finish(uint32_t* label, uint32_t* ipar, uint32_t V, uint32_t* gc) {
-  if (!ld_cg(&gc[GC_LABELS_VALID]) || !ld_cg(&gc[GC_BATCH_MERGE])) return;
-  for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < V; w += gridDim.x * blockDim.x)
-    label[w] = inc_find(ipar, label[w], V);
+  if (warm) gc[GC_WARM] = 1;
 }
 
 cudaError_t launch_incremental(cupc_graph* g, const uint32_t* edges, const int8_t* ops, size_t n, cudaStream_t s) {
@@ -311,9 +309,6 @@ cudaError_t launch_incremental(cupc_graph* g, const uint32_t* edges, const int8_
     if (e != cudaSuccess) return e;
     g->sort_pending = false;
   }
-  cudaError_t e = cudaMemsetAsync(g->gc + GC_BATCH_DEL, 0, sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(g->gc + GC_BATCH_MERGE, 0, sizeof(uint32_t), s);
-  if (e != cudaSuccess) return e;
   IncArgs a;
   a.label = g->label;
   a.ipar = g->ipar;
@@ -325,12 +320,13 @@ cudaError_t launch_incremental(cupc_graph* g, const uint32_t* edges, const int8_
   a.ftab_pos = g->ftab_pos;
   a.ftab_bits = g->ftab_bits;
   a.V = g->V;
+  if (++g->inc_batch == 0) g->inc_batch = 1;  // 0: no batch
+  a.batch = g->inc_batch;
   a.gc = g->gc;
   const int grid = (int)std::min<size_t>((n + 255) / 256, (size_t)g->sms * 8);
   k_incr<<<grid, 256, 0, s>>>(edges, ops, n, a);
-  k_incr_dead<<<grid, 256, 0, s>>>(edges, ops, n, a);
-  k_incr_finish<<<(int)std::min<size_t>((g->V + 255) / 256, (size_t)g->sms * 4), 256, 0, s>>>(g->label, g->ipar,
-                                                                                                g->V, g->gc);
+  const size_t rest = std::max<size_t>(n, g->V);
+  k_incr_rest<<<(int)std::min<size_t>((rest + 255) / 256, (size_t)g->sms * 4), 256, 0, s>>>(edges, ops, n, g->label, a);
   return cudaGetLastError();
 }
 
