@@ -46,38 +46,10 @@ __device__ __forceinline__ bool edge_id_ordered(uint64_t x, uint32_t V) {
   return u < x - u * V;
 }
 
-// Sample a layer-r sum held by a warp (lane l holds buckets l + 32q,
-// q < NQ): ZERO if the deterministic bucket is zero, else the first good
-// bucket in index order j = l + 32q (deterministic bucket, then
-// column-major), else FAIL. A bucket is good when its alpha is non-zero,
-// its checksum holds and alpha is an edge id u*V+v with u < v. Returns 0/1/2
-// in every lane and the edge id in `edge`. Bucket groups q are tested in
-// order and the test stops at the first group holding a good bucket (the
-// flag is warp-uniform, so later groups are skipped, not hashed).
-template <uint32_t NQ>
-__device__ __forceinline__ uint32_t warp_sample(const ulonglong2 (&acc)[NQ], uint32_t W, uint32_t V, uint64_t kchk,
-                                                uint64_t& edge) {
-  const uint32_t lane = threadIdx.x & 31;
-  edge = 0;
-  if (__shfl_sync(0xffffffffu, (acc[0].x | acc[0].y) == 0 ? 1u : 0u, 0)) return 0;
-  uint32_t found = 0;
-  uint64_t e = 0;
-#pragma unroll
-  for (uint32_t q = 0; q < NQ; q++) {
-    if (!found) {
-      const uint32_t j = lane + 32 * q;
-      const bool good =
-          j < W && acc[q].x != 0 && mix64(acc[q].x ^ kchk) == acc[q].y && edge_id_ordered(acc[q].x, V);
-      const uint32_t m = __ballot_sync(0xffffffffu, good);
-      if (m) {
-        e = __shfl_sync(0xffffffffu, acc[q].x, __ffs(m) - 1);
-        found = 1;
-      }
-    }
-  }
-  edge = e;
-  return found ? 1u : 2u;
-}
+// A bucket is good when its alpha is non-zero, its checksum holds and alpha is
+// an edge id u*V+v with u < v. A sum's sample is ZERO if the deterministic
+// bucket is zero, else the first good bucket in index order (deterministic
+// bucket, then column-major), else FAIL.
 
 // Whether buckets base + lane + 32q, q < 2, of a warp's sum hold a good one;
 // `edge` is the first one's id, in index order.
@@ -111,21 +83,6 @@ __device__ __forceinline__ void warp_xor_part(ulonglong2 (&acc)[2], const ulongl
 #pragma unroll
   for (uint32_t q = 0; q < 2; q++) {
     const uint32_t b = base + lane + 32 * q;
-    if (b < W) {
-      const ulonglong2 x = __ldg(row + b);
-      acc[q].x ^= x.x;
-      acc[q].y ^= x.y;
-    }
-  }
-}
-
-// lane l XORs buckets l + 32q of one member's row into acc
-template <uint32_t NQ>
-__device__ __forceinline__ void warp_xor_row(ulonglong2 (&acc)[NQ], const ulonglong2* __restrict__ row, uint32_t W,
-                                             uint32_t lane) {
-#pragma unroll
-  for (uint32_t q = 0; q < NQ; q++) {
-    const uint32_t b = lane + 32 * q;
     if (b < W) {
       const ulonglong2 x = __ldg(row + b);
       acc[q].x ^= x.x;

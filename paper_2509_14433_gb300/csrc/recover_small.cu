@@ -37,30 +37,9 @@ namespace cupc {
 
 namespace {
 
-// Members of a warp's range whose rows are prefetched ahead of the fold.
-constexpr uint32_t kClAhead = 4;
-
-// Rows of two members at once, all loads issued before the first XOR.
-template <uint32_t NQ>
-__device__ __forceinline__ void warp_xor_rows2(ulonglong2 (&acc)[NQ], const ulonglong2* __restrict__ r0,
-                                               const ulonglong2* __restrict__ r1, uint32_t W, uint32_t lane) {
-  ulonglong2 x[NQ], y[NQ];
-#pragma unroll
-  for (uint32_t q = 0; q < NQ; q++) {
-    const uint32_t b = lane + 32 * q;
-    x[q] = make_ulonglong2(0, 0);
-    y[q] = make_ulonglong2(0, 0);
-    if (b < W) {
-      x[q] = __ldg(r0 + b);
-      y[q] = __ldg(r1 + b);
-    }
-  }
-#pragma unroll
-  for (uint32_t q = 0; q < NQ; q++) {
-    acc[q].x ^= x[q].x ^ y[q].x;
-    acc[q].y ^= x[q].y ^ y[q].y;
-  }
-}
+// Sample states of a component in cand[K].y besides 0 ZERO, 1 GOOD and 2 FAIL:
+// the next kPrefix buckets are needed.
+constexpr uint32_t kClAgain = 3;
 
 // The leader's shared memory, V entries each: x (grouping: count and cursor
 // of a label; hook: max edge << 32 | pointer), lab (vertex -> label), e
@@ -275,8 +254,6 @@ __device__ void cl_hook(const RecArgs& a, const ClSmem& m, uint32_t V, uint32_t 
 
 }  // namespace
 
-// NQ: buckets per lane (W <= 32 NQ).
-template <uint32_t NQ>
 __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
   extern __shared__ __align__(16) unsigned char cl_dyn[];
   __shared__ uint32_t s_red[128];
@@ -404,18 +381,23 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
     }
   }
 
-  for (uint32_t r = 0;; r++) {
-    const bool multi = r > 0 || warm;  // components may have several members
-    if (leader) {
+  // r: the round whose samples are taken; a pass over the buckets from `base`
+  // on (all but the first only for components marked kClAgain)
+  uint32_t r = 0, base = 0;
+  bool first = true, grouped = false;
+  while (true) {
+    if (leader && base == 0) {
+      const uint32_t next = first ? 0 : r + 1;
+      const bool multi = next > 0 || warm;  // components may have several members
       // One live component left: every other component is final and its
       // merged sketch is zero, and the XOR of all vertex sketches of a layer
       // is zero, so the live one samples ZERO: log the round, stop. Imported
       // words need not come from a stream: then the round is run.
-      bool stop = c_done || r >= a.L;
+      bool stop = c_done || next >= a.L;
       if (!stop && multi && a.sum_zero && c_nlive == 1) {
         if (tid == 0) {
-          a.log_live[r] = 1;
-          c_rounds = r + 1;
+          a.log_live[next] = 1;
+          c_rounds = next + 1;
           c_complete = 1;
         }
         stop = true;
@@ -425,14 +407,26 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
       if (tid == 0) {
         gc[GC_NMEMBERS] = n;
         gc[GC_ACTIVE] = stop ? 0u : (multi ? 2u : 1u);
+        gc[GC_RETRY] = 0;
       }
+    } else if (leader && tid == 0) {
+      gc[GC_ACTIVE] = 3u;  // another pass of the same round
+      gc[GC_RETRY] = 0;
     }
     cluster_sync_all();  // release/acquire at cluster scope: the groups and gc words are visible
     const uint32_t ctl = ld_cg(&gc[GC_ACTIVE]);
     if (ctl == 0) break;
     const uint32_t n = ld_cg(&gc[GC_NMEMBERS]);
-    const bool grouped = ctl == 2;
-    // ---- reduce + sample: warp g takes members [g q, (g+1) q), q <= 32
+    if (ctl == 3) {
+      if (!leader) base += kPrefix;
+    } else {
+      r = first ? 0 : r + 1;
+      first = false;
+      base = 0;
+      grouped = ctl == 2;
+    }
+    // ---- reduce + sample: warp g takes members [g q, (g+1) q), q <= 32; as in
+    // the grid-wide kernel the first kPrefix buckets nearly always decide
     {
       const uint64_t kchk = a.keys[r * (a.C + 1) + a.C];
       const uint32_t q = (n + nwarps - 1) / nwarps;
@@ -442,14 +436,26 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
         uint32_t pk = kNoneU32;
         if (lane < cnt) pk = grouped ? ld_cg(&a.perm[p0 + lane]) : ((p0 + lane) << 16 | (p0 + lane));
         const ulonglong2* layer = a.sketch + (size_t)r * V * W;
-        // rows of the next kClAhead members head for L1 while earlier ones fold
-        uint32_t pf = 0;
-        auto prefetch_to = [&](uint32_t until) {
-          for (; pf < until; pf++) {
-            const ulonglong2* row = layer + (size_t)(__shfl_sync(0xffffffffu, pk, pf) & 0xFFFFu) * W;
+        // sum of the members that lanes [m0, m1) hold in k, buckets b + lane + 32 i
+        auto sum_rows = [&](ulonglong2(&acc)[2], uint32_t k, uint32_t m0, uint32_t m1, uint32_t b) {
+          for (uint32_t mm = m0; mm < m1; mm += 4) {
+            ulonglong2 x[4][2];
 #pragma unroll
-            for (uint32_t b = 0; b < NQ; b++)
-              if (lane + 32 * b < W) asm volatile("prefetch.global.L1 [%0];" ::"l"(row + lane + 32 * b));
+            for (uint32_t j = 0; j < 4; j++) {
+              const ulonglong2* row = layer + (size_t)(__shfl_sync(0xffffffffu, k, (mm + j) & 31) & 0xFFFFu) * W;
+#pragma unroll
+              for (uint32_t i = 0; i < 2; i++) {
+                const uint32_t bb = b + lane + 32 * i;
+                x[j][i] = mm + j < m1 && bb < W ? __ldg(row + bb) : make_ulonglong2(0, 0);
+              }
+            }
+#pragma unroll
+            for (uint32_t j = 0; j < 4; j++)
+#pragma unroll
+              for (uint32_t i = 0; i < 2; i++) {
+                acc[i].x ^= x[j][i].x;
+                acc[i].y ^= x[j][i].y;
+              }
           }
         };
         uint32_t i = 0;
@@ -458,21 +464,12 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
           const uint32_t run = ~(__ballot_sync(0xffffffffu, (pk >> 16) == K) >> i);  // members i.. of K
           const uint32_t j = min(cnt, run ? i + (uint32_t)__ffs(run) - 1 : 32u);
           const uint32_t seg = grouped ? ld_cg(&a.roff[K]) : 0u;
-          ulonglong2 acc[NQ];
-#pragma unroll
-          for (uint32_t b = 0; b < NQ; b++) acc[b] = make_ulonglong2(0, 0);
-          uint32_t mm = i;
-          for (; mm + 2 <= j; mm += 2) {
-            prefetch_to(min(cnt, mm + 2 + kClAhead));
-            const uint32_t w0 = __shfl_sync(0xffffffffu, pk, mm) & 0xFFFFu;
-            const uint32_t w1 = __shfl_sync(0xffffffffu, pk, mm + 1) & 0xFFFFu;
-            warp_xor_rows2(acc, layer + (size_t)w0 * W, layer + (size_t)w1 * W, W, lane);
+          if (base && ld_cg((const uint64_t*)&a.cand[K].y) != kClAgain) {
+            i = j;
+            continue;
           }
-          if (mm < j) {
-            prefetch_to(min(cnt, mm + 1 + kClAhead));
-            const uint32_t w0 = __shfl_sync(0xffffffffu, pk, mm) & 0xFFFFu;
-            warp_xor_row(acc, layer + (size_t)w0 * W, W, lane);
-          }
+          ulonglong2 acc[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+          sum_rows(acc, pk, i, j, base);
           uint32_t s0 = p0 + i, s1 = s0 + 1;
           if (grouped) {
             s0 = seg & 0xFFFFu;
@@ -483,8 +480,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
           if (npieces > 1) {
             ulonglong2* dst = a.acc + (size_t)K * W;
 #pragma unroll
-            for (uint32_t b = 0; b < NQ; b++) {
-              const uint32_t bb = lane + 32 * b;
+            for (uint32_t b = 0; b < 2; b++) {
+              const uint32_t bb = base + lane + 32 * b;
               if (bb < W && (acc[b].x | acc[b].y)) {
                 atomicXor((unsigned long long*)&dst[bb].x, (unsigned long long)acc[b].x);
                 atomicXor((unsigned long long*)&dst[bb].y, (unsigned long long)acc[b].y);
@@ -497,8 +494,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
             if (mine) {  // the last range: every other range's XOR is in acc[K]
               __threadfence();
 #pragma unroll
-              for (uint32_t b = 0; b < NQ; b++) {
-                const uint32_t bb = lane + 32 * b;
+              for (uint32_t b = 0; b < 2; b++) {
+                const uint32_t bb = base + lane + 32 * b;
                 acc[b] = make_ulonglong2(0, 0);
                 if (bb < W) {
                   acc[b] = __ldcg(dst + bb);
@@ -510,7 +507,26 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
           }
           if (mine) {
             uint64_t e = 0;
-            const uint32_t res = warp_sample(acc, W, V, kchk, e);
+            uint32_t res = 2;
+            if (base == 0)
+              res = warp_sample_prefix(acc, W, V, kchk, e);
+            else if (warp_find(acc, base, W, V, kchk, e))
+              res = 1;
+            // one of at most 32 members reads on at once
+            const bool here = s1 - s0 <= 32;
+            if (res == 2 && here && base + kPrefix < W) {
+              uint32_t k = s0 + lane;
+              if (grouped && k < s1) k = ld_cg(&a.perm[k]);
+              for (uint32_t b = base + kPrefix; res == 2 && b < W; b += kPrefix) {
+                ulonglong2 more[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
+                sum_rows(more, k, 0, s1 - s0, b);
+                if (warp_find(more, b, W, V, kchk, e)) res = 1;
+              }
+            }
+            if (res == 2 && !here && base + kPrefix < W) {
+              res = kClAgain;
+              if (lane == 0) atomicAdd(&gc[GC_RETRY], 1u);
+            }
             if (lane == 0) a.cand[K] = make_ulonglong2(e, res);
           }
           i = j;
@@ -519,6 +535,11 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
     }
     cluster_sync_all();  // the samples in cand are visible to the leader
     if (!leader) continue;
+    if (__syncthreads_or(ld_cg(&gc[GC_RETRY]) != 0)) {  // read by all before it is reset
+      base += kPrefix;
+      continue;
+    }
+    base = 0;
     // ---- book the samples of the live components
     for (uint32_t K = tid; K < V; K += nt) {
       m.e[K] = kNoneU32;
@@ -595,22 +616,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
 
 static size_t cl_smem_bytes(uint32_t V) { return (size_t)V * (8 + 4 * 4 + 2); }
 
-// Buckets per lane of the instantiation that serves W buckets.
-static uint32_t cl_nq(uint32_t W) { return W <= 128 ? 4 : W <= 160 ? 5 : W <= 192 ? 6 : 8; }
-
-static const void* cl_kernel(uint32_t nq) {
-  switch (nq) {
-    case 4: return (const void*)k_recover_cl<4>;
-    case 5: return (const void*)k_recover_cl<5>;
-    case 6: return (const void*)k_recover_cl<6>;
-    default: return (const void*)k_recover_cl<8>;
-  }
-}
-
 cudaError_t setup_recover_cluster(cupc_graph* g) {
   g->rec_cluster = 0;
   if (g->V > kClMaxV || g->W > 32 * kWarpBuckets) return cudaSuccess;
-  const void* fn = cl_kernel(cl_nq(g->W));
+  const void* fn = (const void*)k_recover_cl;
   const size_t smem = cl_smem_bytes(kClMaxV);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -658,7 +667,7 @@ cudaError_t launch_recover_cluster(cupc_graph* g, const RecArgs& a, cudaStream_t
   cfg.numAttrs = 1;
   RecArgs args = a;
   void* params[] = {&args};
-  return cudaLaunchKernelExC(&cfg, cl_kernel(cl_nq(g->W)), params);
+  return cudaLaunchKernelExC(&cfg, (const void*)k_recover_cl, params);
 }
 
 }  // namespace cupc
