@@ -924,11 +924,14 @@ cudaError_t setup_recover(cupc_graph* g) {
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_recover, kRecThreads, kHookBytes);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  // about four vertices per warp in round 0 (every vertex samples its own
-  // sketch); fewer CTAs for small V keep the grid barriers cheap
-  uint32_t want = (g->V + kRecThreads / 8 - 1) / (kRecThreads / 8);
-  if (want < 16) want = 16;
-  uint32_t cap = (uint32_t)(per_sm * g->sms);
+  // 128 vertices a CTA: few CTAs keep the grid barriers cheap and leave room
+  // for other graphs' recoveries (a CTA fills an SM, and a cooperative launch
+  // waits until all of its CTAs fit). GB300, us for one query with 64, 128,
+  // 256 vertices a CTA: V = 8000 165, 163, 172; V = 16384 208, 207, 223; V =
+  // 24000 228, 228, 235; 16 served graphs of 1024..32768 vertices: 2916, 2608,
+  // 2243.
+  const uint32_t want = std::max(16u, (g->V + 127) / 128);
+  const uint32_t cap = (uint32_t)(per_sm * g->sms);
   g->rec_grid = (int)(want < cap ? want : cap);
   return setup_recover_cluster(g);
 }
