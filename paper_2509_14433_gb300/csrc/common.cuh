@@ -230,6 +230,7 @@ struct cupc_graph {
     int smem, grid;
   } tune_b[16];
   int rec_grid;
+  int rec_share;  // at most this many CTAs while other recoveries wait (0: no limit)
   int rec_cluster;  // CTAs of the one-cluster recovery (0: the grid-wide kernel)
   // sketches and keys
   ulonglong2* sketch;  // L*V*W

@@ -929,7 +929,7 @@ cudaError_t setup_recover(cupc_graph* g) {
   // waits until all of its CTAs fit). GB300, us for one query with 64, 128,
   // 256 vertices a CTA: V = 8000 165, 163, 172; V = 16384 208, 207, 223; V =
   // 24000 228, 228, 235; 16 served graphs of 1024..32768 vertices: 2916, 2608,
-  // 2243.
+  // 2243 (the server limits the grids further while several queries wait).
   const uint32_t want = std::max(16u, (g->V + 127) / 128);
   const uint32_t cap = (uint32_t)(per_sm * g->sms);
   g->rec_grid = (int)(want < cap ? want : cap);
@@ -980,7 +980,8 @@ cudaError_t launch_recover(cupc_graph* g, cudaStream_t s, bool force) {
   }
   ProfScope ps(g, s, PC_RECOVER, 1);
   void* args[] = {&a};
-  return cudaLaunchCooperativeKernel((const void*)k_recover, dim3(g->rec_grid), dim3(kRecThreads), args, kHookBytes,
+  const int grid = g->rec_share ? std::min(g->rec_grid, g->rec_share) : g->rec_grid;
+  return cudaLaunchCooperativeKernel((const void*)k_recover, dim3(grid), dim3(kRecThreads), args, kHookBytes,
                                      s);
 }
 

@@ -186,12 +186,27 @@ void finish_ticket(cupc_server* s, const Request& r, cupc_status st, Clock::time
   if (r.pin_bytes) s->pin_alloc.release(r.pin_off);
 }
 
-// Stream-ordered capture of a graph's sticky error word after its work:
-// copied into pinned memory, then cleared, so each request reports the
-// errors its own batch or pairs raised (as cupc_sync would).
-void capture_status(cupc_graph* g, uint32_t* pinned_word, cudaStream_t st) {
-  cudaMemcpyAsync(pinned_word, g->gc + GC_ERR, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
-  cudaMemsetAsync(g->gc + GC_ERR, 0, sizeof(uint32_t), st);
+// Stream-ordered capture of graphs' sticky error words after their work: into
+// pinned memory, then cleared, so each request reports the errors its own
+// batch or pairs raised (as cupc_sync would). One launch per kStatusMax graphs.
+constexpr uint32_t kStatusMax = 64;
+struct StatusArgs {
+  uint32_t* err[kStatusMax];
+  uint32_t* word[kStatusMax];
+  uint32_t n;
+};
+__global__ void k_status(StatusArgs a) {
+  const uint32_t i = threadIdx.x;
+  if (i >= a.n) return;
+  *a.word[i] = *a.err[i];
+  *a.err[i] = 0;
+}
+void capture_status(StatusArgs& a, cupc_graph* g, uint32_t* pinned_word, bool last, cudaStream_t st) {
+  a.err[a.n] = g->gc + GC_ERR;
+  a.word[a.n++] = pinned_word;
+  if (!last && a.n < kStatusMax) return;
+  k_status<<<1, kStatusMax, 0, st>>>(a);
+  a.n = 0;
 }
 
 cupc_status status_of(uint32_t err) {
@@ -241,7 +256,32 @@ void admit(cupc_server* s) {
 constexpr size_t kLaunchEdges = (size_t)1 << 18;
 constexpr int kIdleSpinUs = 500;
 
+// Queries in flight, and those that could be started now.
+size_t queries_pending(const cupc_server* s) {
+  size_t k = 0;
+  for (bool b : s->q_busy) k += b;
+  for (const auto& kv : s->inst) {
+    const Instance& in = kv.second;
+    k += in.resident && !in.busy && !in.q.empty() && in.q.front().kind == K_QUERY;
+  }
+  return k;
+}
+
+// CTAs a recovery may take, so that those of all pending queries (as many as
+// there are streams) run side by side. Alone a recovery is fastest on many
+// CTAs, but with fewer it gets slower by far less than in proportion. GB300, us
+// for a turn of updates and queries: 16 graphs of 1024..32768 vertices 2648
+// with no limit, 1911 with a quarter of the SMs each (4 streams), 2144 with an
+// eighth; 16 graphs of 32768 vertices 5086, 2815, 3321; 3 graphs of 2000..30000
+// vertices 695, 635, 820.
+int recover_share(const cupc_server* s, int sms) {
+  const size_t k = std::min(queries_pending(s), s->q_busy.size());
+  return k > 1 ? std::max(16, sms / (int)k) : 0;
+}
+
 void worker_loop(cupc_server* s) {
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
   cudaSetDevice(s->device);
   Clock::time_point last_busy = Clock::now();
   std::unique_lock<std::mutex> lk(s->mu);
@@ -322,11 +362,13 @@ void worker_loop(cupc_server* s) {
         cudaStream_t qs = s->q_streams[slot];
         const uint8_t* payload = s->pinned + r.pin_off;
         cudaMemcpyAsync(s->q_pairs[slot], payload, r.n * 8, cudaMemcpyHostToDevice, qs);
+        in.g->rec_share = recover_share(s, sms);
         cupc_status st = cupc_query(in.g, s->q_pairs[slot], r.n, s->q_out[slot], (cupc_stream)qs);
         uint8_t* pout = s->pinned + r.pin_off;  // answers reuse the payload space
         cudaMemcpyAsync(pout, s->q_out[slot], r.n, cudaMemcpyDeviceToHost, qs);
         Inflight f;
-        capture_status(in.g, s->stat_words + in.slot, qs);
+        StatusArgs sa{};
+        capture_status(sa, in.g, s->stat_words + in.slot, true, qs);
         f.kind = K_QUERY;
         f.qslot = slot;
         f.m = r.n;
@@ -399,8 +441,9 @@ void worker_loop(cupc_server* s) {
       f.qslot = -1;
       f.m = 0;
       f.pinned_out = nullptr;
+      StatusArgs sa{};
       for (size_t i = 0; i < gs.size(); i++)
-        capture_status(gs[i], s->stat_words + s->inst[upd_insts[i]].slot, s->upd_stream);
+        capture_status(sa, gs[i], s->stat_words + s->inst[upd_insts[i]].slot, i + 1 == gs.size(), s->upd_stream);
       f.ev = take_event(s);
       cudaEventRecord(f.ev, s->upd_stream);
       for (size_t i = 0; i < upd_insts.size(); i++)
