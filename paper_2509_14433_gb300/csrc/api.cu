@@ -68,6 +68,9 @@ uint32_t ftab_bits(uint32_t V) {
   return b < 6 ? 6 : b;
 }
 
+// Arrays of counters of the update's grouping: one where no batch is sharded.
+size_t count_shards(const Dims& d) { return d.V <= kPrivMaxV || d.max_batch < kShardEdges ? 1 : kShards; }
+
 Layout layout(const Dims& d) {
   Layout l{};
   size_t off = 0;
@@ -80,8 +83,8 @@ Layout layout(const Dims& d) {
   l.sketch = take((size_t)d.L * V * d.W * sizeof(ulonglong2));
   l.keys = take(key_words(d.L, d.C) * sizeof(uint64_t));
   l.gc = take(GC_SLOTS * sizeof(uint32_t));
-  l.cnt = take(V * 4);
-  l.cursor = take(V * 4);
+  l.cnt = take(count_shards(d) * V * 4);
+  l.cursor = take(count_shards(d) * V * 4);
   l.rec = take(rec_entries(V, B) * 8);
   l.work = take(kWorkSlots * 4);
   l.stage_edges = take(2 * B * 4);
@@ -213,6 +216,7 @@ cupc_status cupc_init(uint32_t V, uint64_t seed, const cupc_params* params, void
   g->sketch = (ulonglong2*)(b + l.sketch);
   g->keys = (uint64_t*)(b + l.keys);
   g->gc = (uint32_t*)(b + l.gc);
+  g->shards = (uint32_t)count_shards(d);
   g->cnt = (uint32_t*)(b + l.cnt);
   g->cursor = (uint32_t*)(b + l.cursor);
   g->rec = (uint64_t*)(b + l.rec);

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_m(const BatchHead* __rest
   for (uint32_t x = blockIdx.x; x < h->total_slices; x += gridDim.x) {
     const InstDesc& g = d[inst_of<false>(d, k, x)];
     const bool dropped = (ld_cg(&g.gc[GC_ERR]) & kErrInval) != 0;
-    plan_slice(g.cnt, g.cursor, g.rec, g.V, g.cap, x - g.slice_base, g.work, dropped);
+    plan_slice(g.cnt, g.cursor, g.rec, g.V, g.cap, x - g.slice_base, g.work, dropped, 1u);
     if (!dropped && g.n > 0 && x == g.slice_base && threadIdx.x == 0) g.gc[GC_BATCHES] += 1;
   }
 }

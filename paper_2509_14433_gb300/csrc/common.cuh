@@ -43,6 +43,14 @@ constexpr uint32_t kMinItemRecords = 64;
 constexpr uint32_t kPrivMaxV = 24576;
 constexpr uint32_t kPrivPerVertex = 1;
 constexpr uint32_t kPrivMinCtas = 48;
+// Batches of at least kShardEdges edges on larger graphs count and scatter in
+// kShards arrays of counters, one per CTA modulo kShards, so that the records
+// of a hub do not all queue at one address. GB300, us for a batch with 4 arrays
+// (1): V = 2^17, 2^22 R-MAT edges 2407 (2514); V = 2^15, 2^20 R-MAT
+// edges 615 (711). 8 or 16 arrays, or sharding from 2^16 or 2^18 edges, gave
+// nothing more.
+constexpr uint32_t kShards = 4;
+constexpr uint32_t kShardEdges = 1u << 20;
 // The update's plan: vertices per slice (one CTA each) and threads per CTA.
 constexpr uint32_t kPlanSlice = 1024;
 constexpr uint32_t kPlanThreads = 256;
@@ -237,8 +245,9 @@ struct cupc_graph {
   uint64_t* keys;      // key_words(L, C)
   uint32_t* gc;        // GC_SLOTS device counters
   // update scratch
-  uint32_t* cnt;       // V
-  uint32_t* cursor;    // V
+  uint32_t shards;     // arrays of V counters in cnt and cursor
+  uint32_t* cnt;       // shards * V
+  uint32_t* cursor;    // shards * V
   uint64_t* rec;       // rec_cap endpoint records, grouped by vertex
   uint32_t rec_cap;
   uint32_t* work;      // kWorkSlots counters of the current chunk

@@ -135,6 +135,7 @@ extern "C" cupc_status cupc_update_sketch_static(void* sketch, uint32_t V, uint6
   g.sketch = (ulonglong2*)sketch;
   g.gc = (uint32_t*)(ds->scratch + kOffGc);
   g.keys = (uint64_t*)(ds->scratch + kOffKeys);
+  g.shards = 1;
   g.cnt = (uint32_t*)(ds->scratch + kOffCnt);
   g.cursor = (uint32_t*)(ds->scratch + kOffCursor);
   g.rec = (uint64_t*)(ds->scratch + kOffRec);

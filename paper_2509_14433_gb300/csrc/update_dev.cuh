@@ -56,9 +56,10 @@ __device__ __forceinline__ uint64_t block_scan(uint64_t v, uint64_t* total) {
 // (cap), unpadded. A slice takes its two ranges with one atomic each, so
 // slices need not wait on one another; their order in the array does not
 // matter, because the apply kernel reads each record's vertex from the
-// record itself.
+// record itself. Counts come in `shards` arrays of V; a vertex's segment is
+// divided among them, cursor[k*V + w] = the start of shard k's records.
 __device__ __forceinline__ void plan_slice(uint32_t* cnt, uint32_t* cursor, uint64_t* rec, uint32_t V, uint32_t cap,
-                                           uint32_t slice, uint32_t* work, bool dropped) {
+                                           uint32_t slice, uint32_t* work, bool dropped, uint32_t shards) {
   __shared__ uint32_t s_base[2];
   constexpr uint32_t kPer = kPlanSlice / kPlanThreads;
   const uint32_t w0 = slice * kPlanSlice + kPer * threadIdx.x;
@@ -66,13 +67,16 @@ __device__ __forceinline__ void plan_slice(uint32_t* cnt, uint32_t* cursor, uint
   uint64_t sum = 0;  // direct records << 32 | padded fold records
 #pragma unroll
   for (uint32_t k = 0; k < kPer; k++) {
-    c[k] = w0 + k < V ? cnt[w0 + k] : 0;
+    c[k] = 0;
+    for (uint32_t q = 0; q < shards && w0 + k < V; q++) c[k] += cnt[(size_t)q * V + w0 + k];
     sum += c[k] <= kDirectMax ? (uint64_t)c[k] << 32 : (uint64_t)((c[k] + kPad - 1) / kPad * kPad);
   }
-#pragma unroll
-  for (uint32_t k = 0; k < kPer; k++)
-    if (w0 + k < V) cnt[w0 + k] = 0;
-  if (dropped) return;
+  if (dropped) {
+    for (uint32_t q = 0; q < shards; q++)
+      for (uint32_t k = 0; k < kPer; k++)
+        if (w0 + k < V) cnt[(size_t)q * V + w0 + k] = 0;
+    return;
+  }
   uint64_t total;
   const uint64_t before = block_scan(sum, &total);
   if (threadIdx.x < 2) {
@@ -84,11 +88,15 @@ __device__ __forceinline__ void plan_slice(uint32_t* cnt, uint32_t* cursor, uint
 #pragma unroll
   for (uint32_t k = 0; k < kPer; k++) {
     if (c[k] == 0) continue;
-    if (c[k] <= kDirectMax) {
-      direct -= c[k];
-      cursor[w0 + k] = direct;
-    } else {
-      cursor[w0 + k] = fold;
+    uint32_t at = fold;
+    if (c[k] <= kDirectMax) at = direct -= c[k];
+    for (uint32_t q = 0; q < shards; q++) {
+      const size_t i = (size_t)q * V + w0 + k;
+      cursor[i] = at;
+      at += cnt[i];
+      cnt[i] = 0;
+    }
+    if (c[k] > kDirectMax) {
       const uint32_t end = fold + (c[k] + kPad - 1) / kPad * kPad;
       for (uint32_t i = fold + c[k]; i < end; i++) rec[i] = make_record(w0 + k, w0 + k);
       fold = end;

@@ -87,3 +87,21 @@ def test_batches_around_the_one_launch_limit(n):
     assert dev.update(e[:1]) == 0 and ref.update(e[:1]) == O.OK
     assert dev.sync() == 0 and dev.stats()["chunks"] == 2
     assert np.array_equal(dev.export(), ref.export())
+
+
+def test_a_sharded_count_with_hubs():
+    # V above the shared-histogram limit and enough edges for the sharded
+    # counters; few layers and columns keep the oracle quick
+    from tests._dev import Dev
+
+    V, L, C, D = 30000, 2, 2, 6
+    dev, ref = Dev(V, 4, (L, C, D, 1 << 21)), O.Graph(V, 4, L, C, D)
+    g = WL.rng(8)
+    e = np.concatenate([_stars(V, (20000, 9000, 1, 2, 3), g), WL.uniform_pairs(V, 1 << 20, g)])
+    for part in (e, e[: 1 << 20], e[: (1 << 20) - 1]):
+        assert dev.update(part) == 0 and ref.update(part) == O.OK
+        bad = part.copy()
+        bad[5, 0] = V
+        assert dev.update(bad) == 0 and dev.sync() != 0  # its counts are cleared
+    assert dev.sync() == 0
+    assert np.array_equal(dev.export(), ref.export())
