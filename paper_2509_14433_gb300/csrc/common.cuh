@@ -93,12 +93,11 @@ __host__ __device__ constexpr uint32_t layer_groups(uint32_t L, uint32_t P) { re
 // Edge ids of at most 32 bits: V^2 <= 2^32.
 inline bool small_ids(uint32_t V) { return V <= 65536; }
 // Batches of at most kSmallEdges edges are applied by one launch (k_small).
-// Against the grouped path, us, uniform batches: V = 1024, 4096 edges 13 (27),
-// 8192 edges 21 (29), 12000 edges 31 (31); V = 2^14, 8192 edges 56 (72), 12000
-// edges 84 (94); V = 2^17, 4096 edges 40 (46), 8192 edges 83 (86), 12000 edges
-// 120 (118); R-MAT on V = 2^17, 8192 edges 58 (72).
-constexpr uint32_t kSmallEdges = 8192;
-constexpr uint32_t kSmallThreads = 256;
+// Against the grouped path, us, uniform batches: V = 1024, 8192 edges 25.1
+// (28.9), 12288 edges 30.1 (32.5); V = 5003, 12288 edges 39.5 (40.7); V = 2^14,
+// 8192 edges 67 (75), 12288 edges 90 (99); V = 2^17, 8192 edges 95 (98), 12288
+// edges 128 (136); R-MAT on V = 2^17, 10000 edges 72 (85), 12288 edges 90 (85).
+constexpr uint32_t kSmallEdges = 12288;
 // Records per chunk of a batch of nrec records on V vertices: at most `most`,
 // and such that the `warps` of a layer group run out of chunks together (a
 // whole number of chunks each, as near as steps of 16 records and the

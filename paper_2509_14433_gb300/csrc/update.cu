@@ -407,18 +407,17 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply(
 }
 
 // A small batch (n <= kSmallEdges edges, one chunk) in one launch: every CTA
-// validates the whole batch, so that none needs to wait for another, then
-// its warps XOR their records' buckets straight into HBM, P records (a lane
-// each) and one layer group at a time. What bounds it is latency: the launch,
-// the batch's loads and one pass per warp.
+// validates the whole batch, so that none needs to wait for another, then its
+// warps XOR their records' buckets straight into HBM, P records (a lane each)
+// and one layer group at a time. What bounds it is latency: the launch, the
+// batch's loads and one pass per warp; the more edges, the bigger the CTAs, so
+// that the validation stays a few loads a thread.
 template <bool kX32>
-__global__ void __launch_bounds__(kSmallThreads) k_small(ulonglong2* __restrict__ sketch,
-                                                         const uint64_t* __restrict__ keys,
-                                                         const uint32_t* __restrict__ edges,
-                                                         const int8_t* __restrict__ ops, uint32_t n, uint32_t* gc,
-                                                         uint32_t V, uint32_t L, uint32_t C, uint32_t D, uint32_t W,
-                                                         uint32_t P, uint32_t ell) {
-  const uint32_t lane = threadIdx.x & 31, gw = blockIdx.x * (kSmallThreads / 32) + (threadIdx.x >> 5);
+__global__ void __launch_bounds__(1024) k_small(ulonglong2* __restrict__ sketch, const uint64_t* __restrict__ keys,
+                                                const uint32_t* __restrict__ edges, const int8_t* __restrict__ ops,
+                                                uint32_t n, uint32_t* gc, uint32_t V, uint32_t L, uint32_t C,
+                                                uint32_t D, uint32_t W, uint32_t P, uint32_t ell) {
+  const uint32_t lane = threadIdx.x & 31, gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const uint32_t groups = layer_groups(L, P), s = lane % P;
   // this warp's records and lanes, in flight during the validation
   const uint32_t i = gw / groups * P + s;  // record i: endpoint i & 1 of edge i / 2
@@ -427,7 +426,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(ulonglong2* __restrict_
   const ApplyLane l = apply_lane(keys, sketch, V, L, C, D, W, P, ell, gw % groups);
   bool drop = (ld_cg(&gc[GC_ERR]) & kErrInval) != 0, bad = false;
 #pragma unroll 4
-  for (uint32_t j = threadIdx.x; j < n; j += kSmallThreads) {
+  for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
     const uint32_t u = edges[2 * j], v = edges[2 * j + 1];
     const int8_t op = ops[j];
     bad |= (u >= V) | (v >= V) | (u == v) | ((op != 1) & (op != -1));
@@ -506,10 +505,11 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
   if (validate_ops && n <= kSmallEdges) {
     ProfScope ps(g, s, PC_APPLY, 1);
     const uint32_t warps = (uint32_t)((2 * n + g->P - 1) / g->P) * layer_groups(g->L, g->P);
-    const uint32_t grid = (warps + kSmallThreads / 32 - 1) / (kSmallThreads / 32);
+    const uint32_t threads = n <= 512 ? 128 : n <= 8192 ? 256 : 1024;
+    const uint32_t grid = (warps + threads / 32 - 1) / (threads / 32);
     auto kern = small_ids(g->V) ? k_small<true> : k_small<false>;
-    kern<<<grid, kSmallThreads, 0, s>>>(g->sketch, g->keys, edges, validate_ops, (uint32_t)n, g->gc, g->V, g->L, g->C,
-                                        g->D, g->W, g->P, g->ell);
+    kern<<<grid, threads, 0, s>>>(g->sketch, g->keys, edges, validate_ops, (uint32_t)n, g->gc, g->V, g->L, g->C, g->D,
+                                  g->W, g->P, g->ell);
     return cudaGetLastError();
   }
   // the setting of this batch size's bucket, else the graph's default

@@ -42,8 +42,8 @@ def test_record_counts_at_the_edges_of_passes_and_chunks(V, L, C, D, rows):
     dev, ref = Dev(V, 5, (L, C, D, 0)), O.Graph(V, 5, L, C, D)
     assert B.cupc_set_tuning(dev.h, 64 if rows == 1 else 0, min(rows, dev.D), 0) == 0
     g = WL.rng(V + rows)
-    e = np.concatenate([_stars(V, COUNTS * 2, g), WL.uniform_pairs(V, 6000, g)])
-    assert len(e) > 8192  # the grouped path
+    e = np.concatenate([_stars(V, COUNTS * 2, g), WL.uniform_pairs(V, 10000, g)])
+    assert len(e) > 12288  # the grouped path
     assert dev.update(e) == 0 and ref.update(e) == O.OK
     assert dev.sync() == 0
     assert np.array_equal(dev.export(), ref.export())
@@ -57,14 +57,14 @@ def test_every_lane_layout(C, D):
     V, L = 500, 5
     dev, ref = Dev(V, 9, (L, C, D, 0)), O.Graph(V, 9, L, C, D)
     g = WL.rng(C * 10 + D)
-    for n in (300, 10000):  # one launch; grouped
+    for n in (300, 13000):  # one launch; grouped
         e = WL.uniform_pairs(V, n, g)
         assert dev.update(e) == 0 and ref.update(e) == O.OK
     assert dev.sync() == 0
     assert np.array_equal(dev.export(), ref.export())
 
 
-@pytest.mark.parametrize("n", [1, 31, 4096, 8191, 8192, 8193])
+@pytest.mark.parametrize("n", [1, 31, 512, 513, 8192, 8193, 12288, 12289])
 def test_batches_around_the_one_launch_limit(n):
     from paper_2509_14433_gb300 import cupc as B
     from tests._dev import Dev
