@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kReplayThreads) k_cutset_replay(const int4* __
 // deterministic bucket is zero, else the first good bucket in index order
 // (deterministic bucket, then column-major), else FAIL. One warp; the result
 // goes to pinned host memory.
-__global__ void k_cutset_sample(const ulonglong2* __restrict__ layer, uint32_t W, uint32_t V, uint64_t kchk,
+__global__ void k_cutset_sample(const ulonglong2* __restrict__ layer, uint32_t W, IdSplit ids, uint64_t kchk,
                                 uint64_t* out) {
   const uint32_t lane = threadIdx.x;
   uint64_t edge = 0;
@@ -79,8 +79,8 @@ __global__ void k_cutset_sample(const ulonglong2* __restrict__ layer, uint32_t W
     ulonglong2 acc[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
     warp_xor_part(acc, layer, base, W, lane);
     if (base == 0)
-      res = warp_sample_prefix(acc, W, V, kchk, edge);
-    else if (warp_find(acc, base, W, V, kchk, edge))
+      res = warp_sample_prefix(acc, W, ids, kchk, edge);
+    else if (warp_find(acc, base, W, ids, kchk, edge))
       res = 1;
   }
   if (lane == 0) {
@@ -419,7 +419,7 @@ cupc_status cupc_cutset_query(const cupc_cutset* c, uint32_t w, uint32_t r, uint
   const int root = root_of(c, (int)w);
   const ulonglong2* layer = reinterpret_cast<const ulonglong2*>(c->agg + (size_t)root * c->SW) + (size_t)r * c->W;
   const uint64_t kchk = graph_key(c->g->seed, r * (c->g->C + 1) + c->g->C);  // the layer's checksum key
-  k_cutset_sample<<<1, 32, 0, s>>>(layer, c->W, c->V, kchk, c->sample);
+  k_cutset_sample<<<1, 32, 0, s>>>(layer, c->W, IdSplit(c->V), kchk, c->sample);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
     cudaGetLastError();
     return CUPC_ECUDA;

@@ -122,8 +122,10 @@ __device__ __forceinline__ void book_samples(const RecArgs& a, uint32_t r, bool 
     if (res == 0) {
       a.final_[K] = 1;
     } else if (res == 1) {
-      const uint32_t u = (uint32_t)(e / a.V), v = (uint32_t)(e % a.V);
-      const uint32_t lu = multi ? ld_cg(&a.label[u]) : u, lv = multi ? ld_cg(&a.label[v]) : v;
+      uint64_t u, v;
+      a.ids.split(e, u, v);
+      const uint32_t lu = multi ? ld_cg(&a.label[u]) : (uint32_t)u,
+                     lv = multi ? ld_cg(&a.label[v]) : (uint32_t)v;
       if ((lu == K) != (lv == K)) {
         cand = true;
         a.cand[K] = make_ulonglong2(e, ((uint64_t)lu << 32) | lv);
@@ -355,7 +357,7 @@ __device__ __forceinline__ void load_rows(ulonglong2 (&x)[4][2], const ulonglong
 // members perm[s0..s1), by one warp: its edge id, or kNone. Seldom called, so
 // not inlined: its registers would add to the caller's.
 static __device__ __noinline__ uint64_t read_on(const ulonglong2* __restrict__ layer, const uint32_t* perm, uint32_t s0,
-                                                uint32_t s1, uint32_t base, uint32_t W, uint32_t V, uint64_t kchk) {
+                                                uint32_t s1, uint32_t base, uint32_t W, IdSplit ids, uint64_t kchk) {
   const uint32_t lane = threadIdx.x & 31;
   ulonglong2 sum[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
   for (uint32_t t0 = s0; t0 < s1; t0 += 32) {
@@ -373,7 +375,7 @@ static __device__ __noinline__ uint64_t read_on(const ulonglong2* __restrict__ l
     }
   }
   uint64_t e = 0;
-  return warp_find(sum, base, W, V, kchk, e) ? e : kNone;
+  return warp_find(sum, base, W, ids, kchk, e) ? e : kNone;
 }
 
 // The recovery; false if there was nothing to do (no barrier was met).
@@ -621,13 +623,13 @@ __device__ __forceinline__ bool recover_body(const RecArgs& a) {
       uint64_t e = 0;
       uint32_t res = 2;
       if (base == 0)
-        res = warp_sample_prefix(acc, W, V, kchk, e);
-      else if (warp_find(acc, base, W, V, kchk, e))
+        res = warp_sample_prefix(acc, W, a.ids, kchk, e);
+      else if (warp_find(acc, base, W, a.ids, kchk, e))
         res = 1;
       // this warp's own, or a short one: reads on at once
       here = here || s1 - s0 <= kRecSpan;
       for (uint32_t b = base + kPrefix; here && res == 2 && b < W; b += kPrefix) {
-        const uint64_t more = read_on(layer, a.perm, s0, s1, b, W, V, kchk);
+        const uint64_t more = read_on(layer, a.perm, s0, s1, b, W, a.ids, kchk);
         if (more != kNone) {
           e = more;
           res = 1;
@@ -736,15 +738,31 @@ __device__ __forceinline__ bool recover_body(const RecArgs& a) {
             const uint32_t b = lane + 32 * q;
             acc[k][q] = w0 + k < V && b < W ? __ldg(layer + (size_t)(w0 + k) * W + b) : make_ulonglong2(0, 0);
           }
+        // the first 32 buckets of the four tested side by side; they decide
+        // most samples
+        uint32_t zero[kAtOnce], first[kAtOnce];
+#pragma unroll
+        for (uint32_t k = 0; k < kAtOnce; k++) {
+          zero[k] = __ballot_sync(0xffffffffu, (acc[k][0].x | acc[k][0].y) == 0) & 1;
+          first[k] = __ballot_sync(0xffffffffu, good_bucket(acc[k][0], lane, W, a.ids, kchk));
+        }
 #pragma unroll
         for (uint32_t k = 0; k < kAtOnce; k++) {
           if (w0 + k >= V) break;
           uint64_t e = 0;
-          uint32_t res = warp_sample_prefix(acc[k], W, V, kchk, e);
+          uint32_t res = 2;
+          if (zero[k]) {
+            res = 0;
+          } else if (first[k]) {
+            res = 1;
+            e = __shfl_sync(0xffffffffu, acc[k][0].x, __ffs(first[k]) - 1);
+          } else if (warp_find(acc[k], 0, W, a.ids, kchk, e)) {
+            res = 1;
+          }
           for (uint32_t base = kPrefix; res == 2 && base < W; base += kPrefix) {
             ulonglong2 more[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
             warp_xor_part(more, layer + (size_t)(w0 + k) * W, base, W, lane);
-            if (warp_find(more, base, W, V, kchk, e)) res = 1;
+            if (warp_find(more, base, W, a.ids, kchk, e)) res = 1;
           }
           stash(w0 + k, res, e);
         }
@@ -941,6 +959,7 @@ cudaError_t launch_recover(cupc_graph* g, cudaStream_t s, bool force) {
   a.sketch = g->sketch;
   a.keys = g->keys;
   a.V = g->V;
+  a.ids = IdSplit(g->V);
   a.L = g->L;
   a.C = g->C;
   a.D = g->D;

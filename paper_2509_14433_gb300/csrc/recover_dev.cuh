@@ -7,10 +7,35 @@
 
 namespace cupc {
 
+// The endpoints of an edge id x = u*V + v. Every sample tests its id's order,
+// and a 64-bit division is a long chain (V > 2^16); with inv = floor((2^64 -
+// 1) / V) the high half of x * inv is floor(x / V) or one less: x/V - x*inv/2^64
+// = x/2^64 * (2^64/V - inv) < 1, as 2^64/V - inv <= 1.
+struct IdSplit {
+  uint64_t inv;
+  uint32_t V;
+  __host__ explicit IdSplit(uint32_t n) : inv(~0ull / n), V(n) {}
+  IdSplit() = default;
+  __device__ __forceinline__ void split(uint64_t x, uint64_t& u, uint64_t& v) const {
+    u = __umul64hi(x, inv);
+    v = x - u * V;
+    if (v >= V) {
+      u++;
+      v -= V;
+    }
+  }
+  __device__ __forceinline__ bool ordered(uint64_t x) const {
+    uint64_t u, v;
+    split(x, u, v);
+    return u < v;
+  }
+};
+
 struct RecArgs {
   const ulonglong2* sketch;
   const uint64_t* keys;
   uint32_t V, L, C, D, W;
+  IdSplit ids;
   uint32_t *label, *parent, *minv, *rcnt, *roff, *perm, *pcount;
   uint8_t *final_, *merged;
   uint64_t *best0, *best1, *forest, *log_ids;
@@ -36,31 +61,23 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// u < v for an edge id x = u*V + v (32-bit division when x fits 32 bits).
-__device__ __forceinline__ bool edge_id_ordered(uint64_t x, uint32_t V) {
-  if ((x >> 32) == 0) {
-    const uint32_t x32 = (uint32_t)x, u = x32 / V;
-    return u < x32 - u * V;
-  }
-  const uint64_t u = x / V;
-  return u < x - u * V;
-}
-
 // A bucket is good when its alpha is non-zero, its checksum holds and alpha is
 // an edge id u*V+v with u < v. A sum's sample is ZERO if the deterministic
 // bucket is zero, else the first good bucket in index order (deterministic
 // bucket, then column-major), else FAIL.
+__device__ __forceinline__ bool good_bucket(const ulonglong2& x, uint32_t j, uint32_t W, const IdSplit& ids,
+                                            uint64_t kchk) {
+  return j < W && x.x != 0 && mix64(x.x ^ kchk) == x.y && ids.ordered(x.x);
+}
 
 // Whether buckets base + lane + 32q, q < 2, of a warp's sum hold a good one;
 // `edge` is the first one's id, in index order.
-__device__ __forceinline__ bool warp_find(const ulonglong2 (&acc)[2], uint32_t base, uint32_t W, uint32_t V,
+__device__ __forceinline__ bool warp_find(const ulonglong2 (&acc)[2], uint32_t base, uint32_t W, const IdSplit& ids,
                                           uint64_t kchk, uint64_t& edge) {
-  const uint32_t lane = threadIdx.x & 31;
 #pragma unroll
   for (uint32_t q = 0; q < 2; q++) {
-    const bool good = base + lane + 32 * q < W && acc[q].x != 0 && mix64(acc[q].x ^ kchk) == acc[q].y &&
-                      edge_id_ordered(acc[q].x, V);
-    const uint32_t m = __ballot_sync(0xffffffffu, good);
+    const uint32_t m =
+        __ballot_sync(0xffffffffu, good_bucket(acc[q], base + (threadIdx.x & 31) + 32 * q, W, ids, kchk));
     if (m) {
       edge = __shfl_sync(0xffffffffu, acc[q].x, __ffs(m) - 1);
       return true;
@@ -71,10 +88,10 @@ __device__ __forceinline__ bool warp_find(const ulonglong2 (&acc)[2], uint32_t b
 
 // The sample as far as the first kPrefix buckets decide it: 0 ZERO, 1 GOOD,
 // 2 none of them is good.
-__device__ __forceinline__ uint32_t warp_sample_prefix(const ulonglong2 (&acc)[2], uint32_t W, uint32_t V,
-                                                       uint64_t kchk, uint64_t& edge) {
+__device__ __forceinline__ uint32_t warp_sample_prefix(const ulonglong2 (&acc)[2], uint32_t W,
+                                                       const IdSplit& ids, uint64_t kchk, uint64_t& edge) {
   if (__shfl_sync(0xffffffffu, (acc[0].x | acc[0].y) == 0 ? 1u : 0u, 0)) return 0;
-  return warp_find(acc, 0, W, V, kchk, edge) ? 1u : 2u;
+  return warp_find(acc, 0, W, ids, kchk, edge) ? 1u : 2u;
 }
 
 // Buckets base + lane + 32q, q < 2, of one member's row into acc.

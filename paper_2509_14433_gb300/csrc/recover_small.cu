@@ -509,8 +509,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
             uint64_t e = 0;
             uint32_t res = 2;
             if (base == 0)
-              res = warp_sample_prefix(acc, W, V, kchk, e);
-            else if (warp_find(acc, base, W, V, kchk, e))
+              res = warp_sample_prefix(acc, W, a.ids, kchk, e);
+            else if (warp_find(acc, base, W, a.ids, kchk, e))
               res = 1;
             // one of at most 32 members reads on at once
             const bool here = s1 - s0 <= 32;
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
               for (uint32_t b = base + kPrefix; res == 2 && b < W; b += kPrefix) {
                 ulonglong2 more[2] = {make_ulonglong2(0, 0), make_ulonglong2(0, 0)};
                 sum_rows(more, k, 0, s1 - s0, b);
-                if (warp_find(more, b, W, V, kchk, e)) res = 1;
+                if (warp_find(more, b, W, a.ids, kchk, e)) res = 1;
               }
             }
             if (res == 2 && !here && base + kPrefix < W) {
