@@ -108,6 +108,19 @@ __device__ __forceinline__ uint32_t find_root(uint32_t* parent, uint32_t x, uint
   return r;
 }
 
+// The roots of x and y, their walks side by side. Read only: a store to a node
+// near a root, which every walk of a phase passes, makes all of them wait (a
+// relabel of V = 2^14 took 10 to 50 us with find_root, all SMs leaving it at the
+// same moment, against 2).
+__device__ __forceinline__ void walk_roots(const uint32_t* parent, uint32_t& x, uint32_t& y, uint32_t V) {
+  for (uint32_t k = 0; k < V; k++) {
+    const uint32_t p = ld_cg(&parent[x]), q = ld_cg(&parent[y]);
+    if (p == x && q == y) break;
+    x = p;
+    y = q;
+  }
+}
+
 // Book the samples stashed in a warp, one per lane (K = kNoneU32: none):
 // ZERO marks the component final; GOOD with an edge that leaves K becomes
 // its candidate (stored with both endpoint labels) and is logged; GOOD with
@@ -158,16 +171,16 @@ __device__ __forceinline__ void book_samples(const RecArgs& a, uint32_t r, bool 
 __device__ __forceinline__ uint32_t warp_grab(uint32_t* ctr, uint32_t key, bool take) {
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t act = __ballot_sync(0xffffffffu, take);
-  uint32_t pos = 0;
+  uint32_t peers = 0, leader = lane, base = 0;
   if (take) {
-    const uint32_t peers = __match_any_sync(act, key);
-    const uint32_t leader = __ffs(peers) - 1;
-    uint32_t base = 0;
+    peers = __match_any_sync(act, key);
+    leader = __ffs(peers) - 1;
     if (lane == leader) base = atomicAdd(&ctr[key], (uint32_t)__popc(peers));
-    base = __shfl_sync(peers, base, leader);
-    pos = base + __popc(peers & ((1u << lane) - 1));
   }
-  return pos;
+  // one shuffle for all keys (one per key, with its lanes as the mask, would
+  // run them one after another)
+  base = __shfl_sync(0xffffffffu, base, leader);
+  return take ? base + __popc(peers & ((1u << lane) - 1)) : 0;
 }
 
 // Root in a shared-memory forest with path halving; concurrent halving only
@@ -804,22 +817,31 @@ __device__ __forceinline__ bool recover_body(const RecArgs& a) {
       for (uint32_t base = gwarp * 32; base < V; base += nwarps * 32) {
         const uint32_t K = base + lane;
         bool cross = false;
-        uint64_t e = 0;
         uint32_t ra = 0, rb = 0;
+        ulonglong2 c = make_ulonglong2(kNone, 0);
         if (K < V) {
           if (iter == 0) a.rcnt[K] = 0;  // the relabel counts again
-          const ulonglong2 c = __ldcg(&a.cand[K]);
+          c = __ldcg(&a.cand[K]);
           if (c.x != kNone) {
-            e = c.x;
-            ra = find_root(a.parent, (uint32_t)(c.y >> 32), V);
-            rb = find_root(a.parent, (uint32_t)c.y, V);
-            if (ra != rb) {  // read first: most proposals to a big tree's root lose
-              const uint64_t ka = e << vbits | rb, kb = e << vbits | ra;
-              if (ka < ld_cg(&bc[ra])) atomicMin((unsigned long long*)&bc[ra], (unsigned long long)ka);
-              if (kb < ld_cg(&bc[rb])) atomicMin((unsigned long long*)&bc[rb], (unsigned long long)kb);
-              cross = true;
-            }
+            ra = (uint32_t)(c.y >> 32);
+            rb = (uint32_t)c.y;
+            const bool left = ra == K;
+            walk_roots(a.parent, ra, rb, V);
+            // nobody else writes K's word now: the next walks are short
+            const uint32_t root = left ? ra : rb;
+            if (iter && root != K) a.parent[K] = root;
           }
+        }
+        // lanes leave the walk at different steps: together again before the
+        // next loads
+        __syncwarp();
+        const uint64_t e = c.x;
+        if (ra != rb) {  // read first: most proposals to a big tree's root lose
+          const uint64_t ka = e << vbits | rb, kb = e << vbits | ra;
+          const uint64_t ba = ld_cg(&bc[ra]), bb = ld_cg(&bc[rb]);
+          if (ka < ba) atomicMin((unsigned long long*)&bc[ra], (unsigned long long)ka);
+          if (kb < bb) atomicMin((unsigned long long*)&bc[rb], (unsigned long long)kb);
+          cross = true;
         }
         const uint32_t m = __ballot_sync(0xffffffffu, cross);
         if (m) {
@@ -885,10 +907,16 @@ __device__ __forceinline__ bool recover_body(const RecArgs& a) {
         a.cand[w] = make_ulonglong2(kNone, 0);
         a.best0[w] = kNone;
         a.best1[w] = kNone;
-        nl = find_root(a.parent, ld_cg(&a.label[w]), V);
+        nl = ld_cg(&a.label[w]);
+        uint32_t same = nl;
+        walk_roots(a.parent, nl, same, V);
+      }
+      __syncwarp();  // as above
+      if (w < V) {
         a.label[w] = nl;
         live = !ld_cg(&a.final_[nl]);
       }
+      __syncwarp();
       // the member that took position 0 of its component counts the component
       const uint32_t m_first = __ballot_sync(0xffffffffu, warp_grab(a.rcnt, nl, live) == 0 && live);
       if (lane == 0 && m_first) atomicAdd(&gc[GC_NLIVE], (uint32_t)__popc(m_first));
