@@ -8,10 +8,10 @@ records a vertex receives per batch, i.e. on V and the batch size.
 
 tune() times every candidate setting on the device (CUDA events recorded by
 the library around each apply launch) for each batch-size bucket (powers of
-four edges) and keeps the fastest, then times the write-back of single-item
-vertices both ways (load-and-store, XOR atomics) with it and keeps the
-faster; the table is stored as JSON keyed by GPU
-name and graph shape. apply() sets the setting of one batch size as a
+four edges) and keeps the fastest; the table is stored as JSON keyed by GPU
+name and graph shape. Its write-back field is kept for tables that hold it:
+the modes (cupc_set_writeback_bucket) are accepted and timed, but the kernel
+has one write-back, so both read alike. apply() sets the setting of one batch size as a
 graph's default; apply_buckets() gives the graph every bucket's setting, and
 the library then picks one per batch by its size. Run `python -m paper_2509_14433_gb300.autotune --V 16384` on the
 target GPU to (re)write the table; `--batches rmat` times R-MAT batches (the
