@@ -965,7 +965,9 @@ __global__ void k_wait_selftest(uint32_t* gc, uint32_t absent, uint64_t limit_ns
 
 cudaError_t setup_recover(cupc_graph* g) {
   int per_sm = 0;
-  cudaError_t e = cudaFuncSetAttribute(k_recover, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHookBytes);
+  cudaError_t e = setup_recover_cluster(g);
+  if (e != cudaSuccess || g->rec_cluster) return e;  // the grid-wide kernel is not used
+  e = cudaFuncSetAttribute(k_recover, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHookBytes);
   if (e != cudaSuccess) return e;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_recover, kRecThreads, kHookBytes);
   if (e != cudaSuccess) return e;
@@ -979,7 +981,7 @@ cudaError_t setup_recover(cupc_graph* g) {
   const uint32_t want = std::max(16u, (g->V + 127) / 128);
   const uint32_t cap = (uint32_t)(per_sm * g->sms);
   g->rec_grid = (int)(want < cap ? want : cap);
-  return setup_recover_cluster(g);
+  return cudaSuccess;
 }
 
 cudaError_t launch_recover(cupc_graph* g, cudaStream_t s, bool force) {
