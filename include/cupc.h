@@ -316,8 +316,8 @@ cupc_status cupc_selftest_wait_timeout(uint32_t ctas, uint32_t limit_us, int abs
  * search trees on the host; every tree node has an aggregate sketch in
  * device memory. A link or cut changes O(log V) aggregates; the sketch
  * additions it needs are logged and the batch's log is replayed in one
- * launch with one GPU thread per sketch word, each following the whole log
- * for its word (§3.1's parallel execution of the logged additions).
+ * launch, dependent additions in order for every sketch word (§3.1's
+ * parallel execution of the logged additions).
  *
  * The cutset reads g's vertex sketches: after changing them (any update of
  * g), REFRESH every vertex whose sketch changed. g must outlive the cutset.

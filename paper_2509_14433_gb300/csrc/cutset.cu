@@ -1,7 +1,7 @@
 // Parallel cutset (§3.1, Lemma 3.1): the sketch of every tree of a dynamic
 // forest F over the graph's vertex sketches, maintained under link and cut
 // by logging the sketch additions a link or cut needs and replaying the log
-// with one thread per word of a sketch.
+// level by level, 16 words of every sketch to a CTA.
 //
 // The forest is kept as Euler tours (one node per vertex, two arc nodes per
 // forest edge) in randomized search trees ordered by tour position (treaps,
@@ -40,7 +40,7 @@ namespace {
 // (task t, word j) = t * kWords + j, so that a task's words are one 128-byte
 // access. A chain of dependent L2 accesses bounds it: about one per level
 // (some 30) and per kReplayTasks tasks, against one per task when a thread
-// followed the whole log for its word. GB300, V = 1024, 64 cuts: 90 us (270).
+// followed the whole log for its word. GB300, V = 1024, 64 cuts: 28 us (270).
 constexpr uint32_t kWords = 16, kReplayThreads = 1024, kReplayTasks = kReplayThreads / kWords;
 __global__ void __launch_bounds__(kReplayThreads) k_cutset_replay(const int4* __restrict__ tasks,
                                                                   const uint32_t* __restrict__ level, uint32_t nlevels,

@@ -111,7 +111,7 @@ __device__ __forceinline__ uint32_t find_root(uint32_t* parent, uint32_t x, uint
 // The roots of x and y, their walks side by side. Read only: a store to a node
 // near a root, which every walk of a phase passes, makes all of them wait (a
 // relabel of V = 2^14 took 10 to 50 us with find_root, all SMs leaving it at the
-// same moment, against 2).
+// same moment, against 3).
 __device__ __forceinline__ void walk_roots(const uint32_t* parent, uint32_t& x, uint32_t& y, uint32_t V) {
   for (uint32_t k = 0; k < V; k++) {
     const uint32_t p = ld_cg(&parent[x]), q = ld_cg(&parent[y]);
