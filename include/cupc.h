@@ -262,11 +262,12 @@ void cupc_server_destroy(cupc_server* s);
 
 /* Launch tunables of the update's apply kernel (results are identical for
  * every setting; only speed changes): item_records = endpoint records per
- * chunk at most (64..512, 0 = 256), smem_rows = rows per column folded in
- * shared memory, besides the first three, which are folded in registers
- * (1..min(D, 16), 0 = min(D, 8)); deeper rows go straight to HBM),
- * ctas_per_sm = resident CTAs per SM of the persistent grid (0 = as many as
- * fit). CUPC_EINVAL (previous settings kept) when out of range.
+ * chunk at most (64..512, 0 = 256; the kernel takes records in groups of
+ * four, so a setting acts as the multiple of 4 at or below it), smem_rows =
+ * rows per column folded in shared memory, besides the first three, which are
+ * folded in registers (1..min(D, 16), 0 = min(D, 8); deeper rows go straight
+ * to HBM), ctas_per_sm = resident CTAs per SM of the persistent grid (0 = as
+ * many as fit). CUPC_EINVAL (previous settings kept) when out of range.
  * cupc_get_tuning: out4 = {item_records, smem_rows, ctas_per_sm, CTAs per SM
  * in use}. */
 cupc_status cupc_set_tuning(cupc_graph* g, uint32_t item_records, uint32_t smem_rows, uint32_t ctas_per_sm);

@@ -103,8 +103,11 @@ constexpr uint32_t kSmallEdges = 12288;
 // whole number of chunks each, as near as steps of 16 records and the
 // padding, 1.5 records per folded vertex on average, allow); small batches in
 // quarter passes, two for every warp, as the latency of a warp's records is
-// then all that counts.
+// then all that counts. Always a multiple of kPad, whatever `most` is: the
+// apply kernel folds kPad records at a time and no chunk may split a group.
 inline uint32_t chunk_records(uint32_t nrec, uint32_t V, uint32_t warps, uint32_t most) {
+  static_assert(kStage / 4 % kPad == 0 && 16 % kPad == 0 && kMinItemRecords >= kPad, "chunks are whole groups");
+  most = most / kPad * kPad;
   warps = std::max(1u, warps);
   const uint64_t all = (uint64_t)nrec + 3ull * std::min(V, nrec / 3) / 2;
   const uint32_t per = (uint32_t)(all / warps) + 1;
