@@ -45,11 +45,9 @@ Dims derive(uint32_t V, const cupc_params* p) {
   uint32_t P = 1;  // apply threads per layer: the columns and the checksum lane
   while (P < d.C + 1) P <<= 1;
   if (d.L * P > 1024) return d;  // one apply CTA holds every (layer, lane)
-  // the edge index u*V+v must fit the 64-bit bucket word; record offsets are
-  // u32, the padding of the record array included: a longer batch is applied
-  // in chunks
+  // the edge index u*V+v must fit the 64-bit bucket word; staging offsets of
+  // a batch are u32
   if ((uint64_t)d.max_batch * 2 >= 0xFFFFFFFFull) return d;
-  d.max_batch = std::min(d.max_batch, kMaxChunkEdges);
   d.ok = true;
   return d;
 }
@@ -85,7 +83,7 @@ Layout layout(const Dims& d) {
   l.gc = take(GC_SLOTS * sizeof(uint32_t));
   l.cnt = take(count_shards(d) * V * 4);
   l.cursor = take(count_shards(d) * V * 4);
-  l.rec = take(rec_entries(V, B) * 8);
+  l.rec = take(rec_entries(V, chunk_edges(d.max_batch)) * 8);
   l.work = take(kWorkSlots * 4);
   l.stage_edges = take(2 * B * 4);
   l.stage_ops = take(B);
@@ -191,6 +189,7 @@ cupc_status cupc_init(uint32_t V, uint64_t seed, const cupc_params* params, void
   g->seed = seed;
   g->max_batch = d.max_batch;
   g->max_pairs = d.max_pairs;
+  g->max_chunk = chunk_edges(d.max_batch);
   g->ws_bytes = l.total;
   g->owns_ws = workspace == nullptr;
   g->last_recovery = CUPC_OK;
@@ -220,7 +219,7 @@ cupc_status cupc_init(uint32_t V, uint64_t seed, const cupc_params* params, void
   g->cnt = (uint32_t*)(b + l.cnt);
   g->cursor = (uint32_t*)(b + l.cursor);
   g->rec = (uint64_t*)(b + l.rec);
-  g->rec_cap = (uint32_t)rec_entries(d.V, d.max_batch);
+  g->rec_cap = (uint32_t)rec_entries(d.V, g->max_chunk);
   g->work = (uint32_t*)(b + l.work);
   g->stage_edges = (uint32_t*)(b + l.stage_edges);
   g->stage_ops = (int8_t*)(b + l.stage_ops);
@@ -304,16 +303,11 @@ cupc_status cupc_update_batch(cupc_graph* g, const uint32_t* edges, const int8_t
   const size_t B = g->max_batch;
   const bool dev_e = is_device_ptr(edges), dev_o = is_device_ptr(ops);
   if (dev_e && dev_o) {
-    if (n <= B) {
-      CUPC_TRY(launch_update_chunk(g, edges, n, s, ops));  // validated on the way
-    } else {
-      CUPC_TRY(launch_validate(g, edges, ops, n, s));
-      for (size_t i = 0; i < n; i += B) CUPC_TRY(launch_update_chunk(g, edges + 2 * i, (n - i < B ? n - i : B), s));
-    }
+    CUPC_TRY(launch_update(g, edges, n, s, ops));
     if (g->inc) CUPC_TRY(launch_incremental(g, edges, ops, n, s));
     return mark_updated(g, s, true);
   } else if (!dev_e && !dev_o && n <= B) {
-    // host input, one chunk: copy on the graph's copy stream into the
+    // host input that the staging holds: copy on the graph's copy stream into the
     // staging slot not used last, so that the copy overlaps the kernels of
     // the previous batch; the copy waits only for its slot to be free
     CUPC_TRY(ensure_copy_stream(g));
@@ -326,14 +320,14 @@ cupc_status cupc_update_batch(cupc_graph* g, const uint32_t* edges, const int8_t
     CUPC_TRY(cudaMemcpyAsync(so, ops, n, cudaMemcpyHostToDevice, g->copy_stream));
     CUPC_TRY(cudaEventRecord(g->slot_ready[k], g->copy_stream));
     CUPC_TRY(cudaStreamWaitEvent(s, g->slot_ready[k], 0));
-    CUPC_TRY(launch_update_chunk(g, se, n, s, so));
+    CUPC_TRY(launch_update(g, se, n, s, so));
     if (g->inc) CUPC_TRY(launch_incremental(g, se, so, n, s));
     CUPC_TRY(mark_slot_free(g, k, s));
     return mark_updated(g, s, true);
   } else {
-    // a host input mixed with a device one, or several chunks: stage in
-    // slot 0 on the caller's stream; a multi-chunk batch is validated in
-    // a first pass so that a bad entry drops the whole batch
+    // a host input mixed with a device one, or more than the staging holds:
+    // stage in slot 0 on the caller's stream; a batch staged in parts is
+    // validated in a first pass so that a bad entry drops the whole batch
     auto stage = [&](size_t i, size_t k) -> cudaError_t {
       cudaError_t e = cudaMemcpyAsync(g->stage_edges, edges + 2 * i, 2 * k * sizeof(uint32_t),
                                       dev_e ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
@@ -343,7 +337,7 @@ cupc_status cupc_update_batch(cupc_graph* g, const uint32_t* edges, const int8_t
     };
     if (n <= B) {
       CUPC_TRY(stage(0, n));
-      CUPC_TRY(launch_update_chunk(g, g->stage_edges, n, s, g->stage_ops));
+      CUPC_TRY(launch_update(g, g->stage_edges, n, s, g->stage_ops));
     } else {
       for (size_t i = 0; i < n; i += B) {
         size_t k = n - i < B ? n - i : B;
@@ -353,7 +347,7 @@ cupc_status cupc_update_batch(cupc_graph* g, const uint32_t* edges, const int8_t
       for (size_t i = 0; i < n; i += B) {
         size_t k = n - i < B ? n - i : B;
         CUPC_TRY(stage(i, k));
-        CUPC_TRY(launch_update_chunk(g, g->stage_edges, k, s));
+        CUPC_TRY(launch_update(g, g->stage_edges, k, s, nullptr));
       }
     }
     CUPC_TRY(mark_slot_free(g, 0, s));

@@ -357,9 +357,13 @@ cupc_status cupc_batcher_update(cupc_batcher* b, cupc_graph* const* graphs, cons
   InstDesc* d = reinterpret_cast<InstDesc*>(h + 1);
   uint64_t base = 0, units = 0, work = 0, records = 0, vertices = 0;
   uint32_t slices = 0, warp_bytes = 0;
+  // a batch longer than one chunk gets its graph's own launch sequence, and
+  // none of the joined one
+  auto joined = [&](uint32_t i) { return n[i] <= graphs[i]->max_chunk ? (uint32_t)n[i] : 0u; };
   for (uint32_t i = 0; i < k; i++) {
-    work += 2 * (uint64_t)n[i] * layer_groups(graphs[i]->L, graphs[i]->P);
-    records += 2 * (uint64_t)n[i];
+    if (n[i] && !joined(i) && launch_update(graphs[i], edges[i], n[i], s, ops[i]) != cudaSuccess) return CUPC_ECUDA;
+    work += 2 * (uint64_t)joined(i) * layer_groups(graphs[i]->L, graphs[i]->P);
+    records += 2 * (uint64_t)joined(i);
     vertices += graphs[i]->V;
   }
   // records per chunk: about three units for each warp of a full device, but
@@ -383,7 +387,7 @@ cupc_status cupc_batcher_update(cupc_batcher* b, cupc_graph* const* graphs, cons
     x.work = g->work;
     x.gc = g->gc;
     x.edge_base = base;
-    x.n = (uint32_t)n[i];
+    x.n = joined(i);
     x.V = g->V;
     x.L = g->L;
     x.C = g->C;
@@ -396,9 +400,9 @@ cupc_status cupc_batcher_update(cupc_batcher* b, cupc_graph* const* graphs, cons
     x.chunk = chunk;
     x.cap = g->rec_cap;
     x.slice_base = slices;
-    base += n[i];
-    if (n[i]) slices += plan_slices(g->V);
-    units += (uint64_t)layer_groups(g->L, g->P) * (rec_entries(g->V, n[i]) / chunk + 2);
+    base += x.n;
+    if (x.n) slices += plan_slices(g->V);
+    units += (uint64_t)layer_groups(g->L, g->P) * (rec_entries(g->V, x.n) / chunk + 2);
     warp_bytes = std::max(warp_bytes, apply_warp_bytes(x.R, x.P));
   }
   if (units >= 0xFFFFFFFFull) return CUPC_EINVAL;

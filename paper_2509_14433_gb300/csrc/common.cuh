@@ -67,8 +67,11 @@ constexpr uint32_t kPad = 4;
 __host__ __device__ constexpr size_t rec_entries(size_t V, size_t n) {
   return 2 * n + (kPad - 1) * (V < 2 * n / 3 ? V : 2 * n / 3);
 }
-// Most edges of one update chunk: its record offsets fit 32 bits.
+// Most edges of one update chunk: its record offsets fit 32 bits. A graph's
+// max_batch may be larger (up to 2^31 - 1): its staging holds that many, and
+// launch_update splits such a batch.
 constexpr uint32_t kMaxChunkEdges = (1u << 31) - (1u << 22);
+inline uint32_t chunk_edges(uint32_t max_batch) { return std::min(max_batch, kMaxChunkEdges); }
 static_assert(rec_entries(kMaxVertices, kMaxChunkEdges) < 0xFFFFFFFFull - 4096, "record offsets fit 32 bits");
 // Records an apply warp stages per pass (one per lane), and the distance of
 // two layers' checksums of a pass.
@@ -219,7 +222,8 @@ struct cupc_graph {
   uint32_t V, L, C, D, W, P, R;  // P: lanes per layer in the update kernel
   uint32_t ell;                  // bits of one column-hash stage (hash_bits(V))
   uint64_t seed;
-  uint32_t max_batch, max_pairs;
+  uint32_t max_batch, max_pairs;  // edges, pairs the staging holds
+  uint32_t max_chunk;             // edges of one update chunk: chunk_edges(max_batch)
   void* ws;
   size_t ws_bytes;
   bool owns_ws;
@@ -340,6 +344,9 @@ cudaError_t launch_keys(cupc_graph* g, cudaStream_t s);
 // caller has validated the whole batch first.
 cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, cudaStream_t s,
                                 const int8_t* validate_ops = nullptr);
+// A device batch of any length, in chunks of at most g->max_chunk edges; ops:
+// also validate the batch as a whole.
+cudaError_t launch_update(cupc_graph* g, const uint32_t* edges, size_t n, cudaStream_t s, const int8_t* ops);
 cudaError_t launch_validate(cupc_graph* g, const uint32_t* edges, const int8_t* ops, size_t n, cudaStream_t s);
 cudaError_t setup_update(cupc_graph* g);
 cudaError_t configure_apply(cupc_graph* g);

@@ -123,6 +123,7 @@ extern "C" cupc_status cupc_update_sketch_static(void* sketch, uint32_t V, uint6
   fill_dims(g, V);
   g.seed = seed;
   g.max_batch = kMaxEdges;
+  g.max_chunk = chunk_edges(kMaxEdges);
   g.sms = ds->sms;
   g.P = ds->P;
   g.R = g.D < kSmemRows ? g.D : kSmemRows;

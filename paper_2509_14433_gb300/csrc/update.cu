@@ -2,7 +2,7 @@
 // Algorithm": an update of edge (u,v) updates every sketch of u and of v;
 // Theorem A.2: CameoSketch touches one bucket per column per update).
 //
-// One chunk of <= max_batch edges goes through four stream-ordered kernels (a
+// One chunk of <= max_chunk edges goes through four stream-ordered kernels (a
 // batch of several chunks is validated whole by k_validate first, a batch of
 // one chunk inside the count):
 //   k_count   per-vertex record counts (2 records per edge, one per
@@ -551,6 +551,14 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
   kern<<<agrid, 32 * kApplyWarps, smem, s>>>(g->sketch, g->keys, g->rec, g->rec_cap, chunk, g->work, g->gc, g->V,
                                              g->L, g->C, g->D, g->W, g->P, fold_rows(R, g->D), g->ell);
   return cudaGetLastError();
+}
+
+cudaError_t launch_update(cupc_graph* g, const uint32_t* edges, size_t n, cudaStream_t s, const int8_t* ops) {
+  if (n <= g->max_chunk) return launch_update_chunk(g, edges, n, s, ops);  // validated on the way
+  cudaError_t e = ops ? launch_validate(g, edges, ops, n, s) : cudaSuccess;
+  for (size_t i = 0; e == cudaSuccess && i < n; i += g->max_chunk)
+    e = launch_update_chunk(g, edges + 2 * i, std::min<size_t>(n - i, g->max_chunk), s);
+  return e;
 }
 
 }  // namespace cupc

@@ -34,3 +34,27 @@ def test_every_accepted_setting_gives_chunks_of_whole_groups(tmp_path, V):
       }}
   printf("%llu %d", bad, most_used > 1000);""")
     assert out.split() == ["0", "1"]
+
+
+def test_staging_holds_as_much_as_max_batch_says():
+    # host batches and host pairs are staged max_batch at a time in two slots
+    # of 8 bytes an edge and 1 an op, up to the largest max_batch there is
+    from paper_2509_14433_gb300 import cupc as C
+    top, less = (1 << 31) - 1, (1 << 31) - (1 << 23)
+    for V in (2, 1000, 1 << 21):
+        rows = 8 if V > 1000 else 0
+        size = {B: C.cupc_workspace_bytes(V, (0, 0, rows, B)) for B in (less, top)}
+        assert size[top] - size[less] >= 2 * 9 * (top - less) - 4 * 256
+        assert C.cupc_workspace_bytes(V, (0, 0, rows, top + 1)) == 0
+
+
+def test_record_offsets_of_the_longest_chunk_fit_32_bits(tmp_path):
+    out = _run(tmp_path, """
+  int ok = 1;
+  for (uint64_t B = 1; B < (1ull << 31); B = B * 2 + 1)
+    for (uint64_t V = 2; V <= kMaxVertices; V *= 2) {
+      const uint32_t n = chunk_edges((uint32_t)B);
+      ok &= n > 0 && n <= B && (n == B || n == kMaxChunkEdges) && rec_entries(V, n) < 0xFFFFFFFFull - 4096;
+    }
+  printf("%d", ok);""")
+    assert out == "1"
