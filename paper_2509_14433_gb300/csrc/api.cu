@@ -414,9 +414,14 @@ cupc_status cupc_spanning_forest(cupc_graph* g, uint64_t* edge_ids_out, size_t c
   }
   g->forest_stale = false;
   CUPC_TRY(launch_forest_sort(g, s));
-  // into device memory the ids go at once, behind one synchronisation; into
-  // host memory once their number is known
-  const bool direct = edge_ids_out && (uintptr_t)edge_ids_out % 8 == 0 && is_device_ptr(edge_ids_out);
+  // into the graph's device's memory the ids go at once, behind one
+  // synchronisation; elsewhere once their number is known
+  cudaPointerAttributes at{};
+  if (edge_ids_out && cudaPointerGetAttributes(&at, edge_ids_out) != cudaSuccess) {
+    cudaGetLastError();
+    at = cudaPointerAttributes{};
+  }
+  const bool direct = stores_directly(at, edge_ids_out, g->device);
   if (direct) CUPC_TRY(launch_copy_forest(g, edge_ids_out, cap, s));
   uint32_t h[GC_SLOTS];
   CUPC_TRY(cudaMemcpyAsync(h, g->gc, sizeof(h), cudaMemcpyDeviceToHost, s));

@@ -338,6 +338,14 @@ struct ProfScope {
 }  // namespace cupc
 
 namespace cupc {
+// Whether a kernel of `device` may store 64-bit words at p: memory that lives
+// on that device. What lives on another GPU needs peer access, which the
+// runtime's copies do not.
+inline bool stores_directly(const cudaPointerAttributes& at, const void* p, int device) {
+  return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) && at.device == device &&
+         (uintptr_t)p % 8 == 0;
+}
+
 // Launchers (defined in update.cu / recover.cu); all stream-ordered.
 cudaError_t launch_keys(cupc_graph* g, cudaStream_t s);
 // validate_ops: also validate this chunk (a batch of one chunk), else the

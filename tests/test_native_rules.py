@@ -58,3 +58,21 @@ def test_record_offsets_of_the_longest_chunk_fit_32_bits(tmp_path):
     }
   printf("%d", ok);""")
     assert out == "1"
+
+
+def test_which_memory_a_kernel_stores_the_forest_to(tmp_path):
+    # only the graph's own device's memory, aligned; the default attributes
+    # (unregistered) are those of plain host memory and of a null pointer
+    out = _run(tmp_path, """
+  const cudaMemoryType types[4] = {cudaMemoryTypeUnregistered, cudaMemoryTypeHost, cudaMemoryTypeDevice,
+                                   cudaMemoryTypeManaged};
+  for (int t = 0; t < 4; t++)
+    for (int dev = 0; dev < 2; dev++)
+      for (uintptr_t off : {0, 4, 8}) {
+        cudaPointerAttributes at{};
+        at.type = types[t];
+        at.device = dev;
+        printf("%d", stores_directly(at, (void*)(0x1000 + off), 1));
+      }
+  printf(" %d", stores_directly(cudaPointerAttributes{}, nullptr, 0));""")
+    assert out == "000000" * 2 + "000101" * 2 + " 0"
