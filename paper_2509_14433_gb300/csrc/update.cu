@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(1024) k_count_priv(const uint32_t* __restrict_
                                                      const int8_t* __restrict__ ops, size_t n, uint32_t V,
                                                      uint32_t* cnt, uint32_t* work, uint32_t* gc) {
   extern __shared__ uint32_t s_h[];  // V
-  if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
+  // another CTA may set the error meanwhile: the threads of a CTA, which meet
+  // at barriers below, must agree on what they read
+  if (__syncthreads_or(ld_cg(&gc[GC_ERR]) & kErrInval)) return;
   reset_work(work);
   for (uint32_t w = threadIdx.x; w < V; w += blockDim.x) s_h[w] = 0;
   __syncthreads();

@@ -105,3 +105,24 @@ def test_a_sharded_count_with_hubs():
         assert dev.update(bad) == 0 and dev.sync() != 0  # its counts are cleared
     assert dev.sync() == 0
     assert np.array_equal(dev.export(), ref.export())
+
+
+@pytest.mark.parametrize("V,n", [(1024, 60000), (24576, 1 << 20)])
+def test_invalid_edges_all_over_a_shared_histogram_batch(V, n):
+    # every CTA meets bad edges while others start: the batch is dropped whole,
+    # its counts are cleared and the next batch applies
+    from paper_2509_14433_gb300 import cupc as B
+    from tests._dev import Dev
+
+    L, C, D = 3, 2, 6
+    dev, ref = Dev(V, 6, (L, C, D, 0)), O.Graph(V, 6, L, C, D)
+    g = WL.rng(V)
+    e = WL.uniform_pairs(V, n, g)
+    bad = e.copy()
+    bad[::97, 1] = V + 5
+    for part in (bad, e, bad[::-1], bad):
+        if part is e:
+            assert dev.update(e) == 0 and ref.update(e) == O.OK and dev.sync() == 0
+        else:
+            assert dev.update(part) == 0 and dev.sync() == B.CUPC_EINVAL
+    assert np.array_equal(dev.export(), ref.export())
