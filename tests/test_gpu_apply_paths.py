@@ -126,3 +126,30 @@ def test_invalid_edges_all_over_a_shared_histogram_batch(V, n):
         else:
             assert dev.update(part) == 0 and dev.sync() == B.CUPC_EINVAL
     assert np.array_equal(dev.export(), ref.export())
+
+
+def _b_words(seed, L, C):
+    """The addends b of the columns: words L*(C+1) + 3k of the key stream."""
+    j = np.uint64(L * (C + 1)) + np.uint64(3) * np.arange(L * C, dtype=np.uint64)
+    with np.errstate(over="ignore"):
+        z = np.uint64(seed) + np.uint64(0x9E3779B97F4A7C15) * (j + np.uint64(1))
+        z = (z ^ (z >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+        z = (z ^ (z >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+    return z ^ (z >> np.uint64(31))
+
+
+@pytest.mark.parametrize("zeros", [3, 5, 11, 14])
+def test_padding_in_columns_whose_hash_of_zero_is_deep(zeros):
+    # padding records have the id zero, whose depth in a column is the leading
+    # zeros of its b: below, inside and beyond the shared rows
+    from tests._dev import Dev
+
+    V, L, C, D = 900, 6, 7, 20
+    seed = next(s for s in range(1, 1 << 20)
+                if ((_b_words(s, L, C) >> np.uint64(63 - zeros)) == 1).any())
+    dev, ref = Dev(V, seed, (L, C, D, 0)), O.Graph(V, seed, L, C, D)
+    g = WL.rng(zeros)
+    e = np.concatenate([_stars(V, (3, 5, 6, 7, 9, 33, 401), g), WL.uniform_pairs(V, 13000, g)])
+    assert dev.update(e) == 0 and ref.update(e) == O.OK
+    assert dev.sync() == 0
+    assert np.array_equal(dev.export(), ref.export())
