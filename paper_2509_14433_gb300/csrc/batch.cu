@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_m(const BatchHead* __rest
   for (uint32_t x = blockIdx.x; x < h->total_slices; x += gridDim.x) {
     const InstDesc& g = d[inst_of<false>(d, k, x)];
     const bool dropped = (ld_cg(&g.gc[GC_ERR]) & kErrInval) != 0;
-    plan_slice(g.cnt, g.cursor, g.rec, g.V, g.cap, x - g.slice_base, g.work, dropped, 1u);
+    plan_slice(g.cnt, g.cursor, g.rec, g.V, g.cap, x - g.slice_base, g.work, dropped, 1u, kNoneU32);
     if (!dropped && g.n > 0 && x == g.slice_base && threadIdx.x == 0) g.gc[GC_BATCHES] += 1;
   }
 }
@@ -128,7 +128,7 @@ __device__ __forceinline__ void number_units(BatchHead* h) {
     const uint32_t j = j0 + threadIdx.x;
     uint32_t nchunks = 0, units = 0;
     if (j < k && d[j].n && !(ld_cg(&d[j].gc[GC_ERR]) & kErrInval)) {
-      nchunks = chunk_plan(d[j].work, d[j].chunk).total;
+      nchunks = chunk_plan(d[j].work, d[j].chunk, d[j].chunk).total;
       units = nchunks * layer_groups(d[j].L, d[j].P);
     }
     uint64_t total;
@@ -170,7 +170,7 @@ __device__ __forceinline__ Unit unit_at(const InstDesc* d, uint32_t k, uint32_t 
   const InstDesc& g = d[u.j];
   const uint32_t at = x - g.unit_base;
   u.group = at / g.nchunks;
-  u.c = chunk_at(chunk_plan(g.work, g.chunk), at % g.nchunks, g.chunk, g.rec, g.cap);
+  u.c = chunk_at(chunk_plan(g.work, g.chunk, g.chunk), at % g.nchunks, g.rec, g.cap);
   return u;
 }
 

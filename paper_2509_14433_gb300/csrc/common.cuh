@@ -55,10 +55,10 @@ constexpr uint32_t kShardEdges = 1u << 20;
 constexpr uint32_t kPlanSlice = 1024;
 constexpr uint32_t kPlanThreads = 256;
 inline uint32_t plan_slices(uint32_t V) { return (V + kPlanSlice - 1) / kPlanSlice; }
-// Counters of one update chunk: the plan's fold and direct records, and the
-// apply kernel's next chunk of records for each layer group (at most 32,
-// since L*P <= 1024).
-constexpr uint32_t kWorkFold = 0, kWorkDirect = 1, kWorkNext = 32, kWorkSlots = 64;
+// Counters of one update chunk: the plan's fold and direct records and those of
+// hubs, and the apply kernel's next chunk of records for each layer group (at
+// most 32, since L*P <= 1024).
+constexpr uint32_t kWorkFold = 0, kWorkDirect = 1, kWorkHub = 2, kWorkNext = 32, kWorkSlots = 64;
 // A vertex of more than two records starts at, and is padded to, a multiple
 // of kPad records.
 constexpr uint32_t kPad = 4;
@@ -118,6 +118,23 @@ inline uint32_t chunk_records(uint32_t nrec, uint32_t V, uint32_t warps, uint32_
   const uint32_t rounds = (per + most - 1) / most;
   return std::min(most, (per / rounds + 16) / 16 * 16);
 }
+// The same for a batch whose hubs hold more than an eighth of its records: a
+// chunk of a hub's records takes one flush, one of many small vertices a flush
+// for each, so equal chunks, one or two a warp, end far apart. Four or five
+// each, of 32 to 160 records. Used on graphs of at most kPrivMaxV vertices that
+// get kHubMean records or more on average; elsewhere smaller chunks lose more to
+// their flushes than they balance. GB300, us, R-MAT batches (chunk_records
+// alone): V = 2048, 80000 edges 67 (73); V = 4096, 60000 and 280000 edges 77, 149
+// (85, 162); V = 8192, 160000 and 280000 edges 142, 170 (150, 183); the other way
+// V = 16384, 200000 edges 202 (198).
+constexpr uint32_t kHubMean = 24;
+inline uint32_t hub_chunk_records(uint32_t nrec, uint32_t warps, uint32_t most) {
+  const uint32_t per = nrec / std::max(1u, warps) + 1, up = (per / 5 + 15) / 16 * 16;
+  const uint32_t least = std::min(2 * kStage, std::max(kStage, (per / 4 + 15) / 16 * 16));
+  return std::min(most / kPad * kPad, std::min(5 * kStage, std::max(up, least)));
+}
+// A vertex of more records than this is a hub of its batch: four times the mean.
+inline uint32_t hub_records(uint32_t nrec, uint32_t V) { return 4 * (nrec / V) + 8; }
 // Key words of a graph: L*(C+1) (column multipliers and layer checksum
 // keys) + 3*L*C (the other multiply-add-shift words of every column).
 constexpr size_t key_words(uint32_t L, uint32_t C) { return (size_t)L * (C + 1) + (size_t)3 * L * C; }

@@ -338,10 +338,10 @@ cudaError_t launch_incremental(cupc_graph* g, const uint32_t* edges, const int8_
 
 // The work plan of one chunk (plan_slice), one CTA per slice of vertices.
 __global__ void __launch_bounds__(kPlanThreads) k_plan(uint32_t* cnt, uint32_t* cursor, uint64_t* rec, uint32_t V,
-                                                       uint32_t cap, uint32_t shards, uint32_t* work,
-                                                       uint32_t* gc) {
+                                                       uint32_t cap, uint32_t shards, uint32_t hub,
+                                                       uint32_t* work, uint32_t* gc) {
   const bool dropped = (ld_cg(&gc[GC_ERR]) & kErrInval) != 0;  // a dropped batch may have counted: start clean
-  plan_slice(cnt, cursor, rec, V, cap, blockIdx.x, work, dropped, shards);
+  plan_slice(cnt, cursor, rec, V, cap, blockIdx.x, work, dropped, shards, hub);
   if (!dropped && blockIdx.x == 0 && threadIdx.x == 0) gc[GC_BATCHES] += 1;
 }
 
@@ -358,7 +358,8 @@ __global__ void k_scatter(const uint32_t* __restrict__ edges, size_t n, uint32_t
   }
 }
 
-// Apply the records, in chunks of `chunk` records (apply_chunk). A warp keeps
+// Apply the records, in chunks of `chunk` records, or `hub_chunk` if hubs hold
+// more than an eighth of them (apply_chunk). A warp keeps
 // the layer group (its number modulo the groups). Its first two chunks are
 // given, the others come from the group's counter, asked for two chunks
 // ahead, so that the next chunk's records load while it works on this one.
@@ -377,14 +378,14 @@ __global__ void k_scatter(const uint32_t* __restrict__ edges, size_t n, uint32_t
 template <bool kX32>
 __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply(
     ulonglong2* __restrict__ sketch, const uint64_t* __restrict__ keys, const uint64_t* __restrict__ rec, uint32_t cap,
-    uint32_t chunk, uint32_t* work, const uint32_t* gc, uint32_t V, uint32_t L, uint32_t C, uint32_t D, uint32_t W,
+    uint32_t chunk, uint32_t hub_chunk, uint32_t* work, const uint32_t* gc, uint32_t V, uint32_t L, uint32_t C, uint32_t D, uint32_t W,
     uint32_t P, uint32_t R, uint32_t ell) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
   const uint32_t nslots = apply_slots(R);
   const uint32_t gw = blockIdx.x * kApplyWarps + (threadIdx.x >> 5), groups = layer_groups(L, P);
   const uint32_t group = gw % groups, warps = (gridDim.x * kApplyWarps - group + groups - 1) / groups;
-  const ChunkPlan c = chunk_plan(work, chunk);
+  const ChunkPlan c = chunk_plan(work, chunk, hub_chunk);
   uint32_t q = gw / groups;
   if (q >= c.total) return;
   const ApplySmem m = apply_smem(smem_raw + (threadIdx.x >> 5) * apply_warp_bytes(R, P), nslots, P);
@@ -394,11 +395,11 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply(
   clear_sums(a);
   a.dirty = 0;
   bool pending = false;
-  Chunk k = chunk_at(c, q, chunk, rec, cap);
+  Chunk k = chunk_at(c, q, rec, cap);
   uint64_t r = load_record(k, 0, k);
   q += warps;
   while (k.n) {
-    const Chunk next = chunk_at(c, q, chunk, rec, cap);
+    const Chunk next = chunk_at(c, q, rec, cap);
     uint32_t ahead = q;
     if ((threadIdx.x & 31) == 0 && next.n) ahead = 2 * warps + atomicAdd(&work[kWorkNext + group], 1u);
     apply_chunk<kX32>(l, m, a, pending, k, next, r, V, W, C, P, R);
@@ -530,14 +531,15 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
   const bool priv = g->V <= kPrivMaxV && pgrid >= (int)kPrivMinCtas;
   const uint32_t shards = !priv && n >= kShardEdges ? g->shards : 1u;
   const uint32_t nrec = (uint32_t)(2 * n);
+  const bool hubs = g->V <= kPrivMaxV && nrec / g->V >= kHubMean;  // hub_chunk_records
   {
     ProfScope ps(g, s, PC_GROUP, 3);
     if (priv)
       k_count_priv<<<pgrid, 1024, 4 * g->V, s>>>(edges, validate_ops, n, g->V, g->cnt, g->work, g->gc);
     else
       k_count<<<grid, 256, 0, s>>>(edges, validate_ops, n, g->V, g->cnt, shards, g->work, g->gc);
-    k_plan<<<plan_slices(g->V), kPlanThreads, 0, s>>>(g->cnt, g->cursor, g->rec, g->V, g->rec_cap, shards, g->work,
-                                                       g->gc);
+    k_plan<<<plan_slices(g->V), kPlanThreads, 0, s>>>(g->cnt, g->cursor, g->rec, g->V, g->rec_cap, shards,
+                                                       hubs ? hub_records(nrec, g->V) : kNoneU32, g->work, g->gc);
     if (priv)
       k_scatter_priv<<<pgrid, 1024, 8 * g->V, s>>>(edges, n, g->V, g->cursor, g->rec, g->gc);
     else
@@ -545,13 +547,15 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
   }
   ProfScope ps(g, s, PC_APPLY, 1);
   const uint32_t groups = layer_groups(g->L, g->P);
-  const uint32_t chunk = chunk_records(nrec, g->V, (uint32_t)grid_max * kApplyWarps / groups, ir);
+  const uint32_t warps = (uint32_t)grid_max * kApplyWarps / groups;
+  const uint32_t chunk = chunk_records(nrec, g->V, warps, ir);
+  const uint32_t hub_chunk = hubs ? hub_chunk_records(nrec, warps, ir) : chunk;
   // at most: chunks of padded fold records and of direct records
-  const size_t units = (size_t)(rec_entries(g->V, n) / chunk + 2) * groups;
+  const size_t units = (size_t)(rec_entries(g->V, n) / std::min(chunk, hub_chunk) + 2) * groups;
   const int agrid = (int)std::min<size_t>((size_t)grid_max, (units + kApplyWarps - 1) / kApplyWarps);
   auto kern = small_ids(g->V) ? k_apply<true> : k_apply<false>;
-  kern<<<agrid, 32 * kApplyWarps, smem, s>>>(g->sketch, g->keys, g->rec, g->rec_cap, chunk, g->work, g->gc, g->V,
-                                             g->L, g->C, g->D, g->W, g->P, fold_rows(R, g->D), g->ell);
+  kern<<<agrid, 32 * kApplyWarps, smem, s>>>(g->sketch, g->keys, g->rec, g->rec_cap, chunk, hub_chunk, g->work, g->gc,
+                                             g->V, g->L, g->C, g->D, g->W, g->P, fold_rows(R, g->D), g->ell);
   return cudaGetLastError();
 }
 

@@ -57,19 +57,23 @@ __device__ __forceinline__ uint64_t block_scan(uint64_t v, uint64_t* total) {
 // slices need not wait on one another; their order in the array does not
 // matter, because the apply kernel reads each record's vertex from the
 // record itself. Counts come in `shards` arrays of V; a vertex's segment is
-// divided among them, cursor[k*V + w] = the start of shard k's records.
+// divided among them, cursor[k*V + w] = the start of shard k's records. The
+// records of vertices with more than `hub` are counted.
 __device__ __forceinline__ void plan_slice(uint32_t* cnt, uint32_t* cursor, uint64_t* rec, uint32_t V, uint32_t cap,
-                                           uint32_t slice, uint32_t* work, bool dropped, uint32_t shards) {
+                                           uint32_t slice, uint32_t* work, bool dropped, uint32_t shards,
+                                           uint32_t hub) {
   __shared__ uint32_t s_base[2];
   constexpr uint32_t kPer = kPlanSlice / kPlanThreads;
   const uint32_t w0 = slice * kPlanSlice + kPer * threadIdx.x;
   uint32_t c[kPer];
   uint64_t sum = 0;  // direct records << 32 | padded fold records
+  uint32_t nhub = 0;
 #pragma unroll
   for (uint32_t k = 0; k < kPer; k++) {
     c[k] = 0;
     for (uint32_t q = 0; q < shards && w0 + k < V; q++) c[k] += cnt[(size_t)q * V + w0 + k];
     sum += c[k] <= kDirectMax ? (uint64_t)c[k] << 32 : (uint64_t)((c[k] + kPad - 1) / kPad * kPad);
+    if (c[k] > hub) nhub += c[k];
   }
   if (dropped) {
     for (uint32_t q = 0; q < shards; q++)
@@ -77,6 +81,8 @@ __device__ __forceinline__ void plan_slice(uint32_t* cnt, uint32_t* cursor, uint
         if (w0 + k < V) cnt[(size_t)q * V + w0 + k] = 0;
     return;
   }
+  nhub = __reduce_add_sync(0xffffffffu, nhub);
+  if (nhub && (threadIdx.x & 31) == 0) atomicAdd(&work[kWorkHub], nhub);
   uint64_t total;
   const uint64_t before = block_scan(sum, &total);
   if (threadIdx.x < 2) {
@@ -427,22 +433,24 @@ struct Chunk {
   bool fold;
 };
 struct ChunkPlan {
-  uint32_t nfold, ndirect, nf, total;  // records; fold chunks, chunks
+  uint32_t nfold, ndirect, chunk, nf, total;  // records; of a chunk; fold chunks, chunks
 };
-__device__ __forceinline__ ChunkPlan chunk_plan(const uint32_t* work, uint32_t chunk) {
+// hub_chunk: the chunk size if hubs hold more than an eighth of the records.
+__device__ __forceinline__ ChunkPlan chunk_plan(const uint32_t* work, uint32_t chunk, uint32_t hub_chunk) {
   ChunkPlan c;
   c.nfold = ld_cg(&work[kWorkFold]);
   c.ndirect = ld_cg(&work[kWorkDirect]);
-  c.nf = (c.nfold + chunk - 1) / chunk;
-  c.total = c.nf + (c.ndirect + chunk - 1) / chunk;
+  c.chunk = chunk;
+  if (hub_chunk != chunk && ld_cg(&work[kWorkHub]) > (c.nfold + c.ndirect) / 8) c.chunk = hub_chunk;
+  c.nf = (c.nfold + c.chunk - 1) / c.chunk;
+  c.total = c.nf + (c.ndirect + c.chunk - 1) / c.chunk;
   return c;
 }
-__device__ __forceinline__ Chunk chunk_at(const ChunkPlan& c, uint32_t q, uint32_t chunk, const uint64_t* rec,
-                                          uint32_t cap) {
+__device__ __forceinline__ Chunk chunk_at(const ChunkPlan& c, uint32_t q, const uint64_t* rec, uint32_t cap) {
   Chunk k;
   k.fold = q < c.nf;
-  const uint32_t b = (k.fold ? q : q - c.nf) * chunk, all = k.fold ? c.nfold : c.ndirect;
-  k.n = q < c.total ? min(chunk, all - b) : 0u;
+  const uint32_t b = (k.fold ? q : q - c.nf) * c.chunk, all = k.fold ? c.nfold : c.ndirect;
+  k.n = q < c.total ? min(c.chunk, all - b) : 0u;
   k.rec = rec + (k.fold ? 0u : cap - c.ndirect) + b;
   return k;
 }

@@ -153,3 +153,27 @@ def test_padding_in_columns_whose_hash_of_zero_is_deep(zeros):
     assert dev.update(e) == 0 and ref.update(e) == O.OK
     assert dev.sync() == 0
     assert np.array_equal(dev.export(), ref.export())
+
+
+@pytest.mark.parametrize("hub_share", [0.0, 0.1, 0.15, 0.9])
+@pytest.mark.parametrize("records", [0, 70])
+def test_hubs_on_a_small_graph_around_the_share_that_changes_the_chunks(hub_share, records):
+    # a hundred records a vertex on average, so that the plan counts the hubs':
+    # none, an eighth of all records less and more a little, nearly all
+    from paper_2509_14433_gb300 import cupc as B
+    from tests._dev import Dev
+
+    V, n, L, C, D = 700, 35000, 9, 7, 18
+    dev, ref = Dev(V, 3, (L, C, D, 0)), O.Graph(V, 3, L, C, D)
+    assert B.cupc_set_tuning(dev.h, records, 0, 0) == 0
+    g = WL.rng(int(100 * hub_share))
+    e = WL.uniform_pairs(V, n, g)
+    k = int(2 * n * hub_share / 2)  # each edge of the hubs' part gives them one record or two
+    e[:k, 0] = g.integers(0, max(1, k // 1500 + 1), k)
+    e[:k, 1] = np.where(e[:k, 1] == e[:k, 0], 600, e[:k, 1])
+    e = e[g.permutation(n)]
+    for part in (e, e[::-1], e[:12500]):
+        part = np.ascontiguousarray(part)
+        assert dev.update(part) == 0 and ref.update(part) == O.OK
+    assert dev.sync() == 0
+    assert np.array_equal(dev.export(), ref.export())

@@ -29,7 +29,8 @@ def test_every_accepted_setting_gives_chunks_of_whole_groups(tmp_path, V):
     for (uint32_t warps : {{1u, 3u, 32u, 152u, 608u, 760u, 1013u, 3040u}})
       for (uint64_t n = 1; n < (1ull << 31) - 1; n = n * 3 / 2 + 1) {{
         const uint32_t c = chunk_records((uint32_t)(2 * n), V, warps, most);
-        bad += c == 0 || c % kPad || c > most;
+        const uint32_t h = hub_chunk_records((uint32_t)(2 * n), warps, most);
+        bad += c == 0 || c % kPad || c > most || h == 0 || h % kPad || h > most;
         most_used += c + kPad > most;
       }}
   printf("%llu %d", bad, most_used > 1000);""")
