@@ -177,3 +177,31 @@ def test_hubs_on_a_small_graph_around_the_share_that_changes_the_chunks(hub_shar
         assert dev.update(part) == 0 and ref.update(part) == O.OK
     assert dev.sync() == 0
     assert np.array_equal(dev.export(), ref.export())
+
+
+@pytest.mark.parametrize("V", [4097, 70001])
+@pytest.mark.parametrize("C,D", [(1, 3), (2, 1), (3, 2), (7, 4), (7, 5), (8, 9), (16, 6), (31, 5)])
+def test_one_launch_batches_with_hubs(V, C, D):
+    # a star whose centre is now the first, now the second end; two stars; an
+    # edge toggled twice (its sums cancel); no hub; bad edges; and the sizes
+    # around the one from which hubs are looked for and where the CTAs grow
+    from paper_2509_14433_gb300 import cupc as B
+    from tests._dev import Dev
+
+    L = 3
+    dev, ref = Dev(V, 12, (L, C, D, 0)), O.Graph(V, 12, L, C, D)
+    g = WL.rng(C * 100 + D)
+    leaves = 1 + g.permutation(V - 1)[:4096].astype(np.uint32)
+    star = np.stack([np.zeros(4096, np.uint32), leaves], 1)
+    star[::3] = star[::3, ::-1]
+    two = np.concatenate([star[:2500], np.stack([np.full(2600, V - 1), np.arange(1, 2601)], 1)]).astype(np.uint32)
+    for e in (np.concatenate([star, star[:1]]), np.concatenate([star, star]), np.concatenate([two, two[::-1]])[:9000],
+              np.concatenate([WL.uniform_pairs(V, 12287, g), star[:1]]), np.tile(star, (3, 1))[:12288],
+              np.concatenate([star, WL.uniform_pairs(V, 8193 - 4096, g)])):
+        e = np.ascontiguousarray(e, np.uint32)
+        assert 4096 < len(e) <= 12288
+        assert dev.update(e) == 0 and ref.update(e) == O.OK
+        bad = e.copy()
+        bad[len(e) // 2, 1] = bad[len(e) // 2, 0]
+        assert dev.sync() == 0 and dev.update(bad) == 0 and dev.sync() == B.CUPC_EINVAL
+    assert np.array_equal(dev.export(), ref.export())
