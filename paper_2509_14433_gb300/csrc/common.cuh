@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 #include <stdint.h>
 
@@ -111,18 +112,29 @@ constexpr uint32_t kSmallEdges = 12288;
 constexpr uint32_t kSmallHubEdges = 4096;
 // Records per chunk of a batch of nrec records on V vertices: at most `most`,
 // and such that the `warps` of a layer group run out of chunks together (a
-// whole number of chunks each, as near as steps of 16 records and the
-// padding, 1.5 records per folded vertex on average, allow); small batches in
-// quarter passes, two for every warp, as the latency of a warp's records is
-// then all that counts. Always a multiple of kPad, whatever `most` is: the
-// apply kernel folds kPad records at a time and no chunk may split a group.
+// whole number of chunks each, as near as steps of 16 records and the padding,
+// 1.5 records per folded vertex on average, allow); small batches in quarter
+// passes, two for every warp, as the latency of a warp's records is then all
+// that counts. Batches of fewer than kSparseMean records per vertex, whose
+// vertices' costs differ most (one flush each, or none), take 1.6 chunks a warp.
+// GB300, us, uniform batches, 1.6 chunks and one (the kernel that gave a CTA a
+// vertex): V = 2^17, 50000 edges 385 and 434 (403), 30011 edges 259, 261 (271); V
+// = 65536, 50000 edges 283, 323 (323), 30011 edges 215, 233 (234). From 8 records
+// a vertex on one is faster: V = 5003, 50000 edges 57, two take 66. Always a multiple of kPad,
+// whatever `most` is: the apply kernel folds kPad records at a time and no chunk
+// may split a group.
+constexpr uint32_t kSparseMean = 4;
 inline uint32_t chunk_records(uint32_t nrec, uint32_t V, uint32_t warps, uint32_t most) {
   static_assert(kStage / 4 % kPad == 0 && 16 % kPad == 0 && kMinItemRecords >= kPad, "chunks are whole groups");
   most = most / kPad * kPad;
   warps = std::max(1u, warps);
-  const uint64_t all = (uint64_t)nrec + 3ull * std::min(V, nrec / 3) / 2;
+  // vertices of three records or more, were the records spread evenly
+  const double m = (double)nrec / V, folded = V * (1.0 - std::exp(-m) * (1.0 + m + m * m / 2));
+  const uint64_t all = (uint64_t)nrec + (uint64_t)(1.5 * std::max(0.0, folded));
   const uint32_t per = (uint32_t)(all / warps) + 1;
   if (per <= kStage) return std::max(kStage / 4, (per / 2 + kStage / 4 - 1) / (kStage / 4) * (kStage / 4));
+  if (nrec / kSparseMean < V && per / 8 * 5 <= most)
+    return std::min(most, std::max(kStage, (per / 8 * 5 + per % 8 * 5 / 8 + 8) / 16 * 16));
   const uint32_t rounds = (per + most - 1) / most;
   return std::min(most, (per / rounds + 16) / 16 * 16);
 }
