@@ -146,12 +146,12 @@ inline uint32_t chunk_records(uint32_t nrec, uint32_t V, uint32_t warps, uint32_
 // their flushes than they balance. GB300, us, R-MAT batches (chunk_records
 // alone): V = 2048, 80000 edges 67 (73); V = 4096, 60000 and 280000 edges 77, 149
 // (85, 162); V = 8192, 160000 and 280000 edges 142, 170 (150, 183); the other way
-// V = 16384, 200000 edges 202 (198).
+// V = 16384, 200000 edges 202 (198). (With a fifth of a warp's share, but no less
+// than 64 records where a quarter is more: V = 2048, 50000 edges 62, 56 now.)
 constexpr uint32_t kHubMean = 24;
 inline uint32_t hub_chunk_records(uint32_t nrec, uint32_t warps, uint32_t most) {
-  const uint32_t per = nrec / std::max(1u, warps) + 1, up = (per / 5 + 15) / 16 * 16;
-  const uint32_t least = std::min(2 * kStage, std::max(kStage, (per / 4 + 15) / 16 * 16));
-  return std::min(most / kPad * kPad, std::min(5 * kStage, std::max(up, least)));
+  const uint32_t per = nrec / std::max(1u, warps) + 1, part = (per / 9 * 2 + 15) / 16 * 16;
+  return std::min(most / kPad * kPad, std::min(5 * kStage, std::max(kStage, part)));
 }
 // A vertex of more records than this is a hub of its batch: four times the mean.
 inline uint32_t hub_records(uint32_t nrec, uint32_t V) { return 4 * (nrec / V) + 8; }
