@@ -102,14 +102,16 @@ inline bool small_ids(uint32_t V) { return V <= 65536; }
 // 8192 edges 60 (75), 12288 edges 90 (99); V = 2^17, 8192 edges 90 (98), 12288
 // edges 129 (136); R-MAT on V = 2^17, 10000 edges 72 (85), 12288 edges 90 (85).
 constexpr uint32_t kSmallEdges = 12288;
-// More edges than this, on a graph of more vertices (so that a vertex can have
-// as many), and k_small looks for hubs. GB300, us, without -> with, batches whose
-// edges all meet in one vertex (the kernel that folded every batch in brackets):
-// V = 2^14, 6000 edges 56 -> 31 (56), 12000 edges 164 -> 64 (93); V = 2^17, 8000
-// edges 123 -> 60 (85). Uniform and R-MAT batches: between 11 percent faster and
-// 6 slower, the latter above 8192 edges; below 4096 edges hubs cost less than
-// looking for them.
-constexpr uint32_t kSmallHubEdges = 4096;
+// More edges than this, on a graph of more than kSmallHubV vertices (so that a
+// vertex can have as many), and k_small looks for hubs. GB300, us, without ->
+// with, batches whose edges all meet in one vertex (the kernel that folded every
+// batch in brackets): V = 2^14, 4096 edges 34 -> 15 (56), 6000 edges 56 -> 31
+// (56), 12000 edges 164 -> 64 (93); V = 2^17, 4096 edges 51 -> 19 (44), 8000 edges
+// 123 -> 60 (85). Uniform and R-MAT batches: between 11 percent faster and 6
+// slower, the latter above 8192 edges. Below 3072 edges, and on smaller graphs
+// (V = 4096, 12288 edges 35, with 39), hubs cost less than looking for them.
+constexpr uint32_t kSmallHubV = 4096;
+constexpr uint32_t kSmallHubEdges = 3072;
 // Records per chunk of a batch of nrec records on V vertices: at most `most`,
 // and such that the `warps` of a layer group run out of chunks together (a
 // whole number of chunks each, as near as steps of 16 records and the padding,

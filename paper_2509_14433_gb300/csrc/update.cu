@@ -545,7 +545,7 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
   if (n == 0) return cudaSuccess;
   if (validate_ops && n <= kSmallEdges) {
     ProfScope ps(g, s, PC_APPLY, 1);
-    const bool hubs = n > kSmallHubEdges && g->V > kSmallHubEdges;
+    const bool hubs = n > kSmallHubEdges && g->V > kSmallHubV;
     const uint32_t threads = n <= 512 ? 128 : n > 8192 ? 1024 : hubs ? 512 : 256;
     const uint32_t per = threads / 32, groups = layer_groups(g->L, g->P);
     const uint32_t parts = (uint32_t)((2 * n + g->P - 1) / g->P);  // warps of a layer group
