@@ -415,29 +415,18 @@ __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply(
 // and one layer group at a time. What bounds it is latency: the launch, the
 // batch's loads and one pass per warp; the more edges, the bigger the CTAs, so
 // that the validation stays a few loads a thread.
-//
-// kHubs: the records of a hub would queue at its few lines of memory. A CTA then
-// has one layer group; it looks for a hub, the vertex that one of its warps has
-// most records of, if that is more than a quarter, sums its rows below kHubRows
-// in shared memory and sends each once.
-constexpr uint32_t kHubRows = 4;
-template <bool kX32, bool kHubs>
+template <bool kX32>
 __global__ void __launch_bounds__(1024) k_small(ulonglong2* __restrict__ sketch, const uint64_t* __restrict__ keys,
                                                 const uint32_t* __restrict__ edges, const int8_t* __restrict__ ops,
                                                 uint32_t n, uint32_t* gc, uint32_t V, uint32_t L, uint32_t C,
                                                 uint32_t D, uint32_t W, uint32_t P, uint32_t ell) {
-  __shared__ uint32_t s_sum[kHubs ? kHubRows : 1][4][32];  // [row][word][lane]: its slot's sum over the CTA
-  __shared__ uint32_t s_most[32];                          // of each warp: records << 24 | vertex
-  static_assert(kMaxVertices <= 1u << 24, "a vertex id fits beside the count");
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5, s = lane % P;
-  const uint32_t groups = layer_groups(L, P), gw = blockIdx.x * warps + wid;
+  const uint32_t lane = threadIdx.x & 31, gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const uint32_t groups = layer_groups(L, P), s = lane % P;
   // this warp's records and lanes, in flight during the validation
-  const uint32_t i = (kHubs ? blockIdx.x / groups * warps + wid : gw / groups) * P + s;  // endpoint i & 1 of edge i / 2
+  const uint32_t i = gw / groups * P + s;  // record i: endpoint i & 1 of edge i / 2
   const bool have = i < 2 * n;
   const uint32_t w = have ? edges[i] : 0, other = have ? edges[i ^ 1] : 0;
-  const ApplyLane l = apply_lane(keys, sketch, V, L, C, D, W, P, ell, (kHubs ? blockIdx.x : gw) % groups);
-  if (kHubs)
-    for (uint32_t k = threadIdx.x; k < kHubRows * 4 * 32; k += blockDim.x) (&s_sum[0][0][0])[k] = 0;
+  const ApplyLane l = apply_lane(keys, sketch, V, L, C, D, W, P, ell, gw % groups);
   bool drop = (ld_cg(&gc[GC_ERR]) & kErrInval) != 0, bad = false;
 #pragma unroll 4
   for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
@@ -445,23 +434,66 @@ __global__ void __launch_bounds__(1024) k_small(ulonglong2* __restrict__ sketch,
     const int8_t op = ops[j];
     bad |= (u >= V) | (v >= V) | (u == v) | ((op != 1) & (op != -1));
   }
-  if (kHubs) {
-    const uint32_t same = __popc(__match_any_sync(0xffffffffu, w)) / (32 / P);  // the layers repeat the records
-    const uint32_t most =
-        __reduce_max_sync(0xffffffffu, have && same > max(1u, P / 4) ? same << 24 | (w & 0xFFFFFFu) : 0u);
-    if (lane == 0) s_most[wid] = most;
-  }
   if (__syncthreads_or(bad)) {
     if (threadIdx.x == 0) atomicOr(&gc[GC_ERR], kErrInval);
     drop = true;
   }
   if (__syncthreads_or(drop)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) gc[GC_BATCHES] += 1;
-  uint32_t hub = kNoneU32;
-  if (kHubs) {
-    const uint32_t most = __reduce_max_sync(0xffffffffu, lane < warps ? s_most[lane] : 0u);
-    if (most) hub = most & 0xFFFFFFu;
+  const uint64_t x = record_id(make_record(w, other), V), c = mix64(x ^ l.kchk);  // of this lane's layer
+  for (uint32_t k = 0; k < P; k++) {
+    const uint32_t from = (lane & ~(P - 1)) + k;
+    const bool in = __shfl_sync(0xffffffffu, have, from);
+    const uint32_t wk = __shfl_sync(0xffffffffu, w, from);
+    const uint64_t xk = __shfl_sync(0xffffffffu, x, from), ck = __shfl_sync(0xffffffffu, c, from);
+    if (l.active && in) xor_bucket_atomic(l.base + (size_t)wk * W + lane_depth<kX32>(l, xk), make_ulonglong2(xk, ck));
   }
+}
+
+// The same where a vertex may be a hub, whose records would queue at its few lines
+// of memory: a CTA has one layer group; it looks for a hub, the vertex that one of
+// its warps has most records of, if that is more than a quarter, sums its rows
+// below kHubRows in shared memory and sends each once. A kernel of its own: as one
+// template with k_small, batches of 160 to 256 edges took 6.2 us instead of 4.9
+// to 5.7 (V = 1024).
+constexpr uint32_t kHubRows = 4;
+template <bool kX32>
+__global__ void __launch_bounds__(1024) k_small_hubs(ulonglong2* __restrict__ sketch,
+                                                     const uint64_t* __restrict__ keys,
+                                                     const uint32_t* __restrict__ edges,
+                                                     const int8_t* __restrict__ ops, uint32_t n, uint32_t* gc,
+                                                     uint32_t V, uint32_t L, uint32_t C, uint32_t D, uint32_t W,
+                                                     uint32_t P, uint32_t ell) {
+  __shared__ uint32_t s_sum[kHubRows][4][32];  // [row][word][lane]: its slot's sum over the CTA
+  __shared__ uint32_t s_most[32];              // of each warp: records << 24 | vertex
+  static_assert(kMaxVertices <= 1u << 24, "a vertex id fits beside the count");
+  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5, s = lane % P;
+  const uint32_t groups = layer_groups(L, P);
+  // this warp's records and lanes, in flight during the validation
+  const uint32_t i = (blockIdx.x / groups * warps + wid) * P + s;  // endpoint i & 1 of edge i / 2
+  const bool have = i < 2 * n;
+  const uint32_t w = have ? edges[i] : 0, other = have ? edges[i ^ 1] : 0;
+  const ApplyLane l = apply_lane(keys, sketch, V, L, C, D, W, P, ell, blockIdx.x % groups);
+  for (uint32_t k = threadIdx.x; k < kHubRows * 4 * 32; k += blockDim.x) (&s_sum[0][0][0])[k] = 0;
+  bool drop = (ld_cg(&gc[GC_ERR]) & kErrInval) != 0, bad = false;
+#pragma unroll 4
+  for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
+    const uint32_t u = edges[2 * j], v = edges[2 * j + 1];
+    const int8_t op = ops[j];
+    bad |= (u >= V) | (v >= V) | (u == v) | ((op != 1) & (op != -1));
+  }
+  const uint32_t same = __popc(__match_any_sync(0xffffffffu, w)) / (32 / P);  // the layers repeat the records
+  const uint32_t mine =
+      __reduce_max_sync(0xffffffffu, have && same > max(1u, P / 4) ? same << 24 | (w & 0xFFFFFFu) : 0u);
+  if (lane == 0) s_most[wid] = mine;
+  if (__syncthreads_or(bad)) {
+    if (threadIdx.x == 0) atomicOr(&gc[GC_ERR], kErrInval);
+    drop = true;
+  }
+  if (__syncthreads_or(drop)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) gc[GC_BATCHES] += 1;
+  const uint32_t most = __reduce_max_sync(0xffffffffu, lane < warps ? s_most[lane] : 0u);
+  const uint32_t hub = most ? most & 0xFFFFFFu : kNoneU32;
   const uint64_t x = record_id(make_record(w, other), V), c = mix64(x ^ l.kchk);  // of this lane's layer
   for (uint32_t k = 0; k < P; k++) {
     const uint32_t from = (lane & ~(P - 1)) + k;
@@ -470,7 +502,7 @@ __global__ void __launch_bounds__(1024) k_small(ulonglong2* __restrict__ sketch,
     const uint64_t xk = __shfl_sync(0xffffffffu, x, from), ck = __shfl_sync(0xffffffffu, c, from);
     if (!l.active || !in) continue;
     const uint32_t row = lane_depth<kX32>(l, xk);
-    if (kHubs && wk == hub && row < kHubRows) {
+    if (wk == hub && row < kHubRows) {
       atomicXor(&s_sum[row][0][lane], (uint32_t)xk);
       if (!kX32) atomicXor(&s_sum[row][1][lane], (uint32_t)(xk >> 32));
       atomicXor(&s_sum[row][2][lane], (uint32_t)ck);
@@ -479,7 +511,7 @@ __global__ void __launch_bounds__(1024) k_small(ulonglong2* __restrict__ sketch,
       xor_bucket_atomic(l.base + (size_t)wk * W + row, make_ulonglong2(xk, ck));
     }
   }
-  if (!kHubs || hub == kNoneU32) return;
+  if (hub == kNoneU32) return;
   __syncthreads();
   for (uint32_t q = wid; q < kHubRows; q += warps) {
     const ulonglong2 v = make_ulonglong2((uint64_t)s_sum[q][1][lane] << 32 | s_sum[q][0][lane],
@@ -550,8 +582,8 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
     const uint32_t per = threads / 32, groups = layer_groups(g->L, g->P);
     const uint32_t parts = (uint32_t)((2 * n + g->P - 1) / g->P);  // warps of a layer group
     const uint32_t grid = hubs ? (parts + per - 1) / per * groups : (parts * groups + per - 1) / per;
-    auto kern = small_ids(g->V) ? (hubs ? k_small<true, true> : k_small<true, false>)
-                                : (hubs ? k_small<false, true> : k_small<false, false>);
+    auto kern = hubs ? (small_ids(g->V) ? k_small_hubs<true> : k_small_hubs<false>)
+                     : (small_ids(g->V) ? k_small<true> : k_small<false>);
     kern<<<grid, threads, 0, s>>>(g->sketch, g->keys, edges, validate_ops, (uint32_t)n, g->gc, g->V, g->L, g->C, g->D,
                                   g->W, g->P, g->ell);
     return cudaGetLastError();
