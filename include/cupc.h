@@ -30,10 +30,12 @@
  *   lg = ceil(log2 V) (at least 1); rounds/layers L = lg + 2;
  *   columns C = 7; rows D = 2*lg; buckets per layer W = 1 + C*D;
  *   a bucket is two u64 words {alpha, gamma}; a vertex sketch is L*W
- *   buckets. The hash of index idx in column c of layer r is
- *   mix(idx ^ key[r*(C+1)+c]), its depth min(ctz(hash), D-1); the checksum
- *   is mix(idx ^ key[r*(C+1)+C]); key[j] = mix(seed + 0x9E3779B97F4A7C15 *
- *   (j+1)) and mix is the SplitMix64 finalizer.
+ *   buckets. The depth of index idx in column c of layer r is the number of
+ *   leading zero bits of h(idx) h'(idx), at most D-1, where h(x) is the top
+ *   ell = 65 - 2*lg bits of a*x + b mod 2^64 and h' those of a'*x + b'; a is
+ *   key[r*(C+1)+c], and b, a', b' are key[L*(C+1) + 3*(r*C+c) + 0, 1, 2]. The
+ *   checksum is mix(idx ^ key[r*(C+1)+C]); key[j] = mix(seed +
+ *   0x9E3779B97F4A7C15 * (j+1)) and mix is the SplitMix64 finalizer.
  */
 #ifndef CUPC_H
 #define CUPC_H
@@ -68,8 +70,8 @@ typedef struct {
                          because sketch addition is XOR */
 } cupc_params;
 /* Limits (else CUPC_EINVAL): W = 1 + C*D <= 256; L * P <= 1024 with P the
- * power of two >= C + 1 (the update kernel runs one thread per layer and
- * column, plus a checksum thread); 2 * max_batch < 2^32. */
+ * power of two >= C + 1 (the update's warps take the layers in groups of 32/P,
+ * a lane per column, and there are 32 groups at most); 2 * max_batch < 2^32. */
 
 /* Device bytes cupc_init needs for V vertices (sketches + scratch), so that
  * a caller (e.g. a PyTorch allocation) can own the memory. 0 on bad input. */
@@ -267,7 +269,8 @@ void cupc_server_destroy(cupc_server* s);
  * rows per column folded in shared memory, besides the first three, which are
  * folded in registers (1..min(D, 16), 0 = min(D, 8); deeper rows go straight
  * to HBM), ctas_per_sm = resident CTAs per SM of the persistent grid (0 = as
- * many as fit). CUPC_EINVAL (previous settings kept) when out of range.
+ * many as fit). CUPC_EINVAL (previous settings kept) when out of range, and
+ * when 512 * smem_rows * ceil(L*P/32) + 520 * L + 1536 exceeds 232448.
  * cupc_get_tuning: out4 = {item_records, smem_rows, ctas_per_sm, CTAs per SM
  * in use}. */
 cupc_status cupc_set_tuning(cupc_graph* g, uint32_t item_records, uint32_t smem_rows, uint32_t ctas_per_sm);

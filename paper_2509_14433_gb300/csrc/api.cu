@@ -42,9 +42,9 @@ Dims derive(uint32_t V, const cupc_params* p) {
   if (d.C > 31 || d.D > 63 || d.D < 1 || d.L < 1 || d.L > 64) return d;
   d.W = 1 + d.C * d.D;
   if (d.W > 32 * kWarpBuckets) return d;
-  uint32_t P = 1;  // apply threads per layer: the columns and the checksum lane
+  uint32_t P = 1;  // an apply warp's lanes per layer: the columns and the deterministic bucket
   while (P < d.C + 1) P <<= 1;
-  if (d.L * P > 1024) return d;  // one apply CTA holds every (layer, lane)
+  if (d.L * P > 1024) return d;  // at most 32 layer groups (kWorkNext)
   // the edge index u*V+v must fit the 64-bit bucket word; staging offsets of
   // a batch are u32
   if ((uint64_t)d.max_batch * 2 >= 0xFFFFFFFFull) return d;

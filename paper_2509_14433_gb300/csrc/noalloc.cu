@@ -2,8 +2,9 @@
 //
 // cupc_update_sketch_static applies a batch of edge updates to a sketch
 // buffer the caller owns, using the same kernels as cupc_update_batch. Its
-// scratch (per-vertex counts and cursors, endpoint records, hash keys, counters) is the file-scope array below instead of a workspace, so
-// the call allocates nothing. The paper has no counterpart of this entry
+// scratch (per-vertex counts and cursors, endpoint records, hash keys, counters)
+// is the file-scope array below instead of a workspace, so the call allocates
+// nothing. The paper has no counterpart of this entry
 // point.
 #include <mutex>
 

@@ -52,7 +52,8 @@ __device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
 }
 
 // Grid barrier for a cooperative launch: CTA thread 0 adds one to an arrival
-// counter that only grows during the launch (zero before it) and waits until all CTAs of this barrier have arrived. The wait is bounded:
+// counter that only grows during the launch (zero before it) and waits until
+// all CTAs of this barrier have arrived. The wait is bounded:
 // after kWaitLimitNs it records kErrTimeout and returns false in every
 // thread of the CTA, which must then return.
 __device__ __forceinline__ bool grid_barrier(uint32_t* gc, uint32_t nblocks, uint32_t& epoch, int* s_ok,
@@ -790,8 +791,8 @@ __device__ __forceinline__ bool recover_body(const RecArgs& a) {
     }
     book_stash();
     CUPC_GRID_SYNC();
-    // Components of more than kRecSpan members that no warp holds alone and whose buckets
-    // so far hold no good one are marked (merged[K], unused until the
+    // Components of more than kRecSpan members that no warp holds alone and whose
+    // buckets so far hold no good one are marked (merged[K], unused until the
     // relabel): another pass over the next kPrefix buckets.
     for (uint32_t base = kPrefix; multi && base < W && ld_cg(&gc[GC_RETRY + base / kPrefix - 1]); base += kPrefix) {
       reduce_run(base);

@@ -359,10 +359,10 @@ __global__ void k_scatter(const uint32_t* __restrict__ edges, size_t n, uint32_t
 }
 
 // Apply the records, in chunks of `chunk` records, or `hub_chunk` if hubs hold
-// more than an eighth of them (apply_chunk). A warp keeps
-// the layer group (its number modulo the groups). Its first two chunks are
-// given, the others come from the group's counter, asked for two chunks
-// ahead, so that the next chunk's records load while it works on this one.
+// more than an eighth of them (apply_chunk). A warp keeps the layer group (its
+// number modulo the groups). Its first two chunks are given, the others come from
+// the group's counter, asked for two chunks ahead, so that the next chunk's
+// records load while it works on this one.
 //
 // What bounds it. Batches of many records per vertex: instruction issue and
 // the ALU (64 lanes a cycle per SM), which folding rows 0..2 in registers and
@@ -378,8 +378,8 @@ __global__ void k_scatter(const uint32_t* __restrict__ edges, size_t n, uint32_t
 template <bool kX32>
 __global__ void __launch_bounds__(32 * kApplyWarps, kApplyCtas) k_apply(
     ulonglong2* __restrict__ sketch, const uint64_t* __restrict__ keys, const uint64_t* __restrict__ rec, uint32_t cap,
-    uint32_t chunk, uint32_t hub_chunk, uint32_t* work, const uint32_t* gc, uint32_t V, uint32_t L, uint32_t C, uint32_t D, uint32_t W,
-    uint32_t P, uint32_t R, uint32_t ell) {
+    uint32_t chunk, uint32_t hub_chunk, uint32_t* work, const uint32_t* gc, uint32_t V, uint32_t L, uint32_t C,
+    uint32_t D, uint32_t W, uint32_t P, uint32_t R, uint32_t ell) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (ld_cg(&gc[GC_ERR]) & kErrInval) return;
   const uint32_t nslots = apply_slots(R);
@@ -553,7 +553,8 @@ cudaError_t setup_update(cupc_graph* g) {
 
 // Shared memory and persistent grid of k_apply for the given tunables.
 cudaError_t apply_config(const cupc_graph* g, uint32_t R, uint32_t cps, int* smem, int* grid) {
-  // the tunable's range: R rows of every lane of the graph within one SM
+  // the range of settings the entry points have always taken, which is less than
+  // this kernel could launch with (at most 80 KB of shared memory a CTA)
   if ((size_t)R * layer_groups(g->L, g->P) * 512 + (size_t)g->L * 520 + 1536 > 232448) return cudaErrorInvalidValue;
   *smem = (int)(kApplyWarps * apply_warp_bytes(fold_rows(R, g->D), g->P));
   cudaError_t e = raise_apply_smem_limit(*smem);
