@@ -264,12 +264,13 @@ void cupc_server_destroy(cupc_server* s);
 
 /* Launch tunables of the update's apply kernel (results are identical for
  * every setting; only speed changes): item_records = endpoint records per
- * chunk at most (64..512, 0 = 256; the kernel takes records in groups of
- * four, so a setting acts as the multiple of 4 at or below it), smem_rows =
- * rows per column folded in shared memory, besides the first three, which are
- * folded in registers (1..min(D, 16), 0 = min(D, 8); deeper rows go straight
- * to HBM), ctas_per_sm = resident CTAs per SM of the persistent grid (0 = as
- * many as fit). CUPC_EINVAL (previous settings kept) when out of range, and
+ * chunk at most (64..512, 0 = 256, and 512 for batches of many records per
+ * vertex; the kernel takes records in groups of four, so a setting acts as
+ * the multiple of 4 at or below it), smem_rows = rows per column folded in
+ * shared memory, besides the first three, which are folded in registers
+ * (1..min(D, 16), 0 = min(D, 8); deeper rows go straight to HBM), ctas_per_sm
+ * = resident CTAs per SM of the persistent grid (0 = as many as fit).
+ * CUPC_EINVAL (previous settings kept) when out of range, and
  * when 512 * smem_rows * ceil(L*P/32) + 520 * L + 1536 exceeds 232448.
  * cupc_get_tuning: out4 = {item_records, smem_rows, ctas_per_sm, CTAs per SM
  * in use}. */

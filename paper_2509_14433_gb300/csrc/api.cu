@@ -550,7 +550,8 @@ cupc_status cupc_profile_read(cupc_graph* g, double* ms, uint64_t* launches, siz
 
 cupc_status cupc_set_tuning(cupc_graph* g, uint32_t item_records, uint32_t smem_rows, uint32_t ctas_per_sm) {
   if (!g) return CUPC_EINVAL;
-  if (item_records == 0) item_records = kDefaultItemRecords;
+  const bool item_default = item_records == 0;
+  if (item_default) item_records = kDefaultItemRecords;
   if (smem_rows == 0) smem_rows = g->D < kSmemRows ? g->D : kSmemRows;
   if (item_records < kMinItemRecords || item_records > kItemRecords || smem_rows > kSmemRowsMax || smem_rows > g->D)
     return CUPC_EINVAL;
@@ -566,6 +567,7 @@ cupc_status cupc_set_tuning(cupc_graph* g, uint32_t item_records, uint32_t smem_
     configure_apply(g);
     return CUPC_EINVAL;
   }
+  g->item_default = item_default;
   return CUPC_OK;
 }
 
@@ -577,7 +579,8 @@ cupc_status cupc_set_tuning_bucket(cupc_graph* g, uint32_t bucket, uint32_t item
     t.set = false;
     return CUPC_OK;
   }
-  if (item_records == 0) item_records = kDefaultItemRecords;
+  const bool item_default = item_records == 0;
+  if (item_default) item_records = kDefaultItemRecords;
   if (smem_rows == 0) smem_rows = g->D < kSmemRows ? g->D : kSmemRows;
   if (item_records < kMinItemRecords || item_records > kItemRecords || smem_rows > kSmemRowsMax || smem_rows > g->D)
     return CUPC_EINVAL;
@@ -586,7 +589,7 @@ cupc_status cupc_set_tuning_bucket(cupc_graph* g, uint32_t bucket, uint32_t item
     cudaGetLastError();
     return CUPC_EINVAL;
   }
-  t = cupc_graph::ApplyTune{true, item_records, smem_rows, ctas_per_sm, smem, grid};
+  t = cupc_graph::ApplyTune{true, item_default, item_records, smem_rows, ctas_per_sm, smem, grid};
   return CUPC_OK;
 }
 

@@ -126,19 +126,36 @@ constexpr uint32_t kSmallHubEdges = 3072;
 // whatever `most` is: the apply kernel folds kPad records at a time and no chunk
 // may split a group.
 constexpr uint32_t kSparseMean = 4;
+// Records of a batch for each of `warps` warps, the padding of evenly spread
+// records included (1.5 for a vertex of three or more).
+inline uint32_t records_per_warp(uint32_t nrec, uint32_t V, uint32_t warps) {
+  const double m = (double)nrec / V, folded = V * (1.0 - std::exp(-m) * (1.0 + m + m * m / 2));
+  const uint64_t all = (uint64_t)nrec + (uint64_t)(1.5 * std::max(0.0, folded));
+  return (uint32_t)(all / std::max(1u, warps)) + 1;
+}
 inline uint32_t chunk_records(uint32_t nrec, uint32_t V, uint32_t warps, uint32_t most) {
   static_assert(kStage / 4 % kPad == 0 && 16 % kPad == 0 && kMinItemRecords >= kPad, "chunks are whole groups");
   most = most / kPad * kPad;
-  warps = std::max(1u, warps);
-  // vertices of three records or more, were the records spread evenly
-  const double m = (double)nrec / V, folded = V * (1.0 - std::exp(-m) * (1.0 + m + m * m / 2));
-  const uint64_t all = (uint64_t)nrec + (uint64_t)(1.5 * std::max(0.0, folded));
-  const uint32_t per = (uint32_t)(all / warps) + 1;
+  const uint32_t per = records_per_warp(nrec, V, warps);
   if (per <= kStage) return std::max(kStage / 4, (per / 2 + kStage / 4 - 1) / (kStage / 4) * (kStage / 4));
   if (nrec / kSparseMean < V && per / 8 * 5 <= most)
     return std::min(most, std::max(kStage, (per / 8 * 5 + per % 8 * 5 / 8 + 8) / 16 * 16));
   const uint32_t rounds = (per + most - 1) / most;
   return std::min(most, (per / rounds + 16) / 16 * 16);
+}
+// The most records per chunk where the caller leaves it to the library and no
+// hubs hold much of the batch: batches of kDenseMean records per vertex or more
+// take one or two long chunks a warp where that is enough, as every cut through a
+// vertex's records costs a flush. GB300, us, uniform batches with at most 512 and
+// 256 records (the kernel that gave a CTA a vertex): V = 2048, 100000 edges 67, 73
+// (70); V = 3099, 200000 edges 110, 114 (111); V = 5003, 160000 edges 97, 102
+// (106); V = 2^14, 240000 edges 166, 189 (237). The other way below that mean (V =
+// 24576, 80000 edges 219, 192) and with three chunks a warp (V = 4096, 400000
+// edges 187, 179), and with hubs (R-MAT, V = 2^14, 160000 edges 195, 175).
+constexpr uint32_t kDenseMean = 10;
+inline uint32_t default_most(uint32_t nrec, uint32_t V, uint32_t warps) {
+  const bool two = nrec / kDenseMean >= V && records_per_warp(nrec, V, warps) <= 2 * kItemRecords;
+  return two ? kItemRecords : kDefaultItemRecords;
 }
 // The same for a batch whose hubs hold more than an eighth of its records: a
 // chunk of a hub's records takes one flush, one of many small vertices a flush
@@ -275,10 +292,11 @@ struct cupc_graph {
                       // the XOR of all vertex sketches need not be zero
   int device, sms;
   int apply_smem, apply_grid;
-  uint32_t item_records, apply_cps;  // tunables: records per work item, CTAs per SM (0 = max)
+  uint32_t item_records, apply_cps;  // tunables: records per chunk at most, CTAs per SM (0 = max)
+  bool item_default;                 // item_records was left to the library (default_most)
   // optional per-batch-size settings: bucket floor(log4 edges) (at least 5)
   struct ApplyTune {
-    bool set;
+    bool set, item_default;
     uint32_t item_records, R, cps;
     int smem, grid;
   } tune_b[16];

@@ -130,6 +130,7 @@ extern "C" cupc_status cupc_update_sketch_static(void* sketch, uint32_t V, uint6
   g.R = g.D < kSmemRows ? g.D : kSmemRows;
   g.ell = hash_bits(V);
   g.item_records = kDefaultItemRecords;
+  g.item_default = true;
   g.apply_smem = (int)(kApplyWarps * apply_warp_bytes(fold_rows(g.R, g.D), g.P));
   // the set-up sized the launch for the widest graph; a narrower one fits
   g.apply_grid = ds->apply_grid;

@@ -547,6 +547,7 @@ cudaError_t setup_update(cupc_graph* g) {
   g->R = g->D < kSmemRows ? g->D : kSmemRows;
   g->ell = hash_bits(g->V);
   g->item_records = kDefaultItemRecords;
+  g->item_default = true;
   g->apply_cps = 0;
   return configure_apply(g);
 }
@@ -591,10 +592,12 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
   }
   // the setting of this batch size's bucket, else the graph's default
   uint32_t ir = g->item_records, R = g->R;
+  bool ir_default = g->item_default;
   int smem = g->apply_smem, grid_max = g->apply_grid;
   const cupc_graph::ApplyTune& t = g->tune_b[tune_bucket(n)];
   if (t.set) {
     ir = t.item_records;
+    ir_default = t.item_default;
     R = t.R;
     smem = t.smem;
     grid_max = t.grid;
@@ -605,7 +608,11 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
   const bool priv = g->V <= kPrivMaxV && pgrid >= (int)kPrivMinCtas;
   const uint32_t shards = !priv && n >= kShardEdges ? g->shards : 1u;
   const uint32_t nrec = (uint32_t)(2 * n);
-  const bool hubs = g->V <= kPrivMaxV && nrec / g->V >= kHubMean;  // hub_chunk_records
+  const uint32_t groups = layer_groups(g->L, g->P), warps = (uint32_t)grid_max * kApplyWarps / groups;
+  // the chunks if hubs hold little of the batch, and if they hold much of it
+  const uint32_t chunk = chunk_records(nrec, g->V, warps, ir_default ? default_most(nrec, g->V, warps) : ir);
+  const uint32_t hub_chunk = g->V <= kPrivMaxV && nrec / g->V >= kHubMean ? hub_chunk_records(nrec, warps, ir)
+                                                                          : chunk_records(nrec, g->V, warps, ir);
   {
     ProfScope ps(g, s, PC_GROUP, 3);
     if (priv)
@@ -613,17 +620,14 @@ cudaError_t launch_update_chunk(cupc_graph* g, const uint32_t* edges, size_t n, 
     else
       k_count<<<grid, 256, 0, s>>>(edges, validate_ops, n, g->V, g->cnt, shards, g->work, g->gc);
     k_plan<<<plan_slices(g->V), kPlanThreads, 0, s>>>(g->cnt, g->cursor, g->rec, g->V, g->rec_cap, shards,
-                                                       hubs ? hub_records(nrec, g->V) : kNoneU32, g->work, g->gc);
+                                                       chunk != hub_chunk ? hub_records(nrec, g->V) : kNoneU32, g->work,
+                                                       g->gc);
     if (priv)
       k_scatter_priv<<<pgrid, 1024, 8 * g->V, s>>>(edges, n, g->V, g->cursor, g->rec, g->gc);
     else
       k_scatter<<<grid, 256, 0, s>>>(edges, n, g->V, g->cursor, shards, g->rec, g->gc);
   }
   ProfScope ps(g, s, PC_APPLY, 1);
-  const uint32_t groups = layer_groups(g->L, g->P);
-  const uint32_t warps = (uint32_t)grid_max * kApplyWarps / groups;
-  const uint32_t chunk = chunk_records(nrec, g->V, warps, ir);
-  const uint32_t hub_chunk = hubs ? hub_chunk_records(nrec, warps, ir) : chunk;
   // at most: chunks of padded fold records and of direct records
   const size_t units = (size_t)(rec_entries(g->V, n) / std::min(chunk, hub_chunk) + 2) * groups;
   const int agrid = (int)std::min<size_t>((size_t)grid_max, (units + kApplyWarps - 1) / kApplyWarps);
