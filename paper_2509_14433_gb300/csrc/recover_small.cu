@@ -535,23 +535,25 @@ __global__ void __launch_bounds__(kClThreads, 1) k_recover_cl(RecArgs a) {
     }
     cluster_sync_all();  // the samples in cand are visible to the leader
     if (!leader) continue;
-    if (__syncthreads_or(ld_cg(&gc[GC_RETRY]) != 0)) {  // read by all before it is reset
-      base += kPrefix;
-      continue;
-    }
-    base = 0;
-    // ---- book the samples of the live components
+    // ---- book the samples of the live components, unless some need another
+    // pass; that count and the first sample are in flight together
+    const uint32_t again = ld_cg(&gc[GC_RETRY]);
+    const ulonglong2 c0 = tid < V ? __ldcg(&a.cand[tid]) : make_ulonglong2(0, 0);
     for (uint32_t K = tid; K < V; K += nt) {
       m.e[K] = kNoneU32;
       m.f[K] = K;
     }
     if (tid == 0) c_ncand = 0;
-    __syncthreads();
+    if (__syncthreads_or(again != 0)) {  // read by all before it is reset
+      base += kPrefix;
+      continue;
+    }
+    base = 0;
     uint32_t live = 0, nz = 0, fail = 0, fp = 0;
     for (uint32_t K = tid; K < V; K += nt) {
       if (m.lab[K] != K || m.fin[K]) continue;  // not a label, or final
       live++;
-      const ulonglong2 c = __ldcg(&a.cand[K]);
+      const ulonglong2 c = K == tid ? c0 : __ldcg(&a.cand[K]);
       if (c.y == 0) {
         m.fin[K] = 1;
         continue;
