@@ -122,9 +122,9 @@ constexpr uint32_t kSmallHubEdges = 3072;
 // GB300, us, uniform batches, 1.6 chunks and one (the kernel that gave a CTA a
 // vertex): V = 2^17, 50000 edges 385 and 434 (403), 30011 edges 259, 261 (271); V
 // = 65536, 50000 edges 283, 323 (323), 30011 edges 215, 233 (234). From 8 records
-// a vertex on one is faster: V = 5003, 50000 edges 57, two take 66. Always a multiple of kPad,
-// whatever `most` is: the apply kernel folds kPad records at a time and no chunk
-// may split a group.
+// a vertex on one is faster: V = 5003, 50000 edges 57, two take 66. Always a
+// multiple of kPad, whatever `most` is: the apply kernel folds kPad records at a
+// time and no chunk may split a group.
 constexpr uint32_t kSparseMean = 4;
 // Records of a batch for each of `warps` warps, the padding of evenly spread
 // records included (1.5 for a vertex of three or more).
@@ -157,8 +157,8 @@ inline uint32_t default_most(uint32_t nrec, uint32_t V, uint32_t warps) {
   const bool two = nrec / kDenseMean >= V && records_per_warp(nrec, V, warps) <= 2 * kItemRecords;
   return two ? kItemRecords : kDefaultItemRecords;
 }
-// The same for a batch whose hubs hold more than an eighth of its records: a
-// chunk of a hub's records takes one flush, one of many small vertices a flush
+// Records per chunk of a batch whose hubs hold more than an eighth of its records:
+// a chunk of a hub's records takes one flush, one of many small vertices a flush
 // for each, so equal chunks, one or two a warp, end far apart. Four or five
 // each, of 32 to 160 records. Used on graphs of at most kPrivMaxV vertices that
 // get kHubMean records or more on average; elsewhere smaller chunks lose more to
